@@ -94,6 +94,7 @@ template <bool ODD, int SCHED>
 __global__ void __launch_bounds__(256, 2) k_batch_step(const BatchDomain* __restrict__ dom, const BatchTile* __restrict__ tiles,
                                                     const int* __restrict__ ntiles_p, float* __restrict__ pool,
                                                     const uint32_t* __restrict__ links, unsigned int* flag, float rho0) {
+    pdl_wait();
     const int ntiles = *ntiles_p;
     int t = blockIdx.x, t_end = ntiles, t_step = gridDim.x;
     if (SCHED == 1) {
@@ -334,19 +335,11 @@ lbm_status rebuild_tiles(lbm_batch* b) {
 }
 
 cudaError_t launch_batch_step(lbm_batch* b, int odd) {
-#define CMLBM_BATCH_LAUNCH(O, C)                                                                                  \
-    k_batch_step<O, C><<<b->grid, b->threads, 0, b->stream>>>(b->d_dom, b->d_tiles, b->d_ntiles, b->pool, b->links, \
-                                                               b->d_flag, (float)b->rho0)
-    switch (b->schedule * 2 + (odd ? 1 : 0)) {
-    case 0: CMLBM_BATCH_LAUNCH(false, 0); break;
-    case 1: CMLBM_BATCH_LAUNCH(true, 0); break;
-    case 2: CMLBM_BATCH_LAUNCH(false, 1); break;
-    case 3: CMLBM_BATCH_LAUNCH(true, 1); break;
-    case 4: CMLBM_BATCH_LAUNCH(false, 2); break;
-    default: CMLBM_BATCH_LAUNCH(true, 2); break;
-    }
-#undef CMLBM_BATCH_LAUNCH
-    return cudaGetLastError();
+    static constexpr decltype(&k_batch_step<false, 0>) kernels[6] = {k_batch_step<false, 0>, k_batch_step<true, 0>,
+                                                                     k_batch_step<false, 1>, k_batch_step<true, 1>,
+                                                                     k_batch_step<false, 2>, k_batch_step<true, 2>};
+    return launch_pdl(kernels[b->schedule * 2 + (odd ? 1 : 0)], b->grid, b->threads, 0, b->stream, b->d_dom, b->d_tiles,
+                      b->d_ntiles, b->pool, b->links, b->d_flag, (float)b->rho0);
 }
 
 // blocks_per_sm = 0: one block per tile (the grid covers the tile list at this time; later

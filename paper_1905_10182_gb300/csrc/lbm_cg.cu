@@ -141,6 +141,7 @@ __device__ __forceinline__ void gather_two(const float* __restrict__ fr, const f
 
 template <bool ODD, bool LINKS>
 __global__ void __launch_bounds__(CG_BLOCK) k_cg_fields(KParams p, CgArgs q, const float* __restrict__ fr) {
+    pdl_wait();
     const int x = blockIdx.x * CG_BLOCK + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z;
     if (x >= p.nx) return;
@@ -153,6 +154,7 @@ __global__ void __launch_bounds__(CG_BLOCK) k_cg_fields(KParams p, CgArgs q, con
 
 template <bool ODD, bool LINKS>
 __global__ void __launch_bounds__(CG_BLOCK, 4) k_cg_step(KParams p, CgArgs q, float* __restrict__ fr) {
+    pdl_wait();
     const int x = blockIdx.x * CG_BLOCK + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z;
     if (x >= p.nx) return;
@@ -331,11 +333,14 @@ cudaError_t launch_cg_step(const KParams& p, const CgParams& c, void* fr, float*
                            cudaStream_t st) {
     const CgArgs q = cg_args(c, fb, fld);
     float* r = static_cast<float*>(fr);
-    CMLBM_CG_DISPATCH(k_cg_fields, p, q, r);
-    cudaError_t e = cudaGetLastError();
+    const bool links = p.links != nullptr;
+    const auto fields = odd ? (links ? k_cg_fields<true, true> : k_cg_fields<true, false>)
+                            : (links ? k_cg_fields<false, true> : k_cg_fields<false, false>);
+    const auto step = odd ? (links ? k_cg_step<true, true> : k_cg_step<true, false>)
+                          : (links ? k_cg_step<false, true> : k_cg_step<false, false>);
+    const cudaError_t e = launch_pdl(fields, cg_grid(p), CG_BLOCK, 0, st, p, q, r);
     if (e != cudaSuccess) return e;
-    CMLBM_CG_DISPATCH(k_cg_step, p, q, r);
-    return cudaGetLastError();
+    return launch_pdl(step, cg_grid(p), CG_BLOCK, 0, st, p, q, r);
 }
 
 cudaError_t launch_cg_macro(const KParams& p, const CgParams& c, const void* fr, float* fb, int odd, float* out,

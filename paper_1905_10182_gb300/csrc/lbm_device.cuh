@@ -46,6 +46,10 @@ __host__ __device__ constexpr unsigned long long pack_dir(int axis) {
     return c;
 }
 
+// Waits until the kernel before this one in its stream has completed and its writes are visible
+// (returns at once in a kernel launched without programmatic serialisation, see launch_pdl).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 constexpr uint32_t SOLID_BIT = 1u << 31;  // in a link word: the node itself is solid
 constexpr int BLOCK_X = 128;              // one-node kernels: threads per block, one node each along x
 

@@ -26,6 +26,7 @@ __device__ __forceinline__ void check_node(const KParams& p, const Macro& m) {
 // HO: the second-order Hermite truncations (models M4, M5 of Sec. III) instead of the complete ones.
 template <typename S, bool ODD, bool LINKS, int FK, bool TRACE, bool HO>
 __global__ void __launch_bounds__(BLOCK_X, (sizeof(S) == 4 ? 4 : 5)) k_stream_collide(KParams p, S* __restrict__ f) {
+    pdl_wait();
     const int x = blockIdx.x * BLOCK_X + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z + p.z0;
     if (p.pf) k1_prefetch<S, ODD>(p, f);
@@ -58,6 +59,7 @@ __global__ void __launch_bounds__(BLOCK_X, (sizeof(S) == 4 ? 4 : 5)) k_stream_co
 // touched part of the store (up to the 129 MB of L2) still in L2.
 template <typename S, bool ODD, bool LINKS>
 __global__ void __launch_bounds__(BLOCK_X) k_psi(KParams p, const S* __restrict__ f, float* __restrict__ psi) {
+    pdl_wait();
     const int x = (gridDim.x - 1 - blockIdx.x) * BLOCK_X + threadIdx.x;
     const int y = gridDim.y - 1 - blockIdx.y, z = gridDim.z - 1 - blockIdx.z + p.z0;
     if (x >= p.nx) return;
@@ -171,35 +173,28 @@ static cudaError_t launch_step_t(const KParams& p, S* f, int fk, bool trace, cud
             const dim3 grid2 = x2_grid(p);
             const PairDims pd = make_pair_dims(p);
             switch (fk) {
-            case FK_CONST: k_stream_collide_x2<S, ODD, FK_CONST, HO><<<grid2, X2_BLOCK, 0, st>>>(p, pd, f); break;
-            case FK_KOLMOGOROV:
-                k_stream_collide_x2<S, ODD, FK_KOLMOGOROV, HO><<<grid2, X2_BLOCK, 0, st>>>(p, pd, f);
-                break;
-            case FK_FIELD: k_stream_collide_x2<S, ODD, FK_FIELD, HO><<<grid2, X2_BLOCK, 0, st>>>(p, pd, f); break;
-            case FK_SHAN_CHEN:
-                k_stream_collide_x2<S, ODD, FK_SHAN_CHEN, HO><<<grid2, X2_BLOCK, 0, st>>>(p, pd, f);
-                break;
+            case FK_CONST: return launch_pdl(k_stream_collide_x2<S, ODD, FK_CONST, HO>, grid2, X2_BLOCK, 0, st, p, pd, f);
+            case FK_KOLMOGOROV: return launch_pdl(k_stream_collide_x2<S, ODD, FK_KOLMOGOROV, HO>, grid2, X2_BLOCK, 0, st, p, pd, f);
+            case FK_FIELD: return launch_pdl(k_stream_collide_x2<S, ODD, FK_FIELD, HO>, grid2, X2_BLOCK, 0, st, p, pd, f);
+            case FK_SHAN_CHEN: return launch_pdl(k_stream_collide_x2<S, ODD, FK_SHAN_CHEN, HO>, grid2, X2_BLOCK, 0, st, p, pd, f);
             default: return cudaErrorInvalidValue;
             }
-            return cudaGetLastError();
         }
     }
     if (trace) {
         // free streaming is only offered for FP32 storage (bit-exact index checks)
         if constexpr (std::is_same<S, float>::value && !HO)
-            k_stream_collide<S, ODD, LINKS, FK_CONST, true, false><<<grid, block, 0, st>>>(p, f);
+            return launch_pdl(k_stream_collide<S, ODD, LINKS, FK_CONST, true, false>, grid, block, 0, st, p, f);
         else
             return cudaErrorInvalidValue;
-    } else {
-        switch (fk) {
-        case FK_CONST: k_stream_collide<S, ODD, LINKS, FK_CONST, false, HO><<<grid, block, 0, st>>>(p, f); break;
-        case FK_KOLMOGOROV: k_stream_collide<S, ODD, LINKS, FK_KOLMOGOROV, false, HO><<<grid, block, 0, st>>>(p, f); break;
-        case FK_FIELD: k_stream_collide<S, ODD, LINKS, FK_FIELD, false, HO><<<grid, block, 0, st>>>(p, f); break;
-        case FK_SHAN_CHEN: k_stream_collide<S, ODD, LINKS, FK_SHAN_CHEN, false, HO><<<grid, block, 0, st>>>(p, f); break;
-        default: return cudaErrorInvalidValue;
-        }
     }
-    return cudaGetLastError();
+    switch (fk) {
+    case FK_CONST: return launch_pdl(k_stream_collide<S, ODD, LINKS, FK_CONST, false, HO>, grid, block, 0, st, p, f);
+    case FK_KOLMOGOROV: return launch_pdl(k_stream_collide<S, ODD, LINKS, FK_KOLMOGOROV, false, HO>, grid, block, 0, st, p, f);
+    case FK_FIELD: return launch_pdl(k_stream_collide<S, ODD, LINKS, FK_FIELD, false, HO>, grid, block, 0, st, p, f);
+    case FK_SHAN_CHEN: return launch_pdl(k_stream_collide<S, ODD, LINKS, FK_SHAN_CHEN, false, HO>, grid, block, 0, st, p, f);
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 template <typename S, bool ODD, bool HO>
@@ -214,23 +209,11 @@ cudaError_t launch_psi(const KParams& p, const void* f, float* psi, int odd, cud
     const S* fs = static_cast<const S*>(f);
     const dim3 grid = node_grid(p), block(BLOCK_X);
     const bool links = p.links != nullptr;
-    {
-        // fully periodic, even nx: two nodes per thread, with the word gathers of the pair kernel
-        if (!links && p.nx % 2 == 0 && (reinterpret_cast<uintptr_t>(f) & (2 * sizeof(S) - 1)) == 0) {
-            const PairDims pd = make_pair_dims(p);
-            if (odd) k_psi_x2<S, true><<<x2_grid(p), X2_BLOCK, 0, st>>>(p, pd, fs, psi);
-            else k_psi_x2<S, false><<<x2_grid(p), X2_BLOCK, 0, st>>>(p, pd, fs, psi);
-            return cudaGetLastError();
-        }
-    }
-    if (odd) {
-        if (links) k_psi<S, true, true><<<grid, block, 0, st>>>(p, fs, psi);
-        else k_psi<S, true, false><<<grid, block, 0, st>>>(p, fs, psi);
-    } else {
-        if (links) k_psi<S, false, true><<<grid, block, 0, st>>>(p, fs, psi);
-        else k_psi<S, false, false><<<grid, block, 0, st>>>(p, fs, psi);
-    }
-    return cudaGetLastError();
+    // fully periodic, even nx: two nodes per thread, with the word gathers of the pair kernel
+    if (!links && p.nx % 2 == 0 && (reinterpret_cast<uintptr_t>(f) & (2 * sizeof(S) - 1)) == 0)
+        return launch_pdl(odd ? k_psi_x2<S, true> : k_psi_x2<S, false>, x2_grid(p), X2_BLOCK, 0, st, p, make_pair_dims(p), fs, psi);
+    if (odd) return launch_pdl(links ? k_psi<S, true, true> : k_psi<S, true, false>, grid, block, 0, st, p, fs, psi);
+    return launch_pdl(links ? k_psi<S, false, true> : k_psi<S, false, false>, grid, block, 0, st, p, fs, psi);
 }
 
 template <typename S, bool ODD, bool LINKS>

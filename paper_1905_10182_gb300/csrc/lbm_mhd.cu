@@ -136,6 +136,7 @@ struct MhdArgs {
 
 template <bool ODD, bool LINKS>
 __global__ void __launch_bounds__(MHD_BLOCK, 5) k_mhd_step(KParams p, MhdArgs q, float* __restrict__ f) {
+    pdl_wait();
     const int x = blockIdx.x * MHD_BLOCK + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z + p.z0;
     if (x >= p.nx) return;
@@ -259,14 +260,8 @@ cudaError_t launch_mhd_step(const KParams& p, void* f, float* hm, float omega_m,
     const MhdArgs q = args(hm, omega_m, bw);
     float* ff = static_cast<float*>(f);
     const dim3 grid = mhd_grid(p);
-    if (odd) {
-        if (p.links) k_mhd_step<true, true><<<grid, MHD_BLOCK, 0, st>>>(p, q, ff);
-        else k_mhd_step<true, false><<<grid, MHD_BLOCK, 0, st>>>(p, q, ff);
-    } else {
-        if (p.links) k_mhd_step<false, true><<<grid, MHD_BLOCK, 0, st>>>(p, q, ff);
-        else k_mhd_step<false, false><<<grid, MHD_BLOCK, 0, st>>>(p, q, ff);
-    }
-    return cudaGetLastError();
+    if (odd) return launch_pdl(p.links ? k_mhd_step<true, true> : k_mhd_step<true, false>, grid, MHD_BLOCK, 0, st, p, q, ff);
+    return launch_pdl(p.links ? k_mhd_step<false, true> : k_mhd_step<false, false>, grid, MHD_BLOCK, 0, st, p, q, ff);
 }
 
 cudaError_t launch_mhd_fields(const KParams& p, const void* f, float* hm, float omega_m, const float bw[3], int odd,

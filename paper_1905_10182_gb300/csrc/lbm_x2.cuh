@@ -327,6 +327,7 @@ __device__ __forceinline__ void shan_chen_x2(const KParams& p, const uint32_t (&
 template <typename S, bool ODD, int FK, bool HO>
 __global__ void __launch_bounds__(X2_BLOCK, (ODD ? 4 : 5))
     k_stream_collide_x2(KParams p, PairDims pd, S* __restrict__ f) {
+    pdl_wait();
     if (p.pf) x2_prefetch<S, ODD>(p, pd, f);
     const uint32_t G = blockIdx.x * X2_BLOCK + threadIdx.x;
     if (G >= pd.pairs) return;
@@ -455,6 +456,7 @@ __device__ __forceinline__ V2 ld_pair_straddle(const char* a, const char* b) {
 template <typename S, bool ODD>
 __global__ void __launch_bounds__(X2_BLOCK) k_psi_x2(KParams p, PairDims pd, const S* __restrict__ f,
                                                       float* __restrict__ psi) {
+    pdl_wait();
     const uint32_t G = (gridDim.x - 1 - blockIdx.x) * X2_BLOCK + threadIdx.x;
     if (G >= pd.pairs) return;
     const PairMap pm = map_pair(p, pd, G);
