@@ -12,6 +12,7 @@
 // those of the FP64 oracle (orc_cg_*).
 #include "lbm_device.cuh"
 #include "lbm_launch.h"
+#include "lbm_models.cuh"
 
 namespace cmlbm {
 
@@ -190,7 +191,7 @@ __global__ void __launch_bounds__(CG_BLOCK, 4) k_cg_step(KParams p, CgArgs q, fl
 #pragma unroll
     for (int i = 0; i < 27; ++i) f[i] -= weight(i) * p.rho0;
     const CgEquilibriumExtra extra{alpha, nu, gr[0], gr[1], gr[2]};
-    const Macro m = collide_cm<false, CgEquilibriumExtra>(f, Fx, Fy, Fz, omega, p.rho0, 0.0f, 0.0f, extra);
+    const Macro m = model_collide(f, Fx, Fy, Fz, omega, p.rho0, extra);
     const float u2 = m.ux * m.ux + m.uy * m.uy + m.uz * m.uz;
     const bool bad = !(m.rho > 0.0f) || !(u2 < 1.0f);
     if (__any_sync(__activemask(), bad) && bad) atomicOr(p.flag, 1u);

@@ -12,6 +12,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "lbm_vec.cuh"
+
 namespace cmlbm {
 
 // ----------------------------------------------------------------------------- lattice
@@ -339,231 +341,21 @@ __device__ __forceinline__ void inverse_fast_dev(const float (&kd)[3][3][3], flo
 }
 
 // ----------------------------------------------------------------------------- collision
-// The time iteration of Sec. II (steps 1-4), written as an increment so that FP32 rounding
-// scales with the (small) change of each population rather than with the population:
-//   k* - k = Lambda (k^eq - k) + (I - Lambda/2) R        (the post-collision CMs of Sec. II)
-//   f*     = f + (T^T)^-1 (k* - k)                        (Eq. system; T^T is linear)
-// Steps: raw moments of g by three D1Q3 sums; rho, u (Eq. macroscopic); all 27 central moments
-// by three D1Q3 shifts; the increments of Eq. post_collision_central_moments_forcing; the
-// factorised inverse of the increments; g* = g + dg.  The conserved increments are exact by
-// construction: dk_000 = 0 (k0* = k0 = rho) and dk_100 = F_x (k1 = -F_x/2 by Eq. macroscopic,
-// k1* = F_x/2), so mass and momentum move only by rounding of the increment.
+// The collision of one node with FP32 storage: increment form (lbm_vec.cuh), g* = g + dg.
 struct Macro {
     float rho, ux, uy, uz;
 };
 
-// One D1Q3 raw-moment sum along an axis: values at c = -1, 0, +1 -> moments 0, 1, 2.
-__device__ __forceinline__ void d1q3_moments(float pm, float p0, float pp, float& m0, float& m1, float& m2) {
-    const float s2 = pp + pm;
-    m0 = s2 + p0;
-    m1 = pp - pm;
-    m2 = s2;
-}
-
-// One D1Q3 shift from raw to central moments about u, in deviation form: inputs are raw moments
-// minus r*(1, 0, 1/3), outputs central moments minus r*(1, 0, 1/3).
-__device__ __forceinline__ void d1q3_shift_dev(float& m0, float& m1, float& m2, float r, float u) {
-    const float A = r + m0;
-    const float c1 = m1 - u * A;
-    const float c2 = m2 - 2.0f * u * m1 + u * u * A;
-    m1 = c1;
-    m2 = c2;
-}
-
-// One D1Q3 inverse without rest state (a linear map): central moments (m0, m1, m2) about u ->
-// values at c = -1, 0, +1.
-__device__ __forceinline__ void d1q3_inverse_lin(float m0, float m1, float m2, float u, float u2, float& pm,
-                                                 float& p0, float& pp) {
-    const float t = m0 * u2 + m2 + 2.0f * u * m1;
-    const float a = m0 * u + m1;
-    p0 = m0 - t;
-    pp = 0.5f * (t + a);
-    pm = 0.5f * (t - a);
-}
-
-// Models with second-order Hermite truncations (Sec. III: M4 keeps the complete equilibrium with
-// the second-order (Guo) forcing term, M5 truncates both at second order).  For any truncation
-// order >= 2 the central moments of order <= 2 of f^eq and of F_i are those of the complete
-// expansion (the D3Q27 quadrature is exact there), so the five omega-relaxed moments k4..k8 are
-// untouched and only the moments of order >= 3, all relaxed at rate 1 (k* = k^eq + R/2), change.
-// Adds to the monomial post-collision central moments K[a][b][c] (x, y, z orders):
-//   ce * (kappa^eq of the 2nd-order equilibrium - kappa^eq of the complete one)
-// + cf * (kappa of the 2nd-order forcing term - kappa of the complete one),
-// ce = 1 for a second-order equilibrium, cf = 1/2 for a second-order forcing term, else 0.
-// The differences are the central moments of the dropped Hermite terms H^(3)..H^(6) of
-// Eq. eq:truncation and Eq. generalForcing, expanded about u.
-// T: float (one node) or a packed pair of nodes with the same arithmetic operators.
-template <typename T>
-__device__ __forceinline__ void hermite2_correction(T (&K)[3][3][3], T rho, T ux, T uy, T uz, T Fx, T Fy, T Fz,
-                                                    float ce, float cf) {
-    const T re = ce * rho;
-    const T X = ux * ux, Y = uy * uy, Z = uz * uz;
-    // third order, kappa with u_a squared and u_b: -rho u_a^2 u_b; -u_a (2 F_a u_b + F_b u_a)
-    auto t3 = [&](T ua, T ub, T Fa, T Fb) {
-        return -re * ua * ua * ub - cf * ua * (2.0f * Fa * ub + Fb * ua);
-    };
-    K[2][1][0] += t3(ux, uy, Fx, Fy);
-    K[2][0][1] += t3(ux, uz, Fx, Fz);
-    K[1][2][0] += t3(uy, ux, Fy, Fx);
-    K[0][2][1] += t3(uy, uz, Fy, Fz);
-    K[1][0][2] += t3(uz, ux, Fz, Fx);
-    K[0][1][2] += t3(uz, uy, Fz, Fy);
-    K[1][1][1] += -re * ux * uy * uz - cf * (Fx * uy * uz + Fy * ux * uz + Fz * ux * uy);
-    // fourth order, a^2 b^2: 3 rho u_a^2 u_b^2; 4 u_a u_b (F_a u_b + F_b u_a)
-    auto t4 = [&](T ua, T ub, T Fa, T Fb) {
-        return 3.0f * re * ua * ua * ub * ub + 4.0f * cf * ua * ub * (Fa * ub + Fb * ua);
-    };
-    K[2][2][0] += t4(ux, uy, Fx, Fy);
-    K[2][0][2] += t4(ux, uz, Fx, Fz);
-    K[0][2][2] += t4(uy, uz, Fy, Fz);
-    // fourth order, a^2 b c: 3 rho u_a^2 u_b u_c; 2 u_a (2 F_a u_b u_c + F_b u_a u_c + F_c u_a u_b)
-    auto t4m = [&](T ua, T ub, T uc, T Fa, T Fb, T Fc) {
-        return 3.0f * re * ua * ua * ub * uc + 2.0f * cf * ua * (2.0f * Fa * ub * uc + Fb * ua * uc + Fc * ua * ub);
-    };
-    K[2][1][1] += t4m(ux, uy, uz, Fx, Fy, Fz);
-    K[1][2][1] += t4m(uy, ux, uz, Fy, Fx, Fz);
-    K[1][1][2] += t4m(uz, ux, uy, Fz, Fx, Fy);
-    // fifth order, a b^2 c^2: -rho u_a (18 u_b^2 u_c^2 + u_b^2 + u_c^2) / 3;
-    // -(F_a (9 u_b^2 u_c^2 + u_b^2 + u_c^2) + 2 u_a (F_b u_b (9 u_c^2 + 1) + F_c u_c (9 u_b^2 + 1))) / 3
-    auto t5 = [&](T ua, T ub, T uc, T Fa, T Fb, T Fc) {
-        const T b2 = ub * ub, c2 = uc * uc;
-        return -(re * ua * (18.0f * b2 * c2 + b2 + c2) +
-                 cf * (Fa * (9.0f * b2 * c2 + b2 + c2) +
-                       2.0f * ua * (Fb * ub * (9.0f * c2 + 1.0f) + Fc * uc * (9.0f * b2 + 1.0f)))) *
-               (1.0f / 3.0f);
-    };
-    K[1][2][2] += t5(ux, uy, uz, Fx, Fy, Fz);
-    K[2][1][2] += t5(uy, ux, uz, Fy, Fx, Fz);
-    K[2][2][1] += t5(uz, ux, uy, Fz, Fx, Fy);
-    // sixth order: rho (10 X Y Z + X Y + X Z + Y Z); (4/3) sum_a F_a u_a (6 u_b^2 u_c^2 + u_b^2 + u_c^2)
-    K[2][2][2] += re * (10.0f * X * Y * Z + X * Y + X * Z + Y * Z) +
-                  cf * (4.0f / 3.0f) *
-                      (Fx * ux * (6.0f * Y * Z + Y + Z) + Fy * uy * (6.0f * X * Z + X + Z) +
-                       Fz * uz * (6.0f * X * Y + X + Y));
-}
-
-// No change of the equilibrium (the default of collide_increment's Extra hook).
-struct NoExtra {
-    __device__ __forceinline__ void operator()(float (&)[3][3][3], float, float, float, float, float) const {}
-};
-
-// In: K[x][y][z] holds the deviations g arranged by velocity (index c + 1).  Out: K holds the
-// increments dg arranged the same way.  Returns rho and u of the node.  HO: add the
-// second-order-truncation terms of hermite2_correction (weights ce, cf).  extra(K, rho, ux, uy,
-// uz, omega) may add further equilibrium terms to the increments before the inverse transform.
-template <bool HO = false, typename Extra = NoExtra>
-__device__ __forceinline__ Macro collide_increment(float (&K)[3][3][3], float Fx, float Fy, float Fz, float omega,
-                                                   float rho0, float ce = 0.0f, float cf = 0.0f,
-                                                   const Extra& extra = Extra()) {
-    constexpr float s[3] = {1.0f, 0.0f, 1.0f / 3.0f};
-
-    // raw moments of the deviations: z, then y, then x (index: [x][y][z], each either a velocity
-    // c + 1 or a moment order)
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = 0; b < 3; ++b) d1q3_moments(K[a][b][0], K[a][b][1], K[a][b][2], K[a][b][0], K[a][b][1], K[a][b][2]);
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) d1q3_moments(K[a][0][c], K[a][1][c], K[a][2][c], K[a][0][c], K[a][1][c], K[a][2][c]);
-#pragma unroll
-    for (int b = 0; b < 3; ++b)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) d1q3_moments(K[0][b][c], K[1][b][c], K[2][b][c], K[0][b][c], K[1][b][c], K[2][b][c]);
-
-    // step 1: macroscopic variables (Eq. macroscopic)
-    const float dr = K[0][0][0];
-    const float rho = rho0 + dr;
-    const float inv = 1.0f / rho;
-    const float ux = (K[1][0][0] + 0.5f * Fx) * inv;
-    const float uy = (K[0][1][0] + 0.5f * Fy) * inv;
-    const float uz = (K[0][0][1] + 0.5f * Fz) * inv;
-
-    // step 2: central moments (deviation form), x then y then z shifts
-#pragma unroll
-    for (int b = 0; b < 3; ++b)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) d1q3_shift_dev(K[0][b][c], K[1][b][c], K[2][b][c], rho0 * s[b] * s[c], ux);
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) d1q3_shift_dev(K[a][0][c], K[a][1][c], K[a][2][c], rho0 * s[a] * s[c], uy);
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = 0; b < 3; ++b) d1q3_shift_dev(K[a][b][0], K[a][b][1], K[a][b][2], rho0 * s[a] * s[b], uz);
-
-    // step 3: increments k* - k.  k4..k6 = kappa_110, 101, 011 relax at omega; k7 = k200 - k020,
-    // k8 = k200 - k002 at omega; k9 = k200 + k020 + k002 -> rho; every other moment goes to its
-    // post-collision value of Eq. post_collision_central_moments_forcing (rate 1).
-    const float k7 = K[2][0][0] - K[0][2][0];
-    const float k8 = K[2][0][0] - K[0][0][2];
-    const float om1 = 1.0f - omega;
-    const float k7s = om1 * k7, k8s = om1 * k8;
-    const float third = 1.0f / 3.0f;
-    K[0][0][0] = 0.0f;
-    K[1][0][0] = Fx;
-    K[0][1][0] = Fy;
-    K[0][0][1] = Fz;
-    K[1][1][0] = -omega * K[1][1][0];
-    K[1][0][1] = -omega * K[1][0][1];
-    K[0][1][1] = -omega * K[0][1][1];
-    K[2][0][0] = (k7s + k8s + dr) * third - K[2][0][0];
-    K[0][2][0] = (dr - 2.0f * k7s + k8s) * third - K[0][2][0];
-    K[0][0][2] = (dr + k7s - 2.0f * k8s) * third - K[0][0][2];
-    const float fx6 = Fx * (1.0f / 6.0f), fy6 = Fy * (1.0f / 6.0f), fz6 = Fz * (1.0f / 6.0f);
-    K[1][2][0] = fx6 - K[1][2][0];
-    K[1][0][2] = fx6 - K[1][0][2];
-    K[2][1][0] = fy6 - K[2][1][0];
-    K[0][1][2] = fy6 - K[0][1][2];
-    K[2][0][1] = fz6 - K[2][0][1];
-    K[0][2][1] = fz6 - K[0][2][1];
-    K[1][1][1] = -K[1][1][1];
-    const float dr9 = dr * (1.0f / 9.0f);
-    K[2][2][0] = dr9 - K[2][2][0];
-    K[2][0][2] = dr9 - K[2][0][2];
-    K[0][2][2] = dr9 - K[0][2][2];
-    K[2][1][1] = -K[2][1][1];
-    K[1][2][1] = -K[1][2][1];
-    K[1][1][2] = -K[1][1][2];
-    K[1][2][2] = Fx * (1.0f / 18.0f) - K[1][2][2];
-    K[2][1][2] = Fy * (1.0f / 18.0f) - K[2][1][2];
-    K[2][2][1] = Fz * (1.0f / 18.0f) - K[2][2][1];
-    K[2][2][2] = dr * (1.0f / 27.0f) - K[2][2][2];
-    if (HO) hermite2_correction(K, rho, ux, uy, uz, Fx, Fy, Fz, ce, cf);
-    extra(K, rho, ux, uy, uz, omega);
-
-    // step 4: dg = (T^T)^-1 dk, z then y then x inverses; g* = g + dg
-    const float ux2 = ux * ux, uy2 = uy * uy, uz2 = uz * uz;
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = 0; b < 3; ++b)
-            d1q3_inverse_lin(K[a][b][0], K[a][b][1], K[a][b][2], uz, uz2, K[a][b][0], K[a][b][1], K[a][b][2]);
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-            d1q3_inverse_lin(K[a][0][c], K[a][1][c], K[a][2][c], uy, uy2, K[a][0][c], K[a][1][c], K[a][2][c]);
-#pragma unroll
-    for (int b = 0; b < 3; ++b)
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-            d1q3_inverse_lin(K[0][b][c], K[1][b][c], K[2][b][c], ux, ux2, K[0][b][c], K[1][b][c], K[2][b][c]);
-    return Macro{rho, ux, uy, uz};
-}
-
-template <bool HO = false, typename Extra = NoExtra>
+template <bool HO = false>
 __device__ __forceinline__ Macro collide_cm(float (&g)[27], float Fx, float Fy, float Fz, float omega, float rho0,
-                                            float ce = 0.0f, float cf = 0.0f, const Extra& extra = Extra()) {
-    float K[3][3][3];
+                                            float ce = 0.0f, float cf = 0.0f) {
+    F1 K[3][3][3];
 #pragma unroll
-    for (int i = 0; i < 27; ++i) K[dir_x(i) + 1][dir_y(i) + 1][dir_z(i) + 1] = g[i];
-    const Macro m = collide_increment<HO, Extra>(K, Fx, Fy, Fz, omega, rho0, ce, cf, extra);
+    for (int i = 0; i < 27; ++i) K[dir_x(i) + 1][dir_y(i) + 1][dir_z(i) + 1] = F1{g[i]};
+    const MacroT<F1> m = collide_increment<HO>(K, F1{Fx}, F1{Fy}, F1{Fz}, omega, rho0, ce, cf);
 #pragma unroll
-    for (int i = 0; i < 27; ++i) g[i] += K[dir_x(i) + 1][dir_y(i) + 1][dir_z(i) + 1];
-    return m;
+    for (int i = 0; i < 27; ++i) g[i] = __fadd_rn(g[i], K[dir_x(i) + 1][dir_y(i) + 1][dir_z(i) + 1].v);
+    return Macro{m.rho.v, m.ux.v, m.uy.v, m.uz.v};
 }
 
 // Direct form of the same collision, f* = (T^T)^-1 k* (Eq. system) with k* of

@@ -181,6 +181,26 @@ static cudaError_t launch_step_t(const KParams& p, S* f, int fk, bool trace, cud
             }
         }
     }
+    if constexpr (sizeof(S) == 4 && !LINKS) {
+        // FP32 storage, the same (byte offsets within a plane are 32-bit).  Measured against the one-node
+        // kernel: store in L2 64^3 10.9 -> 7.6 us, 128x128x48 25.2 -> 20.2; store beyond L2 (p.pf) 192^3
+        // 241 -> 227 us, where the one-node kernel's rows leave lanes idle (nx no multiple of 128); but
+        // 256^3 528 -> 534 and 512^3 4.20 -> 4.31 ms: there both run at the copy rate and the pair
+        // kernel's odd step pays for its 4-byte stores.  With the Shan-Chen stencil the pair wins at
+        // every size (128^3: psi pass and step 109 -> 101 us).
+        const bool rows_full = p.pf != 0 && p.nx % BLOCK_X == 0 && fk != FK_SHAN_CHEN;
+        if (!trace && !rows_full && p.nx % 2 == 0 && (reinterpret_cast<uintptr_t>(f) & 7) == 0 && p.N < (1LL << 30)) {
+            const dim3 grid2 = x2_grid(p);
+            const PairDims pd = make_pair_dims(p);
+            switch (fk) {
+            case FK_CONST: return launch_pdl(k_stream_collide_x2f<ODD, FK_CONST, HO>, grid2, X2_BLOCK, 0, st, p, pd, f);
+            case FK_KOLMOGOROV: return launch_pdl(k_stream_collide_x2f<ODD, FK_KOLMOGOROV, HO>, grid2, X2_BLOCK, 0, st, p, pd, f);
+            case FK_FIELD: return launch_pdl(k_stream_collide_x2f<ODD, FK_FIELD, HO>, grid2, X2_BLOCK, 0, st, p, pd, f);
+            case FK_SHAN_CHEN: return launch_pdl(k_stream_collide_x2f<ODD, FK_SHAN_CHEN, HO>, grid2, X2_BLOCK, 0, st, p, pd, f);
+            default: return cudaErrorInvalidValue;
+            }
+        }
+    }
     if (trace) {
         // free streaming is only offered for FP32 storage (bit-exact index checks)
         if constexpr (std::is_same<S, float>::value && !HO)

@@ -16,6 +16,7 @@
 // field holds fewer than 2^32 / 27 nodes, so element offsets are 32-bit.
 #include "lbm_device.cuh"
 #include "lbm_launch.h"
+#include "lbm_models.cuh"
 
 namespace cmlbm {
 
@@ -150,7 +151,7 @@ __global__ void __launch_bounds__(MHD_BLOCK, 5) k_mhd_step(KParams p, MhdArgs q,
     const MhdNode m = mhd_node(g, h, p.rho0, Fe, q.omega_m);
     mhd_collide(h, m.b, m.u, q.omega_m);
     mhd_scatter<ODD, LINKS>(q.hm, p.N, nb, link, q.bw, h);
-    const Macro mc = collide_cm(g, Fe[0] + m.FL[0], Fe[1] + m.FL[1], Fe[2] + m.FL[2], p.omega, p.rho0);
+    const Macro mc = model_collide(g, Fe[0] + m.FL[0], Fe[1] + m.FL[1], Fe[2] + m.FL[2], p.omega, p.rho0);
     const float u2 = mc.ux * mc.ux + mc.uy * mc.uy + mc.uz * mc.uz;
     const bool bad = !(mc.rho > 0.0f) || !(u2 < 1.0f);
     if (__any_sync(__activemask(), bad) && bad) atomicOr(p.flag, 1u);

@@ -17,24 +17,6 @@ namespace cmlbm {
 
 constexpr int X2_BLOCK = 128;  // threads per block: 128 consecutive node pairs (rows numbered one after another)
 
-// ----------------------------------------------------------------------------- packed pairs
-struct V2 {
-    float2 v;  // .x: node x, .y: node x + 1
-};
-__device__ __forceinline__ V2 bc(float a) { return V2{make_float2(a, a)}; }
-__device__ __forceinline__ V2 operator+(V2 a, V2 b) { return V2{__fadd2_rn(a.v, b.v)}; }
-__device__ __forceinline__ V2 operator-(V2 a, V2 b) { return V2{__ffma2_rn(b.v, make_float2(-1.0f, -1.0f), a.v)}; }
-__device__ __forceinline__ V2 operator-(V2 a) { return V2{__fmul2_rn(a.v, make_float2(-1.0f, -1.0f))}; }
-__device__ __forceinline__ V2 operator*(V2 a, V2 b) { return V2{__fmul2_rn(a.v, b.v)}; }
-__device__ __forceinline__ V2 operator*(float a, V2 b) { return V2{__fmul2_rn(make_float2(a, a), b.v)}; }
-__device__ __forceinline__ V2 operator*(V2 a, float b) { return V2{__fmul2_rn(a.v, make_float2(b, b))}; }
-__device__ __forceinline__ V2 operator+(V2 a, float b) { return V2{__fadd2_rn(a.v, make_float2(b, b))}; }
-__device__ __forceinline__ V2& operator+=(V2& a, V2 b) {
-    a = a + b;
-    return a;
-}
-__device__ __forceinline__ V2 fma2(V2 a, V2 b, V2 c) { return V2{__ffma2_rn(a.v, b.v, c.v)}; }
-
 // 16-bit codecs of a node pair: the 32-bit word holds node x in its low half.
 template <typename S>
 struct Pair;
@@ -66,18 +48,16 @@ template <bool Z1, bool Z2, bool REST>
 __device__ __forceinline__ void inv1_x2(V2 m0, V2 m1, V2 m2, float r, V2 u, V2 u2, V2 twou, V2& pm, V2& p0,
                                         V2& pp) {
     const V2 A = REST ? m0 + r : m0;
-    V2 t = Z2 ? A * u2 : fma2(A, u2, m2);
-    if (!Z1) t = fma2(twou, m1, t);
+    V2 t = Z2 ? A * u2 : vfma(A, u2, m2);
+    if (!Z1) t = vfma(twou, m1, t);
     p0 = m0 - t;
-    const V2 Au = Z1 ? A * u : fma2(A, u, m1);
+    const V2 Au = Z1 ? A * u : vfma(A, u, m1);
     const V2 ht = t * 0.5f;
-    pp = fma2(bc(0.5f), Au, ht);
-    pm = fma2(bc(-0.5f), Au, ht);
+    pp = vfma(bc(0.5f), Au, ht);
+    pm = vfma(bc(-0.5f), Au, ht);
 }
 
-struct Macro2 {
-    V2 rho, ux, uy, uz;
-};
+using Macro2 = MacroT<V2>;
 
 // The direct-form collision (collide_cm_direct) on a node pair.  g: deviations in, f* - w rho0 out.
 template <bool HO>
@@ -121,19 +101,19 @@ __device__ __forceinline__ Macro2 collide_direct_x2(V2 (&g)[27], V2 Fx, V2 Fy, V
     const V2 dr = m000;
     const V2 rho = dr + rho0;
     const V2 inv = V2{make_float2(1.0f / rho.v.x, 1.0f / rho.v.y)};
-    const V2 ux = fma2(h, Fx, m100) * inv;
-    const V2 uy = fma2(h, Fy, m010) * inv;
-    const V2 uz = fma2(h, Fz, m001) * inv;
+    const V2 ux = vfma(h, Fx, m100) * inv;
+    const V2 uy = vfma(h, Fy, m010) * inv;
+    const V2 uz = vfma(h, Fz, m001) * inv;
     // step 2: k4..k8 (Eq. pre_collision)
     const V2 nrho = -rho;
     const V2 nrux = nrho * ux, nruy = nrho * uy;
-    const V2 k4 = fma2(h, fma2(ux, Fy, uy * Fx), fma2(nrux, uy, m110));
-    const V2 k5 = fma2(h, fma2(ux, Fz, uz * Fx), fma2(nrux, uz, m101));
-    const V2 k6 = fma2(h, fma2(uy, Fz, uz * Fy), fma2(nruy, uz, m011));
+    const V2 k4 = vfma(h, vfma(ux, Fy, uy * Fx), vfma(nrux, uy, m110));
+    const V2 k5 = vfma(h, vfma(ux, Fz, uz * Fx), vfma(nrux, uz, m101));
+    const V2 k6 = vfma(h, vfma(uy, Fz, uz * Fy), vfma(nruy, uz, m011));
     const V2 ux2 = ux * ux, uy2 = uy * uy, uz2 = uz * uz;
     const V2 uFx = ux * Fx, uFy = uy * Fy, uFz = uz * Fz;
-    const V2 k7 = fma2(nrho, ux2 - uy2, m200 - m020) + (uFx - uFy);
-    const V2 k8 = fma2(nrho, ux2 - uz2, m200 - m002) + (uFx - uFz);
+    const V2 k7 = vfma(nrho, ux2 - uy2, m200 - m020) + (uFx - uFy);
+    const V2 k8 = vfma(nrho, ux2 - uz2, m200 - m002) + (uFx - uFz);
     // step 3: post-collision CMs (Eq. post_collision_central_moments_forcing) minus rest moments
     const float om1 = 1.0f - omega;
     const V2 k7s = k7 * om1, k8s = k8 * om1;
@@ -147,8 +127,8 @@ __device__ __forceinline__ Macro2 collide_direct_x2(V2 (&g)[27], V2 Fx, V2 Fy, V
     kd[1][0][1] = k5 * om1;
     kd[0][1][1] = k6 * om1;
     kd[2][0][0] = (k7s + k8s + dr) * third;
-    kd[0][2][0] = fma2(bc(-2.0f), k7s, k8s + dr) * third;
-    kd[0][0][2] = fma2(bc(-2.0f), k8s, k7s + dr) * third;
+    kd[0][2][0] = vfma(bc(-2.0f), k7s, k8s + dr) * third;
+    kd[0][0][2] = vfma(bc(-2.0f), k8s, k7s + dr) * third;
     kd[1][2][0] = kd[1][0][2] = Fx * (1.0f / 6.0f);
     kd[2][1][0] = kd[0][1][2] = Fy * (1.0f / 6.0f);
     kd[2][0][1] = kd[0][2][1] = Fz * (1.0f / 6.0f);
@@ -245,29 +225,33 @@ inline dim3 x2_grid(const KParams& p) {
     return dim3((make_pair_dims(p).pairs + X2_BLOCK - 1) / X2_BLOCK, 1, 1);
 }
 
-// L2 prefetch as in the one-node kernel (k1_prefetch): the 27 x 4 lines (one per 32 pairs and
-// plane) that the block p.pf places later will gather, one per thread (each 32 pairs lie in one
-// row when nx is a multiple of 64; otherwise a line may cover the start of the next row, and the
-// prefetch only misses part of it).
+// L2 prefetch as in the one-node kernel (k1_prefetch): the lines (LPW per 32 pairs and plane) that
+// the block p.pf places later will gather (each 32 pairs lie in one row when nx is a multiple of 64;
+// otherwise a line may cover the start of the next row, and the prefetch only misses part of it).
+// Distance: p.pf blocks for 16-bit storage, 3/4 of it for FP32, whose blocks hold twice the bytes
+// (256^3, one step at 1/2, 3/4, 1 and 3/2 of p.pf: FP32 536, 534, 537, 552 us, FP16 296, 294, 294, 294).
 template <typename S, bool ODD>
 __device__ __forceinline__ void x2_prefetch(const KParams& p, const PairDims& pd, const S* f) {
-    const uint32_t t = threadIdx.x;
-    if (t >= 27 * (X2_BLOCK / 32)) return;
-    const uint32_t k = t / (X2_BLOCK / 32), w = t - k * (X2_BLOCK / 32);
-    const uint32_t G = (blockIdx.x + (uint32_t)p.pf) * X2_BLOCK + 32 * w;
-    if (G >= pd.pairs) return;
-    const uint32_t row = pd.np.div(G);
-    const uint32_t zr = pd.ny.div(row);
-    int yk = (int)(row - zr * (uint32_t)p.ny), zk = (int)zr + p.z0;
-    if (ODD) {
-        constexpr unsigned long long CY = pack_dir(1), CZ = pack_dir(2);
-        yk += (int)((CY >> (2 * k)) & 3ull) - 1;
-        zk += (int)((CZ >> (2 * k)) & 3ull) - 1;
-        yk = yk < 0 ? p.ny - 1 : (yk >= p.ny ? 0 : yk);
-        zk = zk < 0 ? p.nz - 1 : (zk >= p.nz ? 0 : zk);
+    const uint32_t ahead = sizeof(S) == 4 ? (uint32_t)p.pf * 3 / 4 : (uint32_t)p.pf;
+    constexpr uint32_t LPW = 64 * sizeof(S) / 128, LPB = LPW * (X2_BLOCK / 32);  // lines per warp and per block, of a plane
+#pragma unroll
+    for (uint32_t t = threadIdx.x; t < 27 * LPB; t += X2_BLOCK) {
+        const uint32_t k = t / LPB, w = t - k * LPB;
+        const uint32_t G = (blockIdx.x + ahead) * X2_BLOCK + w * (32 / LPW);
+        if (G >= pd.pairs) return;
+        const uint32_t row = pd.np.div(G);
+        const uint32_t zr = pd.ny.div(row);
+        int yk = (int)(row - zr * (uint32_t)p.ny), zk = (int)zr + p.z0;
+        if (ODD) {
+            constexpr unsigned long long CY = pack_dir(1), CZ = pack_dir(2);
+            yk += (int)((CY >> (2 * k)) & 3ull) - 1;
+            zk += (int)((CZ >> (2 * k)) & 3ull) - 1;
+            yk = yk < 0 ? p.ny - 1 : (yk >= p.ny ? 0 : yk);
+            zk = zk < 0 ? p.nz - 1 : (zk >= p.nz ? 0 : zk);
+        }
+        const S* a = f + (unsigned long long)p.N * k + ((unsigned long long)zk * p.ny + yk) * p.nx + 2 * (G - row * pd.np.d);
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(a));
     }
-    const S* a = f + (unsigned long long)p.N * k + ((unsigned long long)zk * p.ny + yk) * p.nx + 2 * (G - row * pd.np.d);
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(a));
 }
 
 // 32-bit words and 16-bit halves of the store at byte addresses.  Row pointers (one per (y, z)
@@ -309,9 +293,9 @@ __device__ __forceinline__ void shan_chen_x2(const KParams& p, const uint32_t (&
                 pl = V2{make_float2(c.y, R.x)};
             }
             const float wyz = w1(dy) * w1(dz);
-            sx = fma2(bc(wyz * w1(1)), pl - m, sx);
+            sx = vfma(bc(wyz * w1(1)), pl - m, sx);
             if (dy != 0 || dz != 0) {
-                const V2 tot = fma2(bc(w1(1)), pl + m, z0 * w1(0)) * wyz;
+                const V2 tot = vfma(bc(w1(1)), pl + m, z0 * w1(0)) * wyz;
                 if (dy != 0) sy = dy > 0 ? sy + tot : sy - tot;
                 if (dz != 0) sz = dz > 0 ? sz + tot : sz - tot;
             } else {
@@ -322,6 +306,43 @@ __device__ __forceinline__ void shan_chen_x2(const KParams& p, const uint32_t (&
     Fx = a * sx;
     Fy = a * sy;
     Fz = a * sz;
+}
+
+// Force density of the pair.
+template <bool ODD, int FK>
+__device__ __forceinline__ void pair_force(const KParams& p, const uint32_t (&yo)[3], const uint32_t (&zo)[3], uint32_t x0,
+                                           uint32_t xl, uint32_t xr, uint32_t y, V2& Fx, V2& Fy, V2& Fz) {
+    if (FK == FK_CONST) {
+        Fx = bc(p.F[0]);
+        Fy = bc(p.F[1]);
+        Fz = bc(p.F[2]);
+    } else if (FK == FK_KOLMOGOROV) {
+        Fx = bc(p.kolm[y]);
+        Fy = Fz = bc(0.0f);
+    } else if (FK == FK_FIELD) {
+        const uint32_t row = zo[1] + yo[1], self = row + x0;
+        if (ODD) {
+            const uint32_t sa = row + (x0 == 0 ? (uint32_t)p.nx - 1 : x0 - 1);
+            Fx = V2{make_float2(p.fx[sa], p.fx[self])};
+            Fy = V2{make_float2(p.fy[sa], p.fy[self])};
+            Fz = V2{make_float2(p.fz[sa], p.fz[self])};
+        } else {
+            Fx = V2{*reinterpret_cast<const float2*>(p.fx + self)};
+            Fy = V2{*reinterpret_cast<const float2*>(p.fy + self)};
+            Fz = V2{*reinterpret_cast<const float2*>(p.fz + self)};
+        }
+    } else {
+        shan_chen_x2<ODD>(p, yo, zo, x0, xl, xr, Fx, Fy, Fz);
+    }
+}
+
+// Flags a pair with a node outside the physical range (see check_node).
+__device__ __forceinline__ void check_pair(const KParams& p, const Macro2& m) {
+    const V2 u2 = vfma(m.ux, m.ux, vfma(m.uy, m.uy, m.uz * m.uz));
+    const bool bad = !(m.rho.v.x > 0.0f) || !(m.rho.v.y > 0.0f) || !(u2.v.x < 1.0f) || !(u2.v.y < 1.0f);
+    if (__any_sync(__activemask(), bad)) {
+        if (bad) atomicOr(p.flag, 1u);
+    }
 }
 
 template <typename S, bool ODD, int FK, bool HO>
@@ -340,7 +361,6 @@ __global__ void __launch_bounds__(X2_BLOCK, (ODD ? 4 : 5))
     const uint32_t pl = nx * ny;
     const uint32_t zm = z == 0 ? nz - 1 : z - 1, zp = z == nz - 1 ? 0 : z + 1;
     const uint32_t zo[3] = {zm * pl, z * pl, zp * pl};
-    const uint32_t self = zo[1] + yo[1] + x0;
     // x of the words W(p - 1), W(p + 1) (periodic in the row)
     const uint32_t xl = x0 == 0 ? nx - 2 : x0 - 2, xr = x0 + 2 == nx ? 0 : x0 + 2;
     const uint64_t PB = (uint64_t)p.N * sizeof(S);
@@ -371,35 +391,9 @@ __global__ void __launch_bounds__(X2_BLOCK, (ODD ? 4 : 5))
     }
 
     V2 Fx, Fy, Fz;
-    if (FK == FK_CONST) {
-        Fx = bc(p.F[0]);
-        Fy = bc(p.F[1]);
-        Fz = bc(p.F[2]);
-    } else if (FK == FK_KOLMOGOROV) {
-        Fx = bc(p.kolm[y]);
-        Fy = Fz = bc(0.0f);
-    } else if (FK == FK_FIELD) {
-        if (ODD) {
-            const uint32_t sa = zo[1] + yo[1] + (x0 == 0 ? nx - 1 : x0 - 1);
-            Fx = V2{make_float2(p.fx[sa], p.fx[self])};
-            Fy = V2{make_float2(p.fy[sa], p.fy[self])};
-            Fz = V2{make_float2(p.fz[sa], p.fz[self])};
-        } else {
-            Fx = V2{*reinterpret_cast<const float2*>(p.fx + self)};
-            Fy = V2{*reinterpret_cast<const float2*>(p.fy + self)};
-            Fz = V2{*reinterpret_cast<const float2*>(p.fz + self)};
-        }
-    } else {
-        shan_chen_x2<ODD>(p, yo, zo, x0, xl, xr, Fx, Fy, Fz);
-    }
+    pair_force<ODD, FK>(p, yo, zo, x0, xl, xr, y, Fx, Fy, Fz);
     const Macro2 m = collide_direct_x2<HO>(g, Fx, Fy, Fz, p.omega, p.rho0, p.ce, p.cf);
-    {
-        const V2 u2 = fma2(m.ux, m.ux, fma2(m.uy, m.uy, m.uz * m.uz));
-        const bool bad = !(m.rho.v.x > 0.0f) || !(m.rho.v.y > 0.0f) || !(u2.v.x < 1.0f) || !(u2.v.y < 1.0f);
-        if (__any_sync(__activemask(), bad)) {
-            if (bad) atomicOr(p.flag, 1u);
-        }
-    }
+    check_pair(p, m);
 
     // AA scatter (w: f*_i of the pair's first node in the low half, of its second in the high half)
     if (ODD) {  // row pointers again, from a value the compiler cannot tie to the ones above (so
@@ -426,6 +420,103 @@ __global__ void __launch_bounds__(X2_BLOCK, (ODD ? 4 : 5))
             } else {  // targets x0 - 1 (high half of W(p - 1)), x0 (low half of W(p))
                 st_half(a + eL + sizeof(S), w & 0xffffu);
                 st_half(a, w >> 16);
+            }
+        }
+    }
+}
+
+// FP32 storage, two nodes per thread: the same pairs and words (now 8 bytes) as the 16-bit kernel,
+// the increment form of the collision.  It needs the 27 populations and their 27 increments of both
+// nodes; the populations wait in shared memory (each thread its own column, filled by cp.async, so
+// no barrier), which leaves the registers to the increments: 92 (even) and 96 registers, five blocks
+// per SM; with both in registers it took 144 and 154, three blocks (128x128x48: 24.8 instead of
+// 22.3 us).  Bound by L2 (store in L2: 8.4 TB/s of 9.2 a plain copy in L2 reaches) or HBM.  A persistent
+// form that prefetched its next tile into a second stage was slower (26.7 us): its blocks drift
+// apart and more bytes in flight only thrash.
+__device__ __forceinline__ void cp_async8(uint32_t s, const char* g) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(s), "l"(g) : "memory");
+}
+__device__ __forceinline__ void cp_async4(uint32_t s, const char* g) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(s), "l"(g) : "memory");
+}
+
+template <bool ODD, int FK, bool HO>
+__global__ void __launch_bounds__(X2_BLOCK, 5) k_stream_collide_x2f(KParams p, PairDims pd, float* __restrict__ f) {
+    __shared__ float2 stage[27][X2_BLOCK];
+    pdl_wait();
+    if (p.pf) x2_prefetch<float, ODD>(p, pd, f);
+    const uint32_t G = blockIdx.x * X2_BLOCK + threadIdx.x;
+    if (G >= pd.pairs) return;
+    const uint32_t nx = p.nx, ny = p.ny, nz = p.nz;
+    const uint64_t PB = (uint64_t)p.N * sizeof(float);
+    char* fb = reinterpret_cast<char*>(f);
+    const uint32_t col = (uint32_t)__cvta_generic_to_shared(&stage[0][threadIdx.x]);
+    constexpr uint32_t LD = X2_BLOCK * sizeof(float2);
+
+    V2 Fx, Fy, Fz;
+    {
+        const PairMap pm = map_pair(p, pd, G);
+        const uint32_t x0 = 2 * pm.pair, y = pm.y, z = pm.z;
+        const uint32_t yo[3] = {(y == 0 ? ny - 1 : y - 1) * nx, y * nx, (y == ny - 1 ? 0 : y + 1) * nx};
+        const uint32_t pl = nx * ny;
+        const uint32_t zo[3] = {(z == 0 ? nz - 1 : z - 1) * pl, z * pl, (z == nz - 1 ? 0 : z + 1) * pl};
+        const uint32_t xl = x0 == 0 ? nx - 2 : x0 - 2, xr = x0 + 2 == nx ? 0 : x0 + 2;
+#pragma unroll
+        for (int i = 0; i < 27; ++i) {
+            const uint32_t s = col + (uint32_t)i * LD;
+            if (!ODD) {
+                cp_async8(s, fb + PB * i + (zo[1] + yo[1] + x0) * 4u);
+            } else {
+                const char* plane = fb + PB * dir_opp(i);
+                const uint32_t r = zo[1 - dir_z(i)] + yo[1 - dir_y(i)];
+                if (dir_x(i) > 0) {
+                    cp_async8(s, plane + (r + xl) * 4u);
+                } else if (dir_x(i) < 0) {
+                    cp_async8(s, plane + (r + x0) * 4u);
+                } else {
+                    cp_async4(s, plane + (r + xl + 1) * 4u);
+                    cp_async4(s + 4, plane + (r + x0) * 4u);
+                }
+            }
+        }
+        pair_force<ODD, FK>(p, yo, zo, x0, xl, xr, y, Fx, Fy, Fz);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    V2 K[3][3][3];
+#pragma unroll
+    for (int i = 0; i < 27; ++i) {
+        float2 v;
+        asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(col + (uint32_t)i * LD));
+        K[dir_x(i) + 1][dir_y(i) + 1][dir_z(i) + 1] = V2{v};
+    }
+    const Macro2 m = collide_increment<HO>(K, Fx, Fy, Fz, p.omega, p.rho0, p.ce, p.cf);
+    check_pair(p, m);
+
+    // AA scatter; the pair's offsets again, from a value the compiler cannot tie to the one above (so
+    // that it holds none of them through the collision)
+    const PairMap pm = map_pair(p, pd, opaque(G));
+    const uint32_t x0 = 2 * pm.pair, y = pm.y, z = pm.z;
+    const uint32_t yo[3] = {(y == 0 ? ny - 1 : y - 1) * nx, y * nx, (y == ny - 1 ? 0 : y + 1) * nx};
+    const uint32_t pl = nx * ny;
+    const uint32_t zo[3] = {(z == 0 ? nz - 1 : z - 1) * pl, z * pl, (z == nz - 1 ? 0 : z + 1) * pl};
+    const uint32_t xl = x0 == 0 ? nx - 2 : x0 - 2;
+#pragma unroll
+    for (int i = 0; i < 27; ++i) {
+        float2 g;
+        asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(g.x), "=f"(g.y) : "r"(col + (uint32_t)i * LD));
+        const V2 v = V2{g} + K[dir_x(i) + 1][dir_y(i) + 1][dir_z(i) + 1];
+        if (!ODD) {
+            *reinterpret_cast<float2*>(fb + PB * dir_opp(i) + (zo[1] + yo[1] + x0) * 4u) = v.v;
+        } else {
+            char* plane = fb + PB * i;
+            const uint32_t r = zo[1 + dir_z(i)] + yo[1 + dir_y(i)];
+            if (dir_x(i) > 0) {
+                *reinterpret_cast<float2*>(plane + (r + x0) * 4u) = v.v;
+            } else if (dir_x(i) < 0) {
+                *reinterpret_cast<float2*>(plane + (r + xl) * 4u) = v.v;
+            } else {
+                *reinterpret_cast<float*>(plane + (r + xl + 1) * 4u) = v.v.x;
+                *reinterpret_cast<float*>(plane + (r + x0) * 4u) = v.v.y;
             }
         }
     }
