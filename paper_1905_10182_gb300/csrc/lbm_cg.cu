@@ -18,8 +18,6 @@ namespace cmlbm {
 
 namespace {
 
-constexpr int CG_BLOCK = 128;
-
 __host__ __device__ constexpr int shell_of(int i) { return dir_x(i) * dir_x(i) + dir_y(i) * dir_y(i) + dir_z(i) * dir_z(i); }
 
 // phi_i(alpha) of App. D
@@ -140,12 +138,11 @@ __device__ __forceinline__ void gather_two(const float* __restrict__ fr, const f
     }
 }
 
-template <bool ODD, bool LINKS>
-__global__ void __launch_bounds__(CG_BLOCK) k_cg_fields(KParams p, CgArgs q, const float* __restrict__ fr) {
+template <bool ODD, bool LINKS, bool FLAT>
+__global__ void __launch_bounds__(BLOCK_X) k_cg_fields(KParams p, CgArgs q, const float* __restrict__ fr) {
     pdl_wait();
-    const int x = blockIdx.x * CG_BLOCK + threadIdx.x;
-    const int y = blockIdx.y, z = blockIdx.z;
-    if (x >= p.nx) return;
+    int x, y, z;
+    if (!node_of<FLAT>(p, x, y, z)) return;
     const Nbr nb(x, y, z, p);
     const uint32_t link = LINKS ? p.links[nb.self()] : 0u;
     float f[27], rr, rb;
@@ -153,12 +150,11 @@ __global__ void __launch_bounds__(CG_BLOCK) k_cg_fields(KParams p, CgArgs q, con
     reinterpret_cast<float2*>(q.fld)[nb.self()] = make_float2(order_param(q, rr, rb), rr + rb);
 }
 
-template <bool ODD, bool LINKS>
-__global__ void __launch_bounds__(CG_BLOCK, 4) k_cg_step(KParams p, CgArgs q, float* __restrict__ fr) {
+template <bool ODD, bool LINKS, bool FLAT>
+__global__ void __launch_bounds__(BLOCK_X, 4) k_cg_step(KParams p, CgArgs q, float* __restrict__ fr) {
     pdl_wait();
-    const int x = blockIdx.x * CG_BLOCK + threadIdx.x;
-    const int y = blockIdx.y, z = blockIdx.z;
-    if (x >= p.nx) return;
+    int x, y, z;
+    if (!node_of<FLAT>(p, x, y, z)) return;
     const Nbr nb(x, y, z, p);
     const uint32_t self = nb.self();
     const uint32_t link = LINKS ? p.links[self] : 0u;
@@ -226,9 +222,9 @@ __global__ void __launch_bounds__(CG_BLOCK, 4) k_cg_step(KParams p, CgArgs q, fl
 
 // rho, u (with F/2), rho_r, rho_b at the current time: 6 planes of N
 template <bool ODD, bool LINKS>
-__global__ void __launch_bounds__(CG_BLOCK) k_cg_macro(KParams p, CgArgs q, const float* __restrict__ fr,
+__global__ void __launch_bounds__(BLOCK_X) k_cg_macro(KParams p, CgArgs q, const float* __restrict__ fr,
                                                        float* __restrict__ out) {
-    const int x = blockIdx.x * CG_BLOCK + threadIdx.x;
+    const int x = blockIdx.x * BLOCK_X + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z;
     if (x >= p.nx) return;
     const Nbr nb(x, y, z, p);
@@ -253,9 +249,9 @@ __global__ void __launch_bounds__(CG_BLOCK) k_cg_macro(KParams p, CgArgs q, cons
 }
 
 // initial state at rest: fk_i = rho_k phi_i(alpha(phi)), natural order (parity 0)
-__global__ void __launch_bounds__(CG_BLOCK) k_cg_init(KParams p, CgArgs q, float* __restrict__ fr,
+__global__ void __launch_bounds__(BLOCK_X) k_cg_init(KParams p, CgArgs q, float* __restrict__ fr,
                                                       const float* __restrict__ rr_in, const float* __restrict__ rb_in) {
-    const int x = blockIdx.x * CG_BLOCK + threadIdx.x;
+    const int x = blockIdx.x * BLOCK_X + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z;
     if (x >= p.nx) return;
     const long long n = (long long)x + (long long)p.nx * ((long long)y + (long long)p.ny * z);
@@ -272,9 +268,9 @@ __global__ void __launch_bounds__(CG_BLOCK) k_cg_init(KParams p, CgArgs q, float
 
 // natural-order copy of both stores (to_buf: out, else in at parity 0); buf: 54 N (red, then blue)
 template <bool ODD, bool LINKS>
-__global__ void __launch_bounds__(CG_BLOCK) k_cg_copy(KParams p, CgArgs q, float* __restrict__ fr, float* __restrict__ buf,
+__global__ void __launch_bounds__(BLOCK_X) k_cg_copy(KParams p, CgArgs q, float* __restrict__ fr, float* __restrict__ buf,
                                                       int to_buf) {
-    const int x = blockIdx.x * CG_BLOCK + threadIdx.x;
+    const int x = blockIdx.x * BLOCK_X + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z;
     if (x >= p.nx) return;
     const Nbr nb(x, y, z, p);
@@ -298,8 +294,6 @@ __global__ void __launch_bounds__(CG_BLOCK) k_cg_copy(KParams p, CgArgs q, float
     }
 }
 
-dim3 cg_grid(const KParams& p) { return dim3((p.nx + CG_BLOCK - 1) / CG_BLOCK, p.ny, p.nz); }
-
 CgArgs cg_args(const CgParams& c, float* fb, float* fld) {
     CgArgs q;
     q.fb = fb;
@@ -322,11 +316,11 @@ CgArgs cg_args(const CgParams& c, float* fb, float* fld) {
 #define CMLBM_CG_DISPATCH(KERNEL, ...)                                                      \
     do {                                                                                   \
         if (odd) {                                                                         \
-            if (p.links) KERNEL<true, true><<<cg_grid(p), CG_BLOCK, 0, st>>>(__VA_ARGS__);   \
-            else KERNEL<true, false><<<cg_grid(p), CG_BLOCK, 0, st>>>(__VA_ARGS__);          \
+            if (p.links) KERNEL<true, true><<<node_grid(p, false), BLOCK_X, 0, st>>>(__VA_ARGS__);   \
+            else KERNEL<true, false><<<node_grid(p, false), BLOCK_X, 0, st>>>(__VA_ARGS__);          \
         } else {                                                                           \
-            if (p.links) KERNEL<false, true><<<cg_grid(p), CG_BLOCK, 0, st>>>(__VA_ARGS__);  \
-            else KERNEL<false, false><<<cg_grid(p), CG_BLOCK, 0, st>>>(__VA_ARGS__);         \
+            if (p.links) KERNEL<false, true><<<node_grid(p, false), BLOCK_X, 0, st>>>(__VA_ARGS__);  \
+            else KERNEL<false, false><<<node_grid(p, false), BLOCK_X, 0, st>>>(__VA_ARGS__);         \
         }                                                                                  \
     } while (0)
 
@@ -334,14 +328,17 @@ cudaError_t launch_cg_step(const KParams& p, const CgParams& c, void* fr, float*
                            cudaStream_t st) {
     const CgArgs q = cg_args(c, fb, fld);
     float* r = static_cast<float*>(fr);
-    const bool links = p.links != nullptr;
-    const auto fields = odd ? (links ? k_cg_fields<true, true> : k_cg_fields<true, false>)
-                            : (links ? k_cg_fields<false, true> : k_cg_fields<false, false>);
-    const auto step = odd ? (links ? k_cg_step<true, true> : k_cg_step<true, false>)
-                          : (links ? k_cg_step<false, true> : k_cg_step<false, false>);
-    const cudaError_t e = launch_pdl(fields, cg_grid(p), CG_BLOCK, 0, st, p, q, r);
+    const int k = (p.flat ? 4 : 0) + (odd ? 2 : 0) + (p.links ? 1 : 0);
+    static constexpr decltype(&k_cg_fields<false, false, false>) fields[8] = {
+        k_cg_fields<false, false, false>, k_cg_fields<false, true, false>, k_cg_fields<true, false, false>, k_cg_fields<true, true, false>,
+        k_cg_fields<false, false, true>,  k_cg_fields<false, true, true>,  k_cg_fields<true, false, true>,  k_cg_fields<true, true, true>};
+    static constexpr decltype(&k_cg_step<false, false, false>) step[8] = {
+        k_cg_step<false, false, false>, k_cg_step<false, true, false>, k_cg_step<true, false, false>, k_cg_step<true, true, false>,
+        k_cg_step<false, false, true>,  k_cg_step<false, true, true>,  k_cg_step<true, false, true>,  k_cg_step<true, true, true>};
+    const dim3 grid = node_grid(p, p.flat != 0);
+    const cudaError_t e = launch_pdl(fields[k], grid, BLOCK_X, 0, st, p, q, r);
     if (e != cudaSuccess) return e;
-    return launch_pdl(step, cg_grid(p), CG_BLOCK, 0, st, p, q, r);
+    return launch_pdl(step[k], grid, BLOCK_X, 0, st, p, q, r);
 }
 
 cudaError_t launch_cg_macro(const KParams& p, const CgParams& c, const void* fr, float* fb, int odd, float* out,
@@ -355,7 +352,7 @@ cudaError_t launch_cg_macro(const KParams& p, const CgParams& c, const void* fr,
 cudaError_t launch_cg_init(const KParams& p, const CgParams& c, void* fr, float* fb, const float* rr, const float* rb,
                            cudaStream_t st) {
     const CgArgs q = cg_args(c, fb, nullptr);
-    k_cg_init<<<cg_grid(p), CG_BLOCK, 0, st>>>(p, q, static_cast<float*>(fr), rr, rb);
+    k_cg_init<<<node_grid(p, false), BLOCK_X, 0, st>>>(p, q, static_cast<float*>(fr), rr, rb);
     return cudaGetLastError();
 }
 

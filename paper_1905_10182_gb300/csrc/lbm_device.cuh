@@ -115,28 +115,74 @@ struct KParams {
     long long local_off;   // z0 * nx * ny: store node index minus caller (local) node index
     int ho;                // 1: second-order Hermite truncation of f^eq and/or F_i (models M4, M5)
     float ce, cf;          // weights of hermite2_correction (1 / 0 and 1/2 / 0)
-    int pf;                // one-node stream-collide: L2 prefetch distance in blocks of the launch (0: off)
-    FastDiv pf_gx, pf_ny;  // its grid's x blocks per row and rows per plane
+    int pf;                // stream-collide: L2 prefetch distance in blocks of the launch (0: off)
+    FastDiv pf_gx, pf_ny;  // division by a row's blocks and by the rows of a plane
+    uint32_t nodes;        // active nodes (nx ny planes), below 2^31
+    FastDiv dnx;           // division by nx
+    int flat;              // node numbering of the kernels with one thread per node, see node_of
 };
+
+// One thread per node.  FLAT = false: a row of blocks for each row of the grid (blockIdx = x block, y, z;
+// y and z stay out of the registers).  FLAT = true: the nodes numbered through rows and planes, so that
+// blocks are full whatever nx is.  set_numbering takes it where rows of blocks leave more than a tenth
+// of their lanes idle: half of them at nx = 64 (two-phase step 174 -> 160 us), 27 % at nx = 93 (a porous
+// channel 93x47x81 18.1 -> 17.0 us).  Otherwise its decoding costs more than it saves: 128^3 with a
+// magnetic field 125.6 -> 127.6 us, Shan-Chen FP16 at nx = 243 4 % slower.  False past the last node.
+__device__ __forceinline__ bool node_at(const KParams& p, uint32_t n, int& x, int& y, int& z) {
+    if (n >= p.nodes) return false;
+    const uint32_t row = p.dnx.div(n), zr = p.pf_ny.div(row);
+    x = (int)(n - row * p.dnx.d);
+    y = (int)(row - zr * p.pf_ny.d);
+    z = (int)zr + p.z0;
+    return true;
+}
+template <bool FLAT>
+__device__ __forceinline__ bool node_of(const KParams& p, int& x, int& y, int& z) {
+    if (FLAT) return node_at(p, blockIdx.x * BLOCK_X + threadIdx.x, x, y, z);
+    x = (int)(blockIdx.x * BLOCK_X + threadIdx.x);
+    y = (int)blockIdx.y;
+    z = (int)blockIdx.z + p.z0;
+    return x < p.nx;
+}
+
+// launch grid of node_of: the ghost planes of a z slab get no threads
+inline dim3 node_grid(const KParams& p, bool flat) {
+    if (flat) return dim3((p.nodes + BLOCK_X - 1) / BLOCK_X);
+    return dim3((p.nx + BLOCK_X - 1) / BLOCK_X, p.ny, p.nz - 2 * p.z0);
+}
+inline void set_numbering(KParams& p) {
+    const int gx = (p.nx + BLOCK_X - 1) / BLOCK_X;
+    p.nodes = (uint32_t)((long long)p.nx * p.ny * (p.nz - 2 * p.z0));
+    p.flat = (long long)gx * BLOCK_X * 9 > (long long)p.nx * 10;
+    p.dnx = make_fastdiv((uint32_t)p.nx);
+    p.pf_ny = make_fastdiv((uint32_t)p.ny);
+    p.pf_gx = make_fastdiv((uint32_t)gx);
+}
 
 // L2 prefetch for K1: the block p.pf places later in launch order will gather 27 row segments of
 // BLOCK_X nodes (on an odd step plane k comes from the row shifted by c_k, the source x - c_i of
 // direction i = opp(k)); one thread per 128-byte line of them issues a prefetch.  This keeps more
 // DRAM requests in flight than the gathers alone, which are latency-bound at 16-20 warps per SM.
-template <typename S, bool ODD>
+template <typename S, bool ODD, bool FLAT>
 __device__ __forceinline__ void k1_prefetch(const KParams& p, const S* f) {
     constexpr uint32_t LPR = BLOCK_X * sizeof(S) / 128;  // lines per row segment
     const uint32_t t = threadIdx.x;
     if (t >= 27 * LPR) return;
-    const uint32_t gx = gridDim.x;
-    const uint32_t b = blockIdx.x + gx * (blockIdx.y + gridDim.y * blockIdx.z) + (uint32_t)p.pf;
-    if (b >= gx * gridDim.y * gridDim.z) return;
-    const uint32_t r = p.pf_gx.div(b);
-    const uint32_t zb = p.pf_ny.div(r);
-    int yk = (int)(r - zb * (uint32_t)p.ny), zk = (int)zb + p.z0;
-    const uint32_t k = t / LPR;
-    const uint32_t xs = (b - r * gx) * BLOCK_X + (t - k * LPR) * (128 / sizeof(S));
-    if (xs >= (uint32_t)p.nx) return;
+    const uint32_t k = t / LPR, dx = (t - k * LPR) * (128 / sizeof(S));
+    int xs, yk, zk;
+    if (FLAT) {  // a segment that runs into the next row is taken to continue in place
+        if (!node_at(p, (blockIdx.x + (uint32_t)p.pf) * BLOCK_X + dx, xs, yk, zk)) return;
+    } else {
+        const uint32_t gx = gridDim.x;
+        const uint32_t b = blockIdx.x + gx * (blockIdx.y + gridDim.y * blockIdx.z) + (uint32_t)p.pf;
+        if (b >= gx * gridDim.y * gridDim.z) return;
+        const uint32_t r = p.pf_gx.div(b);
+        const uint32_t zb = p.pf_ny.div(r);
+        yk = (int)(r - zb * (uint32_t)p.ny);
+        zk = (int)zb + p.z0;
+        xs = (int)((b - r * gx) * BLOCK_X + dx);
+        if (xs >= p.nx) return;
+    }
     if (ODD) {
         constexpr unsigned long long CY = pack_dir(1), CZ = pack_dir(2);
         yk += (int)((CY >> (2 * k)) & 3ull) - 1;

@@ -24,13 +24,12 @@ __device__ __forceinline__ void check_node(const KParams& p, const Macro& m) {
 // K1: one fused AA stream-collide step.  TRACE replaces the collision by the identity, which
 // turns the step into pure streaming with bounce-back (used to check indices bit-exactly).
 // HO: the second-order Hermite truncations (models M4, M5 of Sec. III) instead of the complete ones.
-template <typename S, bool ODD, bool LINKS, int FK, bool TRACE, bool HO>
-__global__ void __launch_bounds__(BLOCK_X, (sizeof(S) == 4 ? 4 : 5)) k_stream_collide(KParams p, S* __restrict__ f) {
+template <typename S, bool ODD, bool LINKS, int FK, bool TRACE, bool HO, bool FLAT>
+__global__ void __launch_bounds__(BLOCK_X, (sizeof(S) == 4 || ODD ? 4 : 5)) k_stream_collide(KParams p, S* __restrict__ f) {
     pdl_wait();
-    const int x = blockIdx.x * BLOCK_X + threadIdx.x;
-    const int y = blockIdx.y, z = blockIdx.z + p.z0;
-    if (p.pf) k1_prefetch<S, ODD>(p, f);
-    if (x >= p.nx) return;
+    if (p.pf) k1_prefetch<S, ODD, FLAT>(p, f);
+    int x, y, z;
+    if (!node_of<FLAT>(p, x, y, z)) return;
     const Nbr nb(x, y, z, p);
     uint32_t link = 0;
     if (LINKS) {
@@ -158,15 +157,9 @@ __global__ void __launch_bounds__(BLOCK_X) k_init_equilibrium(KParams p, S* __re
     for (int i = 0; i < 27; ++i) Codec<S>::st(f + (long long)i * p.N + n, g[i]);
 }
 
-// one block row per active (y, z) line: the ghost planes of a z slab get no threads
-static inline dim3 node_grid(const KParams& p) {
-    return dim3((p.nx + BLOCK_X - 1) / BLOCK_X, p.ny, p.nz - 2 * p.z0);
-}
-
 // ----------------------------------------------------------------------------- launchers
 template <typename S, bool ODD, bool LINKS, bool HO>
 static cudaError_t launch_step_t(const KParams& p, S* f, int fk, bool trace, cudaStream_t st) {
-    const dim3 grid = node_grid(p), block(BLOCK_X);
     if constexpr (sizeof(S) == 2 && !LINKS) {
         // 16-bit storage, fully periodic, even nx, 4-byte aligned store: two nodes per thread
         if (!trace && p.nx % 2 == 0 && (reinterpret_cast<uintptr_t>(f) & 3) == 0) {
@@ -204,17 +197,26 @@ static cudaError_t launch_step_t(const KParams& p, S* f, int fk, bool trace, cud
     if (trace) {
         // free streaming is only offered for FP32 storage (bit-exact index checks)
         if constexpr (std::is_same<S, float>::value && !HO)
-            return launch_pdl(k_stream_collide<S, ODD, LINKS, FK_CONST, true, false>, grid, block, 0, st, p, f);
+            return launch_pdl(k_stream_collide<S, ODD, LINKS, FK_CONST, true, false, false>, node_grid(p, false), BLOCK_X, 0,
+                              st, p, f);
         else
             return cudaErrorInvalidValue;
     }
+    const bool flat = p.flat != 0;
+    const dim3 grid = node_grid(p, flat);
+#define CMLBM_K1(FK)                                                                                        \
+    launch_pdl(flat ? k_stream_collide<S, ODD, LINKS, FK, false, HO, true>                                  \
+                    : k_stream_collide<S, ODD, LINKS, FK, false, HO, false>, grid, BLOCK_X, 0, st, p, f)
     switch (fk) {
-    case FK_CONST: return launch_pdl(k_stream_collide<S, ODD, LINKS, FK_CONST, false, HO>, grid, block, 0, st, p, f);
-    case FK_KOLMOGOROV: return launch_pdl(k_stream_collide<S, ODD, LINKS, FK_KOLMOGOROV, false, HO>, grid, block, 0, st, p, f);
-    case FK_FIELD: return launch_pdl(k_stream_collide<S, ODD, LINKS, FK_FIELD, false, HO>, grid, block, 0, st, p, f);
-    case FK_SHAN_CHEN: return launch_pdl(k_stream_collide<S, ODD, LINKS, FK_SHAN_CHEN, false, HO>, grid, block, 0, st, p, f);
+    case FK_CONST: return CMLBM_K1(FK_CONST);
+    case FK_KOLMOGOROV: return CMLBM_K1(FK_KOLMOGOROV);
+    case FK_FIELD: return CMLBM_K1(FK_FIELD);
+    case FK_SHAN_CHEN:  // fully periodic domains only (lbm_set_force)
+        if constexpr (!LINKS) return CMLBM_K1(FK_SHAN_CHEN);
+        return cudaErrorInvalidValue;
     default: return cudaErrorInvalidValue;
     }
+#undef CMLBM_K1
 }
 
 template <typename S, bool ODD, bool HO>
@@ -227,7 +229,7 @@ cudaError_t launch_step_parity(const KParams& p, void* f, int fk, int trace, cud
 template <typename S>
 cudaError_t launch_psi(const KParams& p, const void* f, float* psi, int odd, cudaStream_t st) {
     const S* fs = static_cast<const S*>(f);
-    const dim3 grid = node_grid(p), block(BLOCK_X);
+    const dim3 grid = node_grid(p, false), block(BLOCK_X);
     const bool links = p.links != nullptr;
     // fully periodic, even nx: two nodes per thread, with the word gathers of the pair kernel
     if (!links && p.nx % 2 == 0 && (reinterpret_cast<uintptr_t>(f) & (2 * sizeof(S) - 1)) == 0)
@@ -239,7 +241,7 @@ cudaError_t launch_psi(const KParams& p, const void* f, float* psi, int odd, cud
 template <typename S, bool ODD, bool LINKS>
 static cudaError_t launch_macro_t(const KParams& p, const S* f, int fk, float* rho, float* ux, float* uy, float* uz,
                                   cudaStream_t st) {
-    const dim3 grid = node_grid(p), block(BLOCK_X);
+    const dim3 grid = node_grid(p, false), block(BLOCK_X);
     switch (fk) {
     case FK_CONST: k_macroscopic<S, ODD, LINKS, FK_CONST><<<grid, block, 0, st>>>(p, f, rho, ux, uy, uz); break;
     case FK_KOLMOGOROV: k_macroscopic<S, ODD, LINKS, FK_KOLMOGOROV><<<grid, block, 0, st>>>(p, f, rho, ux, uy, uz); break;
@@ -264,7 +266,7 @@ cudaError_t launch_macroscopic(const KParams& p, const void* f, int odd, int fk,
 template <typename S>
 cudaError_t launch_get_populations(const KParams& p, const void* f, int odd, float* out, cudaStream_t st) {
     const S* fs = static_cast<const S*>(f);
-    const dim3 grid = node_grid(p), block(BLOCK_X);
+    const dim3 grid = node_grid(p, false), block(BLOCK_X);
     const bool links = p.links != nullptr;
     if (odd) {
         if (links) k_get_populations<S, true, true><<<grid, block, 0, st>>>(p, fs, out);
@@ -278,7 +280,7 @@ cudaError_t launch_get_populations(const KParams& p, const void* f, int odd, flo
 
 template <typename S>
 cudaError_t launch_set_populations(const KParams& p, void* f, const float* in, cudaStream_t st) {
-    k_set_populations<S><<<node_grid(p), BLOCK_X, 0, st>>>(p, static_cast<S*>(f), in);
+    k_set_populations<S><<<node_grid(p, false), BLOCK_X, 0, st>>>(p, static_cast<S*>(f), in);
     return cudaGetLastError();
 }
 
@@ -316,7 +318,7 @@ cudaError_t launch_halo_copy(const KParams& p, void* f, void* buf, int zs, int s
 template <typename S>
 cudaError_t launch_init_equilibrium(const KParams& p, void* f, const float* rho, const float* ux, const float* uy,
                                     const float* uz, cudaStream_t st) {
-    k_init_equilibrium<S><<<node_grid(p), BLOCK_X, 0, st>>>(p, static_cast<S*>(f), rho, ux, uy, uz);
+    k_init_equilibrium<S><<<node_grid(p, false), BLOCK_X, 0, st>>>(p, static_cast<S*>(f), rho, ux, uy, uz);
     return cudaGetLastError();
 }
 

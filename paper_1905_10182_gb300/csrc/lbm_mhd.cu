@@ -22,8 +22,6 @@ namespace cmlbm {
 
 namespace {
 
-constexpr int MHD_BLOCK = 128;
-
 __host__ __device__ constexpr float wm(int l) { return l == 0 ? 0.25f : 0.125f; }
 __host__ __device__ constexpr int opp7(int l) { return l == 0 ? 0 : ((l & 1) ? l + 1 : l - 1); }
 
@@ -135,12 +133,11 @@ struct MhdArgs {
     float bw[3];
 };
 
-template <bool ODD, bool LINKS>
-__global__ void __launch_bounds__(MHD_BLOCK, 5) k_mhd_step(KParams p, MhdArgs q, float* __restrict__ f) {
+template <bool ODD, bool LINKS, bool FLAT>
+__global__ void __launch_bounds__(BLOCK_X, 5) k_mhd_step(KParams p, MhdArgs q, float* __restrict__ f) {
     pdl_wait();
-    const int x = blockIdx.x * MHD_BLOCK + threadIdx.x;
-    const int y = blockIdx.y, z = blockIdx.z + p.z0;
-    if (x >= p.nx) return;
+    int x, y, z;
+    if (!node_of<FLAT>(p, x, y, z)) return;
     const Nbr nb(x, y, z, p);
     const uint32_t link = LINKS ? p.links[nb.self()] : 0u;
     float h[21];
@@ -169,9 +166,9 @@ __global__ void __launch_bounds__(MHD_BLOCK, 5) k_mhd_step(KParams p, MhdArgs q,
 
 // rho, u (with (F_ext + F_L)/2), b, j at the current time; out: 10 planes of N (rho, u, b, j).
 template <bool ODD, bool LINKS>
-__global__ void __launch_bounds__(MHD_BLOCK) k_mhd_fields(KParams p, MhdArgs q, const float* __restrict__ f,
+__global__ void __launch_bounds__(BLOCK_X) k_mhd_fields(KParams p, MhdArgs q, const float* __restrict__ f,
                                                           float* __restrict__ out) {
-    const int x = blockIdx.x * MHD_BLOCK + threadIdx.x;
+    const int x = blockIdx.x * BLOCK_X + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z + p.z0;
     if (x >= p.nx) return;
     const Nbr nb(x, y, z, p);
@@ -193,9 +190,9 @@ __global__ void __launch_bounds__(MHD_BLOCK) k_mhd_fields(KParams p, MhdArgs q, 
 
 // h = h^eq(b, u) with u = (sum f c + F_ext / 2) / rho of the current fluid state (b: 3 planes)
 template <bool ODD>
-__global__ void __launch_bounds__(MHD_BLOCK) k_mhd_init(KParams p, MhdArgs q, const float* __restrict__ f,
+__global__ void __launch_bounds__(BLOCK_X) k_mhd_init(KParams p, MhdArgs q, const float* __restrict__ f,
                                                         const float* __restrict__ b3) {
-    const int x = blockIdx.x * MHD_BLOCK + threadIdx.x;
+    const int x = blockIdx.x * BLOCK_X + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z + p.z0;
     if (x >= p.nx) return;
     const Nbr nb(x, y, z, p);
@@ -223,8 +220,8 @@ __global__ void __launch_bounds__(MHD_BLOCK) k_mhd_init(KParams p, MhdArgs q, co
 
 // natural-order copy of h at the current time (to == 1) or into the store at parity 0 (to == 0)
 template <bool ODD, bool LINKS>
-__global__ void __launch_bounds__(MHD_BLOCK) k_mhd_copy(KParams p, MhdArgs q, float* __restrict__ buf, int to_buf) {
-    const int x = blockIdx.x * MHD_BLOCK + threadIdx.x;
+__global__ void __launch_bounds__(BLOCK_X) k_mhd_copy(KParams p, MhdArgs q, float* __restrict__ buf, int to_buf) {
+    const int x = blockIdx.x * BLOCK_X + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z + p.z0;
     if (x >= p.nx) return;
     const Nbr nb(x, y, z, p);
@@ -242,8 +239,6 @@ __global__ void __launch_bounds__(MHD_BLOCK) k_mhd_copy(KParams p, MhdArgs q, fl
     }
 }
 
-dim3 mhd_grid(const KParams& p) { return dim3((p.nx + MHD_BLOCK - 1) / MHD_BLOCK, p.ny, p.nz - 2 * p.z0); }
-
 MhdArgs args(float* hm, float omega_m, const float bw[3]) {
     MhdArgs q;
     q.hm = hm;
@@ -260,22 +255,25 @@ cudaError_t launch_mhd_step(const KParams& p, void* f, float* hm, float omega_m,
                             cudaStream_t st) {
     const MhdArgs q = args(hm, omega_m, bw);
     float* ff = static_cast<float*>(f);
-    const dim3 grid = mhd_grid(p);
-    if (odd) return launch_pdl(p.links ? k_mhd_step<true, true> : k_mhd_step<true, false>, grid, MHD_BLOCK, 0, st, p, q, ff);
-    return launch_pdl(p.links ? k_mhd_step<false, true> : k_mhd_step<false, false>, grid, MHD_BLOCK, 0, st, p, q, ff);
+    const auto kernel =
+        p.flat ? (odd ? (p.links ? k_mhd_step<true, true, true> : k_mhd_step<true, false, true>)
+                      : (p.links ? k_mhd_step<false, true, true> : k_mhd_step<false, false, true>))
+               : (odd ? (p.links ? k_mhd_step<true, true, false> : k_mhd_step<true, false, false>)
+                      : (p.links ? k_mhd_step<false, true, false> : k_mhd_step<false, false, false>));
+    return launch_pdl(kernel, node_grid(p, p.flat != 0), BLOCK_X, 0, st, p, q, ff);
 }
 
 cudaError_t launch_mhd_fields(const KParams& p, const void* f, float* hm, float omega_m, const float bw[3], int odd,
                               float* out, cudaStream_t st) {
     const MhdArgs q = args(hm, omega_m, bw);
     const float* ff = static_cast<const float*>(f);
-    const dim3 grid = mhd_grid(p);
+    const dim3 grid = node_grid(p, false);
     if (odd) {
-        if (p.links) k_mhd_fields<true, true><<<grid, MHD_BLOCK, 0, st>>>(p, q, ff, out);
-        else k_mhd_fields<true, false><<<grid, MHD_BLOCK, 0, st>>>(p, q, ff, out);
+        if (p.links) k_mhd_fields<true, true><<<grid, BLOCK_X, 0, st>>>(p, q, ff, out);
+        else k_mhd_fields<true, false><<<grid, BLOCK_X, 0, st>>>(p, q, ff, out);
     } else {
-        if (p.links) k_mhd_fields<false, true><<<grid, MHD_BLOCK, 0, st>>>(p, q, ff, out);
-        else k_mhd_fields<false, false><<<grid, MHD_BLOCK, 0, st>>>(p, q, ff, out);
+        if (p.links) k_mhd_fields<false, true><<<grid, BLOCK_X, 0, st>>>(p, q, ff, out);
+        else k_mhd_fields<false, false><<<grid, BLOCK_X, 0, st>>>(p, q, ff, out);
     }
     return cudaGetLastError();
 }
@@ -284,21 +282,21 @@ cudaError_t launch_mhd_init(const KParams& p, const void* f, float* hm, int odd,
     const float zero[3] = {0.0f, 0.0f, 0.0f};
     const MhdArgs q = args(hm, 1.0f, zero);
     const float* ff = static_cast<const float*>(f);
-    if (odd) k_mhd_init<true><<<mhd_grid(p), MHD_BLOCK, 0, st>>>(p, q, ff, b3);
-    else k_mhd_init<false><<<mhd_grid(p), MHD_BLOCK, 0, st>>>(p, q, ff, b3);
+    if (odd) k_mhd_init<true><<<node_grid(p, false), BLOCK_X, 0, st>>>(p, q, ff, b3);
+    else k_mhd_init<false><<<node_grid(p, false), BLOCK_X, 0, st>>>(p, q, ff, b3);
     return cudaGetLastError();
 }
 
 cudaError_t launch_mhd_copy(const KParams& p, float* hm, const float bw[3], int odd, float* buf, int to_buf,
                             cudaStream_t st) {
     const MhdArgs q = args(hm, 1.0f, bw);
-    const dim3 grid = mhd_grid(p);
+    const dim3 grid = node_grid(p, false);
     if (odd) {
-        if (p.links) k_mhd_copy<true, true><<<grid, MHD_BLOCK, 0, st>>>(p, q, buf, to_buf);
-        else k_mhd_copy<true, false><<<grid, MHD_BLOCK, 0, st>>>(p, q, buf, to_buf);
+        if (p.links) k_mhd_copy<true, true><<<grid, BLOCK_X, 0, st>>>(p, q, buf, to_buf);
+        else k_mhd_copy<true, false><<<grid, BLOCK_X, 0, st>>>(p, q, buf, to_buf);
     } else {
-        if (p.links) k_mhd_copy<false, true><<<grid, MHD_BLOCK, 0, st>>>(p, q, buf, to_buf);
-        else k_mhd_copy<false, false><<<grid, MHD_BLOCK, 0, st>>>(p, q, buf, to_buf);
+        if (p.links) k_mhd_copy<false, true><<<grid, BLOCK_X, 0, st>>>(p, q, buf, to_buf);
+        else k_mhd_copy<false, false><<<grid, BLOCK_X, 0, st>>>(p, q, buf, to_buf);
     }
     return cudaGetLastError();
 }
