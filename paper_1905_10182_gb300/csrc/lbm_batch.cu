@@ -10,6 +10,7 @@
 #include <chrono>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -267,6 +268,9 @@ struct lbm_batch {
     unsigned int* h_flag = nullptr;
     double* h_res = nullptr;
     int tile_capacity = 0;
+    int device = 0;
+    float* scratch = nullptr;  // 4 planes of the largest domain, made for the first array that is not in device memory
+    std::mutex scratch_mutex;  // held by the call that uses it
 
     // launch shape (autotuned)
     int threads = 128;
@@ -441,6 +445,16 @@ KParams domain_params(const lbm_batch* b, int k) {
     return p;
 }
 
+// Scratch for fields that are not in device memory, kept for the batch's life: allocated and freed in
+// each call it cost 0.15 ms and a device-wide synchronisation per domain (40 domains set and read: 12 ms).
+lbm_status ensure_scratch(lbm_batch* b) {
+    if (b->scratch) return LBM_OK;
+    uint32_t most = 0;
+    for (const BatchDomain& d : b->dom) most = std::max(most, d.N);
+    BCK(b, cudaMalloc(&b->scratch, sizeof(float) * 4 * most), "cudaMalloc(fields)");
+    return LBM_OK;
+}
+
 // parity of domain k's store: active domains share the batch parity, retired ones are natural
 int domain_parity(const lbm_batch* b, int k) { return b->active[k] ? b->parity : 0; }
 
@@ -489,9 +503,8 @@ lbm_status lbm_batch_create(const lbm_domain* d, int count, double rho0, void* s
     }
     b->nodes = nodes;
     b->tile_capacity = tiles_max;
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaError_t e = cudaGetDevice(&b->device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, b->device);
     if (e != cudaSuccess) return bail(LBM_ERR_CUDA);
     if ((e = cudaMalloc(&b->pool, sizeof(float) * pop)) != cudaSuccess) return bail(LBM_ERR_OOM);
     if ((e = cudaMalloc(&b->links, sizeof(uint32_t) * nodes)) != cudaSuccess) return bail(LBM_ERR_OOM);
@@ -680,38 +693,42 @@ lbm_status lbm_batch_run(lbm_batch* b, double tol, long long max_steps, int chec
 lbm_status lbm_batch_set_state(lbm_batch* b, int k, const float* rho, const float* ux, const float* uy, const float* uz) {
     if (!b || k < 0 || k >= b->ndom || !rho || !ux || !uy || !uz) return LBM_ERR_ARG;
     if (b->active[k] && b->parity) return bfail(b, LBM_ERR_STATE, "set_state needs the batch at even parity");
-    const size_t bytes = sizeof(float) * b->dom[k].N;
-    float* tmp = nullptr;
-    BCK(b, cudaMalloc(&tmp, 4 * bytes), "cudaMalloc(state)");
-    const float* src[4] = {rho, ux, uy, uz};
-    cudaError_t e = cudaSuccess;
-    for (int j = 0; j < 4 && e == cudaSuccess; ++j)
-        e = cudaMemcpyAsync(reinterpret_cast<char*>(tmp) + j * bytes, src[j], bytes, cudaMemcpyDefault, b->stream);
     const long long N = b->dom[k].N;
-    if (e == cudaSuccess)
-        e = launch_init_equilibrium<float>(domain_params(b, k), b->pool + b->dom[k].f_off, tmp, tmp + N, tmp + 2 * N,
-                                           tmp + 3 * N, b->stream);
-    cudaError_t e2 = cudaStreamSynchronize(b->stream);
-    cudaFree(tmp);
-    if (e != cudaSuccess) return bcuda(b, e, "set_state");
-    if (e2 != cudaSuccess) return bcuda(b, e2, "set_state sync");
+    const float* src[4] = {rho, ux, uy, uz};
+    std::lock_guard<std::mutex> lock(b->scratch_mutex);
+    for (int j = 0; j < 4; ++j) {
+        if (in_place(src[j], b->device)) continue;
+        const lbm_status st = ensure_scratch(b);
+        if (st) return st;
+        BCK(b, cudaMemcpyAsync(b->scratch + j * N, src[j], sizeof(float) * N, cudaMemcpyDefault, b->stream), "set_state copy");
+        src[j] = b->scratch + j * N;
+    }
+    BCK(b, launch_init_equilibrium<float>(domain_params(b, k), b->pool + b->dom[k].f_off, src[0], src[1], src[2], src[3], b->stream),
+        "set_state");
+    BCK(b, cudaStreamSynchronize(b->stream), "set_state sync");
     return LBM_OK;
 }
 
 lbm_status lbm_batch_macroscopic(lbm_batch* b, int k, float* rho, float* ux, float* uy, float* uz) {
     if (!b || k < 0 || k >= b->ndom) return LBM_ERR_ARG;
     const long long N = b->dom[k].N;
-    float* tmp = nullptr;
-    BCK(b, cudaMalloc(&tmp, sizeof(float) * 4 * N), "cudaMalloc(macroscopic)");
-    cudaError_t e = launch_macroscopic<float>(domain_params(b, k), b->pool + b->dom[k].f_off, domain_parity(b, k),
-                                              FK_CONST, tmp, tmp + N, tmp + 2 * N, tmp + 3 * N, b->stream);
     float* outs[4] = {rho, ux, uy, uz};
-    for (int j = 0; j < 4 && e == cudaSuccess; ++j)
-        if (outs[j]) e = cudaMemcpyAsync(outs[j], tmp + j * N, sizeof(float) * N, cudaMemcpyDefault, b->stream);
-    cudaError_t e2 = cudaStreamSynchronize(b->stream);
-    cudaFree(tmp);
-    if (e != cudaSuccess) return bcuda(b, e, "macroscopic");
-    if (e2 != cudaSuccess) return bcuda(b, e2, "macroscopic sync");
+    float* dst[4];
+    std::lock_guard<std::mutex> lock(b->scratch_mutex);
+    for (int j = 0; j < 4; ++j) {
+        dst[j] = outs[j];
+        if (outs[j] && in_place(outs[j], b->device)) continue;
+        const lbm_status st = ensure_scratch(b);
+        if (st) return st;
+        dst[j] = b->scratch + j * N;
+    }
+    BCK(b, launch_macroscopic<float>(domain_params(b, k), b->pool + b->dom[k].f_off, domain_parity(b, k), FK_CONST, dst[0], dst[1],
+                                     dst[2], dst[3], b->stream),
+        "macroscopic");
+    for (int j = 0; j < 4; ++j)
+        if (outs[j] && outs[j] != dst[j])
+            BCK(b, cudaMemcpyAsync(outs[j], dst[j], sizeof(float) * N, cudaMemcpyDefault, b->stream), "macroscopic copy");
+    BCK(b, cudaStreamSynchronize(b->stream), "macroscopic sync");
     return LBM_OK;
 }
 
@@ -742,6 +759,7 @@ void lbm_batch_destroy(lbm_batch* b) {
     cudaFree(b->pool);
     cudaFree(b->links);
     cudaFree(b->uprev);
+    cudaFree(b->scratch);
     cudaFree(b->d_dom);
     cudaFree(b->d_tiles);
     cudaFree(b->d_ntiles);

@@ -230,14 +230,17 @@ lbm_status refresh_psi(lbm_ctx* c, const KParams& p) {
     return LBM_OK;
 }
 
-lbm_status run_macro(lbm_ctx* c) {
-    lbm_status st = ensure_macro(c);
+// rho, u (and the models' fields) into the scratch planes of c->macro; out (plain flow only): per field,
+// where to write it instead
+lbm_status run_macro(lbm_ctx* c, float* const* out = nullptr) {
+    lbm_status st = out && out[0] && out[1] && out[2] && out[3] ? LBM_OK : ensure_macro(c);
     if (st) return st;
     KParams p = make_params(c);
     st = refresh_psi(c, p);
     if (st) return st;
     float* m = c->macro;
     const long long NL = c->NL;
+    auto plane = [&](int k) { return out && out[k] ? out[k] : m + k * NL; };
     if (c->hm) {
         CK(c, launch_mhd_fields(p, c->f, c->hm, c->omega_m, c->bw, c->parity, m, c->stream), "magnetic fields kernel");
         return LBM_OK;
@@ -246,7 +249,7 @@ lbm_status run_macro(lbm_ctx* c) {
         CK(c, launch_cg_macro(p, c->cg, c->f, c->cgb, c->parity, m, c->stream), "two-phase fields kernel");
         return LBM_OK;
     }
-    CK(c, DISPATCH(c, launch_macroscopic, p, c->f, c->parity, kernel_force_kind(c), m, m + NL, m + 2 * NL, m + 3 * NL,
+    CK(c, DISPATCH(c, launch_macroscopic, p, c->f, c->parity, kernel_force_kind(c), plane(0), plane(1), plane(2), plane(3),
                    c->stream),
        "macroscopic kernel");
     return LBM_OK;
@@ -633,17 +636,18 @@ lbm_status lbm_set_state(lbm_ctx* c, const float* rho, const float* ux, const fl
     if (c && c->cgb) return fail(c, LBM_ERR_UNSUPPORTED, "two-phase model: lbm_set_colour_gradient sets the two-phase state");
     if (!c) return LBM_ERR_ARG;
     if (!rho || !ux || !uy || !uz) return fail(c, LBM_ERR_ARG, "rho, ux, uy, uz are required");
-    lbm_status st = ensure_macro(c);
-    if (st) return st;
+    // device arrays are read where they lie (copied first, they cost 32 B per node more: 512^3 0.65 ms)
     const long long NL = c->NL;
-    const size_t b = sizeof(float) * NL;
-    float* m = c->macro;
-    CK(c, copy_in(m, rho, b, c->stream), "state copy");
-    CK(c, copy_in(m + NL, ux, b, c->stream), "state copy");
-    CK(c, copy_in(m + 2 * NL, uy, b, c->stream), "state copy");
-    CK(c, copy_in(m + 3 * NL, uz, b, c->stream), "state copy");
+    const float* src[4] = {rho, ux, uy, uz};
+    for (int k = 0; k < 4; ++k) {
+        if (in_place(src[k], c->device)) continue;
+        lbm_status st = ensure_macro(c);
+        if (st) return st;
+        CK(c, copy_in(c->macro + k * NL, src[k], sizeof(float) * NL, c->stream), "state copy");
+        src[k] = c->macro + k * NL;
+    }
     KParams p = make_params(c);
-    CK(c, DISPATCH(c, launch_init_equilibrium, p, c->f, m, m + NL, m + 2 * NL, m + 3 * NL, c->stream), "init kernel");
+    CK(c, DISPATCH(c, launch_init_equilibrium, p, c->f, src[0], src[1], src[2], src[3], c->stream), "init kernel");
     CK(c, cudaStreamSynchronize(c->stream), "init sync");
     c->parity = 0;
     c->t = 0;
@@ -715,11 +719,15 @@ lbm_status lbm_stream_only(lbm_ctx* c, int nsteps) {
 
 lbm_status lbm_macroscopic(lbm_ctx* c, float* rho, float* ux, float* uy, float* uz) {
     if (!c) return LBM_ERR_ARG;
-    lbm_status st = run_macro(c);
-    if (st) return st;
     float* outs[4] = {rho, ux, uy, uz};
+    float* there[4] = {};
+    if (!c->hm && !c->cgb)
+        for (int k = 0; k < 4; ++k)
+            if (outs[k] && in_place(outs[k], c->device)) there[k] = outs[k];
+    lbm_status st = run_macro(c, there);
+    if (st) return st;
     for (int k = 0; k < 4; ++k)
-        if (outs[k]) CK(c, copy_out(outs[k], c->macro + k * c->NL, sizeof(float) * c->NL, c->stream), "macroscopic copy");
+        if (outs[k] && !there[k]) CK(c, copy_out(outs[k], c->macro + k * c->NL, sizeof(float) * c->NL, c->stream), "macroscopic copy");
     return sync_and_check(c);
 }
 

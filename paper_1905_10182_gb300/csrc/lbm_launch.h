@@ -30,6 +30,17 @@ inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_
     return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
 }
 
+// A caller's array that the kernels may read or write where it lies: device memory of device `dev` (host,
+// managed and other devices' memory goes through a copy).
+inline bool in_place(const void* p, int dev) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == dev;
+}
+
 template <typename S, bool ODD, bool HO>
 cudaError_t launch_step_parity(const KParams& p, void* f, int fk, int trace, cudaStream_t st);
 // ho: the second-order Hermite truncation variants (instantiated in lbm_k_*_ho_*.cu)
