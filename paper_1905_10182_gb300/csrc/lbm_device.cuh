@@ -13,6 +13,7 @@
 #include <stdint.h>
 
 #include "lbm_vec.cuh"
+#include "pdl.cuh"
 
 namespace cmlbm {
 
@@ -47,10 +48,6 @@ __host__ __device__ constexpr unsigned long long pack_dir(int axis) {
     for (int i = 0; i < 27; ++i) c |= (unsigned long long)((axis == 1 ? dir_y(i) : dir_z(i)) + 1) << (2 * i);
     return c;
 }
-
-// Waits until the kernel before this one in its stream has completed and its writes are visible
-// (returns at once in a kernel launched without programmatic serialisation, see launch_pdl).
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 constexpr uint32_t SOLID_BIT = 1u << 31;  // in a link word: the node itself is solid
 constexpr int BLOCK_X = 128;              // one-node kernels: threads per block, one node each along x

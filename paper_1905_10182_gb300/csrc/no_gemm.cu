@@ -29,6 +29,7 @@
 
 #include "../../include/cmlbm.h"
 #include "no_gemm.h"
+#include "pdl.cuh"
 
 namespace cmlbm {
 namespace {
@@ -221,6 +222,7 @@ __device__ __forceinline__ void stage_tile(uint8_t* dst, const __nv_bfloat16* __
 
 template <int TN>
 __global__ void __launch_bounds__(THREADS) k_gemm_bf16_tc(GemmArgs g) {
+    pdl_wait();
     constexpr int A_BYTES = TM * TK * 2, STAGE_BYTES = A_BYTES + TN * TK * 2;
     constexpr uint32_t TMEM_COLS = TN <= 32 ? 32 : 64;  // FP32 accumulator: 128 lanes x TN columns
     extern __shared__ __align__(1024) uint8_t smem[];    // two stages of [A | B]
@@ -634,6 +636,9 @@ __global__ void __launch_bounds__(Shape<GROUPS>::threads, Shape<GROUPS>::blocks_
         asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(&map_a)) : "memory");
         asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(&map_b)) : "memory");
     }
+    // the set-up above overlaps the kernel before this one; its results are read, and its inputs may be
+    // overwritten, from here on
+    pdl_wait();
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
@@ -905,7 +910,7 @@ cudaError_t launch_tn(const GemmArgs& g, int batch, cudaStream_t st) {
     }
     const dim3 grid((g.N + TN - 1) / TN, (g.M + TM - 1) / TM, batch);
     if (grid.y > 65535 || grid.z > 65535) return cudaErrorInvalidValue;
-    k_gemm_bf16_tc<TN><<<grid, THREADS, smem, st>>>(g);
+    launch_pdl(k_gemm_bf16_tc<TN>, grid, THREADS, smem, st, g);
     return cudaGetLastError();
 }
 
@@ -1038,7 +1043,7 @@ cudaError_t launch_tma_tn(const CUtensorMap& ma, const CUtensorMap& mb, const CU
     static const int sms = sm_count();
     const long long slots = (long long)sms * Sh::blocks_per_sm;
     const long long grid = a.tiles < slots ? a.tiles : slots;
-    tma::k_gemm_bf16_tma<TN, GROUPS><<<(unsigned)grid, Sh::threads, tma::smem_bytes<GROUPS>(), st>>>(ma, mb, mc, a);
+    launch_pdl(tma::k_gemm_bf16_tma<TN, GROUPS>, (unsigned)grid, Sh::threads, tma::smem_bytes<GROUPS>(), st, ma, mb, mc, a);
     return cudaGetLastError();
 }
 
@@ -1133,6 +1138,7 @@ namespace {
 
 // K = 0: the product is an empty sum, so C = 0 without beta (and C is left as it is with beta).
 __global__ void k_gemm_zero_c(GemmArgs g, int batch) {
+    pdl_wait();
     const long long total = (long long)batch * g.M * g.N;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
         const long long b = i / ((long long)g.M * g.N), r = i - b * g.M * g.N;
@@ -1153,7 +1159,7 @@ cudaError_t launch_gemm_bf16(const GemmArgs& g_in, int batch, cudaStream_t st) {
         if (g_in.beta) return cudaSuccess;
         const long long total = (long long)batch * g_in.M * g_in.N;
         const long long blocks = std::min<long long>((total + 255) / 256, 4096);
-        k_gemm_zero_c<<<(unsigned)blocks, 256, 0, st>>>(g_in, batch);
+        launch_pdl(k_gemm_zero_c, (unsigned)blocks, 256, 0, st, g_in, batch);
         return cudaGetLastError();
     }
     GemmArgs g = g_in;

@@ -19,6 +19,7 @@
 
 #include "../../include/cmlbm.h"
 #include "no_gemm.h"
+#include "pdl.cuh"
 
 using namespace cmlbm;
 
@@ -28,6 +29,7 @@ typedef __nv_bfloat16 bf16;
 
 // ------------------------------------------------------------------------------ elementwise kernels
 __global__ void k_f32_to_bf16(const float* __restrict__ x, bf16* __restrict__ y, long long n) {
+    pdl_wait();
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         y[i] = __float2bfloat16(x[i]);
 }
@@ -35,6 +37,7 @@ __global__ void k_f32_to_bf16(const float* __restrict__ x, bf16* __restrict__ y,
 // out[b][c][s] = sum_i P[c][i] a[b][i][s] + p[c]  (FP32 and BF16 copies)
 __global__ void k_lift(const float* __restrict__ a, const float* __restrict__ P, const float* __restrict__ p, int B, int Ci,
                        int W, long long S, float* __restrict__ h, bf16* __restrict__ hb) {
+    pdl_wait();
     const long long total = (long long)B * W * S;
     for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
          idx += (long long)gridDim.x * blockDim.x) {
@@ -51,6 +54,7 @@ __global__ void k_lift(const float* __restrict__ a, const float* __restrict__ P,
 // out[b][o][s] = sum_c Q[o][c] h[b][c][s] + q[o]
 __global__ void k_project(const float* __restrict__ h, const float* __restrict__ Q, const float* __restrict__ q, int B, int W,
                           int Co, long long S, float* __restrict__ out) {
+    pdl_wait();
     const long long total = (long long)B * Co * S;
     for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
          idx += (long long)gridDim.x * blockDim.x) {
@@ -66,6 +70,7 @@ __global__ void k_project(const float* __restrict__ h, const float* __restrict__
 // dh[b][c][s] = sum_o Q[o][c] dout[b][o][s]
 __global__ void k_project_bwd_x(const float* __restrict__ dout, const float* __restrict__ Q, int B, int W, int Co, long long S,
                                 float* __restrict__ dh) {
+    pdl_wait();
     const long long total = (long long)B * W * S;
     for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
          idx += (long long)gridDim.x * blockDim.x) {
@@ -88,6 +93,7 @@ __device__ __forceinline__ float gelu_grad(float x) {
 // z[b][o][s] += bias[o]; h = act(z) (BF16 copy for the next GEMMs)
 __global__ void k_bias_act(float* __restrict__ z, const float* __restrict__ bias, int W, long long S, long long total,
                            int use_gelu, bf16* __restrict__ hb) {
+    pdl_wait();
     for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
          idx += (long long)gridDim.x * blockDim.x) {
         const int o = (int)((idx / S) % W);
@@ -100,6 +106,7 @@ __global__ void k_bias_act(float* __restrict__ z, const float* __restrict__ bias
 // dz = dh * act'(z); BF16 copy for the GEMMs
 __global__ void k_act_bwd(const float* __restrict__ dh, const float* __restrict__ z, long long total, int use_gelu,
                           float* __restrict__ dz, bf16* __restrict__ dzb) {
+    pdl_wait();
     for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
          idx += (long long)gridDim.x * blockDim.x) {
         const float v = use_gelu ? dh[idx] * gelu_grad(z[idx]) : dh[idx];
@@ -124,6 +131,7 @@ constexpr int CENTER_PARTS = 16;
 
 __global__ void __launch_bounds__(256) k_center_partials(const float* __restrict__ src, long long S, int use_gelu,
                                                          double* __restrict__ part) {
+    pdl_wait();
     const int bc = blockIdx.x / CENTER_PARTS, p = blockIdx.x % CENTER_PARTS;
     const long long per = (S + CENTER_PARTS - 1) / CENTER_PARTS;
     const long long lo = p * per, hi = lo + per < S ? lo + per : S;
@@ -147,6 +155,7 @@ __global__ void __launch_bounds__(256) k_center_partials(const float* __restrict
 // a row covers the float4 groups [p per4, (p + 1) per4).
 __global__ void __launch_bounds__(256) k_center_partials_v(const float* __restrict__ src, long long S, int use_gelu,
                                                            double* __restrict__ part) {
+    pdl_wait();
     const int bc = blockIdx.x / CENTER_PARTS, p = blockIdx.x % CENTER_PARTS;
     const long long S4 = S / 4, per = (S4 + CENTER_PARTS - 1) / CENTER_PARTS;
     const long long lo = p * per, hi = lo + per < S4 ? lo + per : S4;
@@ -180,6 +189,7 @@ __global__ void __launch_bounds__(256) k_center_partials_v(const float* __restri
 // one warp per channel: mean[bc] = (sum of its parts) / S, the parts split over the lanes and the
 // lanes' sums combined by a shuffle tree (FP64)
 __global__ void k_center_means(const double* __restrict__ part, int channels, int parts, long long S, float* __restrict__ mean) {
+    pdl_wait();
     const int bc = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (bc >= channels) return;
     double t = 0.0;
@@ -192,6 +202,7 @@ __global__ void k_center_means(const double* __restrict__ part, int channels, in
 // db[o] += sum over samples and parts of the per-row partial sums part[(b W + o) parts + p]; one
 // warp per o
 __global__ void k_rows_to_bias(const double* __restrict__ part, int B, int W, int parts, float* __restrict__ db) {
+    pdl_wait();
     const int o = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (o >= W) return;
     double t = 0.0;
@@ -220,6 +231,7 @@ __device__ __forceinline__ void block_sum_to(float v, double* out) {
 // grid (chunks, channels): each block strides over its channel's S values
 __global__ void k_center_apply(const float* __restrict__ src, long long S, int use_gelu, const float* __restrict__ mean,
                                bf16* __restrict__ out) {
+    pdl_wait();
     const long long base = (long long)blockIdx.y * S;
     const float m = mean[blockIdx.y];
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < S; i += (long long)gridDim.x * blockDim.x) {
@@ -230,6 +242,7 @@ __global__ void k_center_apply(const float* __restrict__ src, long long S, int u
 
 __global__ void __launch_bounds__(256) k_center_apply_v(const float* __restrict__ src, long long S, int use_gelu,
                                                         const float* __restrict__ mean, bf16* __restrict__ out) {
+    pdl_wait();
     const long long base = (long long)blockIdx.y * S;
     const float m = mean[blockIdx.y];
     const float4* x = reinterpret_cast<const float4*>(src + base);
@@ -246,6 +259,7 @@ __global__ void __launch_bounds__(256) k_center_apply_v(const float* __restrict_
 // [b][c][kx][ky][ri][kz]: += scale * mean[b * W + c].
 __global__ void k_add_dc(float* __restrict__ modes, const float* __restrict__ mean, int rows, long long stride,
                          float scale) {
+    pdl_wait();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < rows) modes[(long long)k * stride] += scale * mean[k];
 }
@@ -256,6 +270,7 @@ struct Perm6 {
     int perm[6];
 };
 __global__ void k_permute6(const bf16* __restrict__ in, bf16* __restrict__ out, Perm6 P, long long total) {
+    pdl_wait();
     long long sin[6];
     sin[5] = 1;
     for (int a = 4; a >= 0; --a) sin[a] = sin[a + 1] * P.din[a + 1];
@@ -278,6 +293,7 @@ __global__ void k_permute6(const bf16* __restrict__ in, bf16* __restrict__ out, 
 // vectors; needs D and 2 MY multiples of 8 and 16-byte aligned buffers.
 __global__ void __launch_bounds__(256) k_to_zlast(const bf16* __restrict__ in, bf16* __restrict__ out, int D, int MX,
                                                   int MY) {
+    pdl_wait();
     extern __shared__ bf16 sm[];  // [z][ri * MY + ky]
     const int L = 2 * MY, R = L + 2;
     const long long bc = blockIdx.x / MX;
@@ -306,6 +322,7 @@ __global__ void __launch_bounds__(256) k_to_zlast(const bf16* __restrict__ in, b
 
 __global__ void __launch_bounds__(256) k_from_zlast(const bf16* __restrict__ in, bf16* __restrict__ out, int D, int MX,
                                                     int MY) {
+    pdl_wait();
     extern __shared__ bf16 sm[];  // [ky 2 + ri][z]
     const int L = 2 * MY, R = D + 2;
     const long long bc = blockIdx.x / MX;
@@ -360,6 +377,7 @@ __device__ __forceinline__ void mode_of(const MixDims& d, long long m, int& kx, 
 // Y[b][o] = sum_c W[o][c] X[b][c] (complex), Y in BF16 for the inverse transforms
 __global__ void __launch_bounds__(256) k_mix_fwd(const float* __restrict__ X, const float* __restrict__ Wm, MixDims d,
                                                  bf16* __restrict__ Y) {
+    pdl_wait();
     const long long m = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (m >= (long long)d.MX * d.MY * d.MZ) return;
     int kx, ky, kz;
@@ -393,6 +411,7 @@ __global__ void __launch_bounds__(256) k_mix_fwd(const float* __restrict__ X, co
 // dX[b][c] = sum_o conj(W[o][c]) dY[b][o] (BF16 out); lanes over c read W[o][c] coalesced
 __global__ void __launch_bounds__(256) k_mix_bwd_x(const float* __restrict__ dY, const float* __restrict__ Wm,
                                                    MixDims d, bf16* __restrict__ dX) {
+    pdl_wait();
     const long long m = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (m >= (long long)d.MX * d.MY * d.MZ) return;
     int kx, ky, kz;
@@ -426,6 +445,7 @@ __global__ void __launch_bounds__(256) k_mix_bwd_x(const float* __restrict__ dY,
 // dW[o][c] += sum_b dY[b][o] conj(X[b][c]); lanes over c write dW coalesced
 __global__ void __launch_bounds__(256) k_mix_bwd_w(const float* __restrict__ dY, const float* __restrict__ X, MixDims d,
                                                    float* __restrict__ dW) {
+    pdl_wait();
     const long long m = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (m >= (long long)d.MX * d.MY * d.MZ) return;
     int kx, ky, kz;
@@ -518,6 +538,7 @@ __device__ __forceinline__ void wait_mode_matrix() {
 
 __global__ void __launch_bounds__(256) k_mix_fwd32(const float* __restrict__ X, const float* __restrict__ Wm, MixDims d,
                                                    bf16* __restrict__ Y) {
+    pdl_wait();
     extern __shared__ __align__(16) float smat[];  // MIX_MODES matrices, MIX_W rows of MIX_PITCH
     __shared__ __align__(16) float sbuf[MIX_MODES][MIX_BUF];
     __shared__ __align__(16) bf16 so[MIX_S * MIX_W * 2][MIX_MODES];
@@ -562,6 +583,7 @@ __global__ void __launch_bounds__(256) k_mix_fwd32(const float* __restrict__ X, 
 
 __global__ void __launch_bounds__(256) k_mix_bwd_x32(const float* __restrict__ dY, const float* __restrict__ Wm,
                                                      MixDims d, bf16* __restrict__ dX) {
+    pdl_wait();
     extern __shared__ __align__(16) float smat[];  // MIX_MODES matrices, MIX_W rows of MIX_PITCH
     __shared__ __align__(16) float sbuf[MIX_MODES][MIX_BUF];
     __shared__ __align__(16) bf16 so[MIX_S * MIX_W * 2][MIX_MODES];
@@ -608,6 +630,7 @@ __global__ void __launch_bounds__(256) k_mix_bwd_x32(const float* __restrict__ d
 // `add`: accumulate onto dW, else overwrite.
 __global__ void __launch_bounds__(256) k_mix_bwd_w32(const float* __restrict__ dY, const float* __restrict__ X, MixDims d,
                                                      float* __restrict__ dW, int add) {
+    pdl_wait();
     __shared__ __align__(16) float sy[MIX_MODES][MIX_BUF];
     __shared__ __align__(16) float sx[MIX_MODES][MIX_BUF];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -659,6 +682,7 @@ __global__ void __launch_bounds__(256) k_mix_bwd_w32(const float* __restrict__ d
 // fixed order afterwards (k_sum_partials), so gradients are reproducible run to run.
 __global__ void k_reduce_bs(const float* __restrict__ X, const float* __restrict__ Y, int B, int Cx, int Cy, long long S,
                             int chunks, float* __restrict__ part) {
+    pdl_wait();
     const int pairs = Cx * Cy;
     const int pair = blockIdx.x / chunks, chunk = blockIdx.x % chunks;
     const int i = pair / Cy, j = pair % Cy;
@@ -689,6 +713,7 @@ __global__ void k_reduce_bs(const float* __restrict__ X, const float* __restrict
 // out[k] += sum_p part[p][k]: a block takes 32 consecutive k (lanes) and splits the partials among
 // its 16 warps (warp w: p = w, w + 16, ...); the warps' sums are then added in warp order.
 __global__ void __launch_bounds__(512) k_sum_partials(const float* __restrict__ part, int P, int K, float* __restrict__ out) {
+    pdl_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int k = blockIdx.x * 32 + lane;
     float a = 0.0f;
@@ -709,6 +734,7 @@ __global__ void __launch_bounds__(512) k_sum_partials(const float* __restrict__ 
 // mean squared error over all elements; dout = 2 (out - t) / n; loss accumulated in FP64
 __global__ void k_mse(const float* __restrict__ out, const float* __restrict__ t, long long n, float* __restrict__ dout,
                       double* __restrict__ loss) {
+    pdl_wait();
     double acc = 0.0;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const float e = out[i] - t[i];
@@ -736,6 +762,7 @@ __device__ __forceinline__ void adam1(float& p, float g, float& m, float& v, flo
 __global__ void __launch_bounds__(256) k_adam_v(float4* __restrict__ p, const float4* __restrict__ g, float4* __restrict__ m,
                                                 float4* __restrict__ v, long long n4, const float* __restrict__ sc, float b1,
                                                 float b2, float eps) {
+    pdl_wait();
     const float lr = sc[0], c1 = sc[1], c2 = sc[2];
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (long long)gridDim.x * blockDim.x) {
         const float4 gi = g[i];
@@ -751,6 +778,7 @@ __global__ void __launch_bounds__(256) k_adam_v(float4* __restrict__ p, const fl
 }
 
 __global__ void k_set_adam_scalars(float* __restrict__ sc, float lr, float c1, float c2) {
+    pdl_wait();
     sc[0] = lr;
     sc[1] = c1;
     sc[2] = c2;
@@ -758,6 +786,7 @@ __global__ void k_set_adam_scalars(float* __restrict__ sc, float lr, float c1, f
 
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v, long long n,
                        const float* __restrict__ sc, float b1, float b2, float eps) {
+    pdl_wait();
     const float lr = sc[0], c1 = sc[1], c2 = sc[2];
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const float gi = g[i];
@@ -791,6 +820,7 @@ inline int row_blocks(long long S) { return (int)((S / 4 + 256 * ROW_PER - 1) / 
 // the next layer's centring sums.
 __global__ void __launch_bounds__(256) k_bias_act_v(float* __restrict__ z, const float* __restrict__ bias, int W, long long S,
                                                     int use_gelu, bf16* __restrict__ hb, double* __restrict__ part) {
+    pdl_wait();
     const long long row = blockIdx.y, S4 = S / 4;
     const float bo = bias[row % W];
     float4* zr = reinterpret_cast<float4*>(z + row * S);
@@ -819,6 +849,7 @@ __global__ void __launch_bounds__(256) k_bias_act_v(float* __restrict__ z, const
 __global__ void __launch_bounds__(256) k_act_bwd_v(const float* __restrict__ dh, const float* __restrict__ z, long long S,
                                                    int use_gelu, float* __restrict__ dz, bf16* __restrict__ dzb,
                                                    double* __restrict__ part) {
+    pdl_wait();
     const long long row = blockIdx.y, S4 = S / 4;
     float sum = 0.0f;
 #pragma unroll
@@ -842,6 +873,7 @@ __global__ void __launch_bounds__(256) k_act_bwd_v(const float* __restrict__ dh,
 // h[b][c][s] = p[c] + sum_i P[c][i] a[b][i][s] (Ci <= VEC_CH), h also as BF16; grid (positions / 1024, B)
 __global__ void __launch_bounds__(256) k_lift_v(const float* __restrict__ a, const float* __restrict__ P, const float* __restrict__ p,
                                                 int Ci, int W, long long S, float* __restrict__ h, bf16* __restrict__ hb) {
+    pdl_wait();
     const long long s4 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (s4 * 4 >= S) return;
     const long long b = blockIdx.y;
@@ -869,6 +901,7 @@ __global__ void __launch_bounds__(256) k_lift_v(const float* __restrict__ a, con
 // out[b][k][s] = q[k] + sum_c Q[k][c] h[b][c][s] (Co <= VEC_CH); grid (positions / 1024, B)
 __global__ void __launch_bounds__(256) k_project_v(const float* __restrict__ h, const float* __restrict__ Q, const float* __restrict__ q,
                                                    int W, int Co, long long S, float* __restrict__ out) {
+    pdl_wait();
     const long long s4 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (s4 * 4 >= S) return;
     const long long b = blockIdx.y;
@@ -896,6 +929,7 @@ __global__ void __launch_bounds__(256) k_project_v(const float* __restrict__ h, 
 // dh[b][c][s] = sum_k Q[k][c] dout[b][k][s] (Co <= VEC_CH); grid (positions / 1024, B)
 __global__ void __launch_bounds__(256) k_project_bwd_x_v(const float* __restrict__ dout, const float* __restrict__ Q, int W, int Co,
                                                          long long S, float* __restrict__ dh) {
+    pdl_wait();
     const long long s4 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (s4 * 4 >= S) return;
     const long long b = blockIdx.y;
@@ -1038,9 +1072,9 @@ cudaError_t permute(lbm_no* n, const bf16* in, bf16* out, const long long din[6]
     if (vec && din[0] * din[1] * MX == bcx && perm[0] == 0 && perm[1] == 1 && (to_z || from_z) && bcx < (1LL << 31) &&
         smem <= 48 * 1024) {
         if (to_z)
-            k_to_zlast<<<(unsigned)bcx, 256, smem, n->stream>>>(in, out, D, MX, MY);
+            launch_pdl(k_to_zlast, (unsigned)bcx, 256, smem, n->stream, in, out, D, MX, MY);
         else
-            k_from_zlast<<<(unsigned)bcx, 256, smem, n->stream>>>(in, out, D, MX, MY);
+            launch_pdl(k_from_zlast, (unsigned)bcx, 256, smem, n->stream, in, out, D, MX, MY);
         return cudaGetLastError();
     }
     Perm6 P;
@@ -1050,7 +1084,7 @@ cudaError_t permute(lbm_no* n, const bf16* in, bf16* out, const long long din[6]
         P.perm[a] = perm[a];
         total *= din[a];
     }
-    k_permute6<<<grid_for(total), 256, 0, n->stream>>>(in, out, P, total);
+    launch_pdl(k_permute6, grid_for(total), 256, 0, n->stream, in, out, P, total);
     return cudaGetLastError();
 }
 
@@ -1065,15 +1099,15 @@ cudaError_t center(lbm_no* n, const float* src, int use_gelu, int parts = 0) {
     if (parts <= 0) {
         parts = CENTER_PARTS;
         if (v4)
-            k_center_partials_v<<<ch * CENTER_PARTS, 256, 0, n->stream>>>(src, n->S, use_gelu, n->cpart);
+            launch_pdl(k_center_partials_v, ch * CENTER_PARTS, 256, 0, n->stream, src, n->S, use_gelu, n->cpart);
         else
-            k_center_partials<<<ch * CENTER_PARTS, 256, 0, n->stream>>>(src, n->S, use_gelu, n->cpart);
+            launch_pdl(k_center_partials, ch * CENTER_PARTS, 256, 0, n->stream, src, n->S, use_gelu, n->cpart);
     }
-    k_center_means<<<(ch + 3) / 4, 128, 0, n->stream>>>(n->cpart, ch, parts, n->S, n->hmean);
+    launch_pdl(k_center_means, (ch + 3) / 4, 128, 0, n->stream, n->cpart, ch, parts, n->S, n->hmean);
     if (v4)
-        k_center_apply_v<<<dim3(32, ch), 256, 0, n->stream>>>(src, n->S, use_gelu, n->hmean, n->hs);
+        launch_pdl(k_center_apply_v, dim3(32, ch), 256, 0, n->stream, src, n->S, use_gelu, n->hmean, n->hs);
     else
-        k_center_apply<<<dim3(32, ch), 256, 0, n->stream>>>(src, n->S, use_gelu, n->hmean, n->hs);
+        launch_pdl(k_center_apply, dim3(32, ch), 256, 0, n->stream, src, n->S, use_gelu, n->hmean, n->hs);
     return cudaGetLastError();
 }
 
@@ -1087,6 +1121,7 @@ constexpr int RED_SMALL = 8;
 __global__ void __launch_bounds__(256) k_reduce_pairs(const float* __restrict__ big, const float* __restrict__ small, int Cb,
                                                       int Cs, int B, long long S, int chunks, int big_is_x, int Cy,
                                                       float* __restrict__ part) {
+    pdl_wait();
     const int chunk = blockIdx.x, r = blockIdx.y;
     const long long S4 = S / 4, n4 = (long long)B * S4;
     const long long per = (n4 + chunks - 1) / chunks;
@@ -1155,6 +1190,7 @@ constexpr int PAIR_CHUNKS = 256;
 template <int CS>
 __global__ void __launch_bounds__(256) k_reduce_pairs32(const float* __restrict__ big, const float* __restrict__ small, int B,
                                                         long long S, int big_is_x, int Cy, float* __restrict__ part) {
+    pdl_wait();
     constexpr int CB = 32, NA = CB * CS;  // accumulators per thread, index c CS + k
     const long long S4 = S / 4, n4 = (long long)B * S4;
     const long long per = (n4 + gridDim.x - 1) / gridDim.x;
@@ -1216,9 +1252,9 @@ cudaError_t reduce_bs(lbm_no* n, const float* X, const float* Y, int Cx, int Cy,
     if (Y && n->S % 4 == 0 && ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Y)) & 15u) == 0 &&
         ((Cx == 32 && Cy == 4) || (Cx == 4 && Cy == 32))) {
         const bool x_big = Cx == 32;
-        k_reduce_pairs32<4><<<PAIR_CHUNKS, 256, 0, n->stream>>>(x_big ? X : Y, x_big ? Y : X, n->B, n->S, x_big ? 1 : 0, Cy,
+        launch_pdl(k_reduce_pairs32<4>, PAIR_CHUNKS, 256, 0, n->stream, x_big ? X : Y, x_big ? Y : X, n->B, n->S, x_big ? 1 : 0, Cy,
                                                                  n->red);
-        k_sum_partials<<<(pairs + 31) / 32, 512, 0, n->stream>>>(n->red, PAIR_CHUNKS, pairs, out);
+        launch_pdl(k_sum_partials, (pairs + 31) / 32, 512, 0, n->stream, n->red, PAIR_CHUNKS, pairs, out);
         return cudaGetLastError();
     }
     const bool al = ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Y)) & 15u) == 0;
@@ -1227,13 +1263,13 @@ cudaError_t reduce_bs(lbm_no* n, const float* X, const float* Y, int Cx, int Cy,
         const float* big = x_big ? X : Y;
         const float* small = x_big ? Y : X;
         const int Cb = x_big ? Cx : Cy, Cs = Y == nullptr ? 1 : (x_big ? Cy : Cx);
-        k_reduce_pairs<<<dim3(REDUCE_CHUNKS, Cb), 256, 0, n->stream>>>(big, small, Cb, Cs, n->B, n->S, REDUCE_CHUNKS,
+        launch_pdl(k_reduce_pairs, dim3(REDUCE_CHUNKS, Cb), 256, 0, n->stream, big, small, Cb, Cs, n->B, n->S, REDUCE_CHUNKS,
                                                                         x_big ? 1 : 0, Cy, n->red);
-        k_sum_partials<<<(pairs + 31) / 32, 512, 0, n->stream>>>(n->red, REDUCE_CHUNKS, pairs, out);
+        launch_pdl(k_sum_partials, (pairs + 31) / 32, 512, 0, n->stream, n->red, REDUCE_CHUNKS, pairs, out);
         return cudaGetLastError();
     }
-    k_reduce_bs<<<pairs * REDUCE_CHUNKS, 256, 0, n->stream>>>(X, Y, n->B, Cx, Cy, n->S, REDUCE_CHUNKS, n->red);
-    k_sum_partials<<<(pairs + 31) / 32, 512, 0, n->stream>>>(n->red, REDUCE_CHUNKS, pairs, out);
+    launch_pdl(k_reduce_bs, pairs * REDUCE_CHUNKS, 256, 0, n->stream, X, Y, n->B, Cx, Cy, n->S, REDUCE_CHUNKS, n->red);
+    launch_pdl(k_sum_partials, (pairs + 31) / 32, 512, 0, n->stream, n->red, REDUCE_CHUNKS, pairs, out);
     return cudaGetLastError();
 }
 
@@ -1341,15 +1377,15 @@ lbm_status spectral_fwd(lbm_no* n, int l, const float* src, int use_gelu, float*
     const long long R = (long long)B * W * MX * MY;
     NCK(n, gemm(n, (int)R, 2 * MZ, 2 * D, 1, n->t2p, 2 * D, 1, 0, n->GZ, 2 * MZ, 1, 0, n->Xh[l], 2 * MZ, 1, 0, 0, 0), "fz");
     // the mean's mode: sum over the grid = S * mean
-    k_add_dc<<<(B * W + 127) / 128, 128, 0, n->stream>>>(n->Xh[l], n->hmean, B * W, (long long)MX * MY * 2 * MZ,
+    launch_pdl(k_add_dc, (B * W + 127) / 128, 128, 0, n->stream, n->Xh[l], n->hmean, B * W, (long long)MX * MY * 2 * MZ,
                                                          (float)n->S);
     NCK(n, cudaGetLastError(), "dc mode");
     MixDims md{B, W, MX, MY, MZ};
     const unsigned mix_grid = (unsigned)(((long long)MX * MY * MZ + 7) / 8);
     if (mix32(n, n->params + n->oWm[l]))
-        k_mix_fwd32<<<mix_grid, 256, MIX_SMAT, n->stream>>>(n->Xh[l], n->params + n->oWm[l], md, n->yh);
+        launch_pdl(k_mix_fwd32, mix_grid, 256, MIX_SMAT, n->stream, n->Xh[l], n->params + n->oWm[l], md, n->yh);
     else
-        k_mix_fwd<<<mix_grid, 256, 0, n->stream>>>(n->Xh[l], n->params + n->oWm[l], md, n->yh);
+        launch_pdl(k_mix_fwd, mix_grid, 256, 0, n->stream, n->Xh[l], n->params + n->oWm[l], md, n->yh);
     NCK(n, cudaGetLastError(), "mix");
     // inverse z: rows (b,o,kx,ky), K = (ri,kz) -> u1 [b][o][kx][ky][ri][z]
     NCK(n, gemm(n, (int)R, 2 * D, 2 * MZ, 1, n->yh, 2 * MZ, 1, 0, n->HZ, 2 * D, 1, 0, n->u1, 2 * D, 1, 0, 1, 0), "iz");
@@ -1387,19 +1423,19 @@ lbm_status spectral_bwd(lbm_no* n, int l, const float* dz, float* dh, int parts)
     // adjoint of inverse z -> dYh (FP32)
     NCK(n, gemm(n, (int)R, 2 * MZ, 2 * D, 1, n->u1, 2 * D, 1, 0, n->HZ, 1, 2 * D, 0, n->dyh, 2 * MZ, 1, 0, 0, 0), "iz^T");
     // the mean's mode: the adjoint of the inverse's 1/D^3 sum over the grid = the mean
-    k_add_dc<<<(B * W + 127) / 128, 128, 0, n->stream>>>(n->dyh, n->hmean, B * W, (long long)MX * MY * 2 * MZ, 1.0f);
+    launch_pdl(k_add_dc, (B * W + 127) / 128, 128, 0, n->stream, n->dyh, n->hmean, B * W, (long long)MX * MY * 2 * MZ, 1.0f);
     NCK(n, cudaGetLastError(), "dc mode");
     MixDims md{B, W, MX, MY, MZ};
     const unsigned mix_grid = (unsigned)(((long long)MX * MY * MZ + 7) / 8);
     if (mix32(n, n->params + n->oWm[l]) && mix32(n, n->grads + n->oWm[l])) {
         // the gradient buffer was zeroed by backward() and this is the only writer of the block
-        k_mix_bwd_w32<<<mix_grid, 256, 0, n->stream>>>(n->dyh, n->Xh[l], md, n->grads + n->oWm[l], 0);
+        launch_pdl(k_mix_bwd_w32, mix_grid, 256, 0, n->stream, n->dyh, n->Xh[l], md, n->grads + n->oWm[l], 0);
         NCK(n, cudaGetLastError(), "mix dW");
-        k_mix_bwd_x32<<<mix_grid, 256, MIX_SMAT, n->stream>>>(n->dyh, n->params + n->oWm[l], md, n->yh);
+        launch_pdl(k_mix_bwd_x32, mix_grid, 256, MIX_SMAT, n->stream, n->dyh, n->params + n->oWm[l], md, n->yh);
     } else {
-        k_mix_bwd_w<<<mix_grid, 256, 0, n->stream>>>(n->dyh, n->Xh[l], md, n->grads + n->oWm[l]);
+        launch_pdl(k_mix_bwd_w, mix_grid, 256, 0, n->stream, n->dyh, n->Xh[l], md, n->grads + n->oWm[l]);
         NCK(n, cudaGetLastError(), "mix dW");
-        k_mix_bwd_x<<<mix_grid, 256, 0, n->stream>>>(n->dyh, n->params + n->oWm[l], md, n->yh);
+        launch_pdl(k_mix_bwd_x, mix_grid, 256, 0, n->stream, n->dyh, n->params + n->oWm[l], md, n->yh);
     }
     NCK(n, cudaGetLastError(), "mix dX");
     // adjoint of forward z -> t2p layout
@@ -1433,15 +1469,15 @@ lbm_status forward(lbm_no* n, int B, const float* in, float* out) {
     // the row-vectorised maps need S a multiple of 4; every buffer here is 16-byte aligned
     const bool rowv = S % 4 == 0;
     if (rowv && n->Ci <= VEC_CH)
-        k_lift_v<<<grid_rows(S, B), 256, 0, n->stream>>>(n->a_in, n->params + n->oP, n->params + n->op, n->Ci, W, S, n->h0,
+        launch_pdl(k_lift_v, grid_rows(S, B), 256, 0, n->stream, n->a_in, n->params + n->oP, n->params + n->op, n->Ci, W, S, n->h0,
                                                           n->hb[0]);
     else
-        k_lift<<<grid_for(tot), 256, 0, n->stream>>>(n->a_in, n->params + n->oP, n->params + n->op, B, n->Ci, W, S, n->h0,
+        launch_pdl(k_lift, grid_for(tot), 256, 0, n->stream, n->a_in, n->params + n->oP, n->params + n->op, B, n->Ci, W, S, n->h0,
                                                     n->hb[0]);
     NCK(n, cudaGetLastError(), "lift");
     int parts = 0;
     for (int l = 0; l < n->L; ++l) {
-        k_f32_to_bf16<<<grid_for((long long)W * W), 256, 0, n->stream>>>(n->params + n->oWc[l], n->wcb + (long long)l * W * W,
+        launch_pdl(k_f32_to_bf16, grid_for((long long)W * W), 256, 0, n->stream, n->params + n->oWc[l], n->wcb + (long long)l * W * W,
                                                                            (long long)W * W);
         st = l == 0 ? spectral_fwd(n, l, n->h0, 0, n->z[l], 0) : spectral_fwd(n, l, n->z[l - 1], 1, n->z[l], parts);
         if (st) return st;
@@ -1452,19 +1488,19 @@ lbm_status forward(lbm_no* n, int B, const float* in, float* out) {
         // the row kernel also leaves the next layer's centring sums of act(z) in cpart
         parts = rowv && l < n->L - 1 ? n->rowparts : 0;
         if (rowv)
-            k_bias_act_v<<<dim3(row_blocks(S), B * W), 256, 0, n->stream>>>(n->z[l], n->params + n->obc[l], W, S,
+            launch_pdl(k_bias_act_v, dim3(row_blocks(S), B * W), 256, 0, n->stream, n->z[l], n->params + n->obc[l], W, S,
                                                                                   l < n->L - 1 ? 1 : 0, n->hb[l + 1],
                                                                                   parts ? n->cpart : nullptr);
         else
-            k_bias_act<<<grid_for(tot), 256, 0, n->stream>>>(n->z[l], n->params + n->obc[l], W, S, tot,
+            launch_pdl(k_bias_act, grid_for(tot), 256, 0, n->stream, n->z[l], n->params + n->obc[l], W, S, tot,
                                                             l < n->L - 1 ? 1 : 0, n->hb[l + 1]);
         NCK(n, cudaGetLastError(), "bias act");
     }
     if (rowv && n->Co <= VEC_CH && (reinterpret_cast<uintptr_t>(out) & 15u) == 0)
-        k_project_v<<<grid_rows(S, B), 256, 0, n->stream>>>(n->z[n->L - 1], n->params + n->oQ, n->params + n->oq, W, n->Co,
+        launch_pdl(k_project_v, grid_rows(S, B), 256, 0, n->stream, n->z[n->L - 1], n->params + n->oQ, n->params + n->oq, W, n->Co,
                                                              S, out);
     else
-        k_project<<<grid_for((long long)B * n->Co * S), 256, 0, n->stream>>>(n->z[n->L - 1], n->params + n->oQ,
+        launch_pdl(k_project, grid_for((long long)B * n->Co * S), 256, 0, n->stream, n->z[n->L - 1], n->params + n->oQ,
                                                                             n->params + n->oq, B, W, n->Co, S, out);
     NCK(n, cudaGetLastError(), "project");
     return LBM_OK;
@@ -1479,22 +1515,22 @@ lbm_status backward(lbm_no* n, const float* dout) {
     NCK(n, reduce_bs(n, dout, n->z[L - 1], n->Co, W, n->grads + n->oQ), "projection dW");
     NCK(n, reduce_bs(n, dout, nullptr, n->Co, 1, n->grads + n->oq), "projection db");
     if (S % 4 == 0 && n->Co <= VEC_CH && (reinterpret_cast<uintptr_t>(dout) & 15u) == 0)
-        k_project_bwd_x_v<<<grid_rows(S, B), 256, 0, n->stream>>>(dout, n->params + n->oQ, W, n->Co, S, n->dh);
+        launch_pdl(k_project_bwd_x_v, grid_rows(S, B), 256, 0, n->stream, dout, n->params + n->oQ, W, n->Co, S, n->dh);
     else
-        k_project_bwd_x<<<grid_for(tot), 256, 0, n->stream>>>(dout, n->params + n->oQ, B, W, n->Co, S, n->dh);
+        launch_pdl(k_project_bwd_x, grid_for(tot), 256, 0, n->stream, dout, n->params + n->oQ, B, W, n->Co, S, n->dh);
     NCK(n, cudaGetLastError(), "project bwd");
     for (int l = L - 1; l >= 0; --l) {
         // the row kernel leaves the row sums of dz in cpart: the bias gradient and the centring
         // of the spectral adjoint's input
         const int parts = n->rowparts;
         if (parts) {
-            k_act_bwd_v<<<dim3(row_blocks(S), B * W), 256, 0, n->stream>>>(n->dh, n->z[l], S, l < L - 1 ? 1 : 0, n->dz,
+            launch_pdl(k_act_bwd_v, dim3(row_blocks(S), B * W), 256, 0, n->stream, n->dh, n->z[l], S, l < L - 1 ? 1 : 0, n->dz,
                                                                                  n->dzb, n->cpart);
             NCK(n, cudaGetLastError(), "act bwd");
-            k_rows_to_bias<<<(W + 3) / 4, 128, 0, n->stream>>>(n->cpart, B, W, parts, n->grads + n->obc[l]);
+            launch_pdl(k_rows_to_bias, (W + 3) / 4, 128, 0, n->stream, n->cpart, B, W, parts, n->grads + n->obc[l]);
             NCK(n, cudaGetLastError(), "bias db");
         } else {
-            k_act_bwd<<<grid_for(tot), 256, 0, n->stream>>>(n->dh, n->z[l], tot, l < L - 1 ? 1 : 0, n->dz, n->dzb);
+            launch_pdl(k_act_bwd, grid_for(tot), 256, 0, n->stream, n->dh, n->z[l], tot, l < L - 1 ? 1 : 0, n->dz, n->dzb);
             NCK(n, reduce_bs(n, n->dz, nullptr, W, 1, n->grads + n->obc[l]), "bias db");
             NCK(n, cudaGetLastError(), "act bwd");
         }
@@ -1526,7 +1562,7 @@ lbm_status backward(lbm_no* n, const float* dout) {
                             part_b + (long long)full * W * W, W, 1, 0, 0, 0),
                     "conv dW rest");
         }
-        k_sum_partials<<<(W * W + 31) / 32, 512, 0, n->stream>>>(n->part, B * nk, W * W, n->grads + n->oWc[l]);
+        launch_pdl(k_sum_partials, (W * W + 31) / 32, 512, 0, n->stream, n->part, B * nk, W * W, n->grads + n->oWc[l]);
         NCK(n, cudaGetLastError(), "conv dW sum");
         // dh_l = Wc^T dz (conv) + spectral adjoint
         NCK(n, gemm(n, (int)S, W, W, B, n->dzb, 1, S, (long long)W * S, n->wcb + (long long)l * W * W, W, 1, 0, n->dh2, 1, S,
@@ -1715,7 +1751,7 @@ lbm_status step_body(lbm_no* n, int batch) {
     if (st) return st;
     const long long cnt = (long long)batch * n->Co * n->S;
     NCK(n, cudaMemsetAsync(n->loss_d, 0, sizeof(double), n->stream), "loss reset");
-    k_mse<<<grid_for(cnt), 256, 0, n->stream>>>(out, n->tgt, cnt, n->dout, n->loss_d);
+    launch_pdl(k_mse, grid_for(cnt), 256, 0, n->stream, out, n->tgt, cnt, n->dout, n->loss_d);
     NCK(n, cudaGetLastError(), "loss");
     st = backward(n, n->dout);
     if (st) return st;
@@ -1724,11 +1760,11 @@ lbm_status step_body(lbm_no* n, int batch) {
     // last n mod 4 one by one
     const long long n4 = n->nparam / 4, tail = n->nparam - 4 * n4;
     if (n4 > 0)
-        k_adam_v<<<grid_for(n4), 256, 0, n->stream>>>(reinterpret_cast<float4*>(n->params), reinterpret_cast<const float4*>(n->grads),
+        launch_pdl(k_adam_v, grid_for(n4), 256, 0, n->stream, reinterpret_cast<float4*>(n->params), reinterpret_cast<const float4*>(n->grads),
                                                       reinterpret_cast<float4*>(n->adam_m), reinterpret_cast<float4*>(n->adam_v), n4,
                                                       n->adam_sc, b1, b2, 1e-8f);
     if (tail > 0)
-        k_adam<<<1, 32, 0, n->stream>>>(n->params + 4 * n4, n->grads + 4 * n4, n->adam_m + 4 * n4, n->adam_v + 4 * n4, tail, n->adam_sc,
+        launch_pdl(k_adam, 1, 32, 0, n->stream, n->params + 4 * n4, n->grads + 4 * n4, n->adam_m + 4 * n4, n->adam_v + 4 * n4, tail, n->adam_sc,
                                         b1, b2, 1e-8f);
     NCK(n, cudaGetLastError(), "adam");
     return LBM_OK;
@@ -1779,7 +1815,7 @@ lbm_status lbm_no_train_step(lbm_no* n, int batch, const float* in, const float*
     ++n->adam_t;
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.0f - powf(b1, (float)n->adam_t), c2 = 1.0f - powf(b2, (float)n->adam_t);
-    k_set_adam_scalars<<<1, 1, 0, n->stream>>>(n->adam_sc, lr, c1, c2);
+    launch_pdl(k_set_adam_scalars, 1, 1, 0, n->stream, n->adam_sc, lr, c1, c2);
     NCK(n, cudaGetLastError(), "adam scalars");
     // the first step runs eagerly (one-time set-up of kernel attributes), later ones replay a graph
     bool replayed = false;
