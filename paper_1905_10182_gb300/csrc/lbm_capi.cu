@@ -567,6 +567,7 @@ lbm_status lbm_set_colour_gradient(lbm_ctx* c, const lbm_cg_params* prm, const f
     c->cg.A = prm->A;
     c->cg.beta = prm->beta;
     for (int a = 0; a < 3; ++a) c->cg.g[a] = prm->g[a];
+    c->cg.rev = 2.0 * 27.0 * sizeof(float) * (double)c->N > (double)c->l2;
     if (!c->cgb) {
         CK(c, cudaMalloc(&c->cgb, sizeof(float) * 27 * c->N), "cudaMalloc(blue store)");
         CK(c, cudaMalloc(&c->cgf, sizeof(float) * 2 * c->N), "cudaMalloc(phase fields)");

@@ -133,12 +133,14 @@ __device__ __forceinline__ bool node_at(const KParams& p, uint32_t n, int& x, in
     z = (int)zr + p.z0;
     return true;
 }
+// rev: the blocks in reverse order.
 template <bool FLAT>
-__device__ __forceinline__ bool node_of(const KParams& p, int& x, int& y, int& z) {
-    if (FLAT) return node_at(p, blockIdx.x * BLOCK_X + threadIdx.x, x, y, z);
-    x = (int)(blockIdx.x * BLOCK_X + threadIdx.x);
-    y = (int)blockIdx.y;
-    z = (int)blockIdx.z + p.z0;
+__device__ __forceinline__ bool node_of(const KParams& p, int& x, int& y, int& z, bool rev = false) {
+    const uint32_t bx = rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+    if (FLAT) return node_at(p, bx * BLOCK_X + threadIdx.x, x, y, z);
+    x = (int)(bx * BLOCK_X + threadIdx.x);
+    y = (int)(rev ? gridDim.y - 1 - blockIdx.y : blockIdx.y);
+    z = (int)(rev ? gridDim.z - 1 - blockIdx.z : blockIdx.z) + p.z0;
     return x < p.nx;
 }
 

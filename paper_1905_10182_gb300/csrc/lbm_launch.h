@@ -63,6 +63,7 @@ cudaError_t launch_mhd_copy(const KParams& p, float* hm, const float bw[3], int 
 // fb the blue store, fld 2 N (phi, rho); macro out: 6 planes (rho, u, rho_r, rho_b)
 struct CgParams {
     double rho_r0, rho_b0, nu_r, nu_b, A, beta, g[3];
+    int rev;  // the two stores exceed L2: the fields pass walks the grid backwards
 };
 cudaError_t launch_cg_step(const KParams& p, const CgParams& c, void* fr, float* fb, float* fld, int odd,
                            cudaStream_t st);
