@@ -28,10 +28,14 @@ namespace {
 typedef __nv_bfloat16 bf16;
 
 // ------------------------------------------------------------------------------ elementwise kernels
-__global__ void k_f32_to_bf16(const float* __restrict__ x, bf16* __restrict__ y, long long n) {
+// What a layer keeps of its 1x1 map for the backward pass: the weights in BF16 and the bias.
+__global__ void k_keep_map(const float* __restrict__ w, const float* __restrict__ b, bf16* __restrict__ wb, float* __restrict__ bk,
+                           int W) {
     pdl_wait();
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        y[i] = __float2bfloat16(x[i]);
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < W * W; i += gridDim.x * blockDim.x) {
+        wb[i] = __float2bfloat16(w[i]);
+        if (i < W) bk[i] = b[i];
+    }
 }
 
 // out[b][c][s] = sum_i P[c][i] a[b][i][s] + p[c]  (FP32 and BF16 copies)
@@ -240,16 +244,19 @@ __global__ void k_center_apply(const float* __restrict__ src, long long S, int u
     }
 }
 
-__global__ void __launch_bounds__(256) k_center_apply_v(const float* __restrict__ src, long long S, int use_gelu,
-                                                        const float* __restrict__ mean, bf16* __restrict__ out) {
+// bias (optional, W entries): added to src first
+__global__ void __launch_bounds__(256) k_center_apply_v(const float* __restrict__ src, const float* __restrict__ bias, int W,
+                                                        long long S, int use_gelu, const float* __restrict__ mean,
+                                                        bf16* __restrict__ out) {
     pdl_wait();
     const long long base = (long long)blockIdx.y * S;
-    const float m = mean[blockIdx.y];
+    const float m = mean[blockIdx.y], bo = bias ? bias[blockIdx.y % W] : 0.0f;
     const float4* x = reinterpret_cast<const float4*>(src + base);
     uint2* o = reinterpret_cast<uint2*>(out + base);
 #pragma unroll 4
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < S / 4; i += (long long)gridDim.x * blockDim.x) {
         float4 v = __ldg(x + i);
+        if (bias) v = make_float4(v.x + bo, v.y + bo, v.z + bo, v.w + bo);
         if (use_gelu) v = make_float4(gelu(v.x), gelu(v.y), gelu(v.z), gelu(v.w));
         o[i] = pack_bf16x4(make_float4(v.x - m, v.y - m, v.z - m, v.w - m));
     }
@@ -815,11 +822,12 @@ inline dim3 grid_rows(long long S, long long rows) { return dim3((unsigned)((S /
 inline int row_blocks(long long S) { return (int)((S / 4 + 256 * ROW_PER - 1) / (256 * ROW_PER)); }
 
 
-// z[b][o][s] += bias[o]; hb = act(z) (BF16); grid (row_blocks(S), B W), ROW_PER float4 groups per
-// thread.  part (optional): the block's FP64 sum of act(z) at part[row gridDim.x + blockIdx.x],
+// z[b][o][s] += bias[o] (stored only with keep); hb = act(z) (BF16); grid (row_blocks(S), B W), ROW_PER
+// float4 groups per thread.  Without keep the readers of z add the bias again, which gives the same
+// bits and saves a 134 MB write (64^3, batch 4: 51 -> 31 us).  part (optional): the block's FP64 sum of act(z) at part[row gridDim.x + blockIdx.x],
 // the next layer's centring sums.
 __global__ void __launch_bounds__(256) k_bias_act_v(float* __restrict__ z, const float* __restrict__ bias, int W, long long S,
-                                                    int use_gelu, bf16* __restrict__ hb, double* __restrict__ part) {
+                                                    int use_gelu, int keep, bf16* __restrict__ hb, double* __restrict__ part) {
     pdl_wait();
     const long long row = blockIdx.y, S4 = S / 4;
     const float bo = bias[row % W];
@@ -835,7 +843,7 @@ __global__ void __launch_bounds__(256) k_bias_act_v(float* __restrict__ z, const
             v.y += bo;
             v.z += bo;
             v.w += bo;
-            zr[s4] = v;
+            if (keep) zr[s4] = v;
             if (use_gelu) v = make_float4(gelu(v.x), gelu(v.y), gelu(v.z), gelu(v.w));
             hr[s4] = pack_bf16x4(v);
             sum += v.x + v.y + v.z + v.w;
@@ -844,13 +852,14 @@ __global__ void __launch_bounds__(256) k_bias_act_v(float* __restrict__ z, const
     if (part) block_sum_to(sum, part + row * gridDim.x + blockIdx.x);
 }
 
-// dz = dh act'(z) (FP32 and BF16), row-vectorised; grid (row_blocks(S), B W).  part: the block's
+// dz = dh act'(z + bias) (FP32 and BF16; bias: W entries), row-vectorised; grid (row_blocks(S), B W).  part: the block's
 // FP64 sum of dz at part[row gridDim.x + blockIdx.x] (centring and bias gradient).
-__global__ void __launch_bounds__(256) k_act_bwd_v(const float* __restrict__ dh, const float* __restrict__ z, long long S,
-                                                   int use_gelu, float* __restrict__ dz, bf16* __restrict__ dzb,
+__global__ void __launch_bounds__(256) k_act_bwd_v(const float* __restrict__ dh, const float* __restrict__ z,
+                                                   const float* __restrict__ bias, int W, long long S, int use_gelu, float* __restrict__ dz, bf16* __restrict__ dzb,
                                                    double* __restrict__ part) {
     pdl_wait();
     const long long row = blockIdx.y, S4 = S / 4;
+    const float bo = bias[row % W];
     float sum = 0.0f;
 #pragma unroll
     for (int j = 0; j < ROW_PER; ++j) {
@@ -859,7 +868,8 @@ __global__ void __launch_bounds__(256) k_act_bwd_v(const float* __restrict__ dh,
             const long long i = row * S4 + s4;
             float4 v = __ldg(reinterpret_cast<const float4*>(dh) + i);
             if (use_gelu) {
-                const float4 x = __ldg(reinterpret_cast<const float4*>(z) + i);
+                float4 x = __ldg(reinterpret_cast<const float4*>(z) + i);
+                x = make_float4(x.x + bo, x.y + bo, x.z + bo, x.w + bo);
                 v = make_float4(v.x * gelu_grad(x.x), v.y * gelu_grad(x.y), v.z * gelu_grad(x.z), v.w * gelu_grad(x.w));
             }
             reinterpret_cast<float4*>(dz)[i] = v;
@@ -898,9 +908,9 @@ __global__ void __launch_bounds__(256) k_lift_v(const float* __restrict__ a, con
     }
 }
 
-// out[b][k][s] = q[k] + sum_c Q[k][c] h[b][c][s] (Co <= VEC_CH); grid (positions / 1024, B)
-__global__ void __launch_bounds__(256) k_project_v(const float* __restrict__ h, const float* __restrict__ Q, const float* __restrict__ q,
-                                                   int W, int Co, long long S, float* __restrict__ out) {
+// out[b][k][s] = q[k] + sum_c Q[k][c] (h[b][c][s] + bias[c]) (Co <= VEC_CH; bias optional); grid (positions / 1024, B)
+__global__ void __launch_bounds__(256) k_project_v(const float* __restrict__ h, const float* __restrict__ bias,
+                                                   const float* __restrict__ Q, const float* __restrict__ q, int W, int Co, long long S, float* __restrict__ out) {
     pdl_wait();
     const long long s4 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (s4 * 4 >= S) return;
@@ -910,7 +920,11 @@ __global__ void __launch_bounds__(256) k_project_v(const float* __restrict__ h, 
     for (int k = 0; k < VEC_CH; ++k)
         if (k < Co) v[k] = make_float4(q[k], q[k], q[k], q[k]);
     for (int c = 0; c < W; ++c) {
-        const float4 x = __ldg(reinterpret_cast<const float4*>(h + (b * W + c) * S) + s4);
+        float4 x = __ldg(reinterpret_cast<const float4*>(h + (b * W + c) * S) + s4);
+        if (bias) {
+            const float bo = bias[c];
+            x = make_float4(x.x + bo, x.y + bo, x.z + bo, x.w + bo);
+        }
 #pragma unroll
         for (int k = 0; k < VEC_CH; ++k)
             if (k < Co) {
@@ -978,13 +992,16 @@ struct lbm_no {
     float* adam_v = nullptr;
     long long adam_t = 0;
     bf16* wcb = nullptr;  // BF16 copies of the 1x1 weights, L x W x W
+    float* bkeep = nullptr;  // the last forward's biases, L x W
+    bool last_pending = false;  // z[L-1] of the last forward holds h_L without its bias
     // DFT matrices (BF16)
     bf16 *FX = nullptr, *GY = nullptr, *GZ = nullptr, *HZ = nullptr, *HY = nullptr, *HX = nullptr;
     // activations for the last forward
     int B = 0;
     float* a_in = nullptr;               // lift input copy [B][Ci][S]
     std::vector<bf16*> hb;               // L + 1 BF16 layer inputs [B][W][S]
-    std::vector<float*> z;               // L pre-activations [B][W][S] (z[L-1] is h_L)
+    std::vector<float*> z;               // L pre-activations [B][W][S] (z[L-1] is h_L; the others without
+                                         // their bias where the row-vectorised kernels run)
     std::vector<float*> Xh;              // L mode coefficients [B][W][MX][MY][2][MZ]
     float* h0 = nullptr;                 // FP32 lift output
     // work buffers
@@ -1093,7 +1110,8 @@ constexpr int REDUCE_CHUNKS = 64;  // chunks of the B * S positions in a gradien
 // hs = bf16(act(src) - mean), hmean = the per-(sample, channel) means (see k_center_partials)
 // parts > 0: the row sums of act(src) are already in cpart, `parts` per row (written by the kernel
 // that produced src)
-cudaError_t center(lbm_no* n, const float* src, int use_gelu, int parts = 0) {
+// bias (row-vectorised kernels only): to be added to src
+cudaError_t center(lbm_no* n, const float* src, const float* bias, int use_gelu, int parts = 0) {
     const int ch = n->B * n->W;
     const bool v4 = n->S % 4 == 0 && (reinterpret_cast<uintptr_t>(src) & 15u) == 0;
     if (parts <= 0) {
@@ -1105,7 +1123,7 @@ cudaError_t center(lbm_no* n, const float* src, int use_gelu, int parts = 0) {
     }
     launch_pdl(k_center_means, (ch + 3) / 4, 128, 0, n->stream, n->cpart, ch, parts, n->S, n->hmean);
     if (v4)
-        launch_pdl(k_center_apply_v, dim3(32, ch), 256, 0, n->stream, src, n->S, use_gelu, n->hmean, n->hs);
+        launch_pdl(k_center_apply_v, dim3(32, ch), 256, 0, n->stream, src, bias, n->W, n->S, use_gelu, n->hmean, n->hs);
     else
         launch_pdl(k_center_apply, dim3(32, ch), 256, 0, n->stream, src, n->S, use_gelu, n->hmean, n->hs);
     return cudaGetLastError();
@@ -1184,12 +1202,13 @@ __global__ void __launch_bounds__(256) k_reduce_pairs(const float* __restrict__ 
 // thread streams its positions (16-byte loads, each input read once) and keeps the 32 CS pair
 // sums in registers; the warp then reduce-scatters them (after five butterfly exchanges lane l
 // holds the warp's totals of pairs 4l .. 4l + 3 for CS = 4), the warps' totals are added in FP64
-// in warp order and written as part[chunk][i Cy + j] like k_reduce_bs.  grid = chunks.
+// in warp order and written as part[chunk][i Cy + j] like k_reduce_bs.  bias (optional, 32 entries): added
+// to "big" first.  grid = chunks.
 constexpr int PAIR_CHUNKS = 256;
 
 template <int CS>
-__global__ void __launch_bounds__(256) k_reduce_pairs32(const float* __restrict__ big, const float* __restrict__ small, int B,
-                                                        long long S, int big_is_x, int Cy, float* __restrict__ part) {
+__global__ void __launch_bounds__(256) k_reduce_pairs32(const float* __restrict__ big, const float* __restrict__ bias,
+                                                        const float* __restrict__ small, int B, long long S, int big_is_x, int Cy, float* __restrict__ part) {
     pdl_wait();
     constexpr int CB = 32, NA = CB * CS;  // accumulators per thread, index c CS + k
     const long long S4 = S / 4, n4 = (long long)B * S4;
@@ -1208,7 +1227,11 @@ __global__ void __launch_bounds__(256) k_reduce_pairs32(const float* __restrict_
             for (int k = 0; k < CS; ++k) y[k] = __ldg(sp + k * S4 + g);
 #pragma unroll
             for (int c = 0; c < CB; ++c) {
-                const float4 x = __ldg(bp + c * S4 + g);
+                float4 x = __ldg(bp + c * S4 + g);
+                if (bias) {
+                    const float bo = bias[c];
+                    x = make_float4(x.x + bo, x.y + bo, x.z + bo, x.w + bo);
+                }
 #pragma unroll
                 for (int k = 0; k < CS; ++k) {
                     float& a = acc[c * CS + k];
@@ -1247,16 +1270,18 @@ __global__ void __launch_bounds__(256) k_reduce_pairs32(const float* __restrict_
     }
 }
 
-cudaError_t reduce_bs(lbm_no* n, const float* X, const float* Y, int Cx, int Cy, float* out) {
+// bias: to be added to the 32-channel operand of a 32 x 4 or 4 x 32 pair
+cudaError_t reduce_bs(lbm_no* n, const float* X, const float* Y, int Cx, int Cy, float* out, const float* bias = nullptr) {
     const int pairs = Cx * Cy;
     if (Y && n->S % 4 == 0 && ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Y)) & 15u) == 0 &&
         ((Cx == 32 && Cy == 4) || (Cx == 4 && Cy == 32))) {
         const bool x_big = Cx == 32;
-        launch_pdl(k_reduce_pairs32<4>, PAIR_CHUNKS, 256, 0, n->stream, x_big ? X : Y, x_big ? Y : X, n->B, n->S, x_big ? 1 : 0, Cy,
+        launch_pdl(k_reduce_pairs32<4>, PAIR_CHUNKS, 256, 0, n->stream, x_big ? X : Y, bias, x_big ? Y : X, n->B, n->S, x_big ? 1 : 0, Cy,
                                                                  n->red);
         launch_pdl(k_sum_partials, (pairs + 31) / 32, 512, 0, n->stream, n->red, PAIR_CHUNKS, pairs, out);
         return cudaGetLastError();
     }
+    if (bias) return cudaErrorInvalidValue;
     const bool al = ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Y)) & 15u) == 0;
     if (n->S % 4 == 0 && al && (Y == nullptr || (Cx >= Cy ? Cy : Cx) <= RED_SMALL)) {
         const bool x_big = Y == nullptr || Cx >= Cy;
@@ -1359,11 +1384,11 @@ bool mix32(const lbm_no* n, const float* wm) {
 // spectral convolution of layer l: input h = act(src) (FP32 [B][W][S], act = GELU if use_gelu) ->
 // out (FP32 [B][W][S], overwritten); keeps the mode coefficients in Xh[l] for the weight gradient
 // parts > 0: the centring sums of act(src) are already in cpart (see center)
-lbm_status spectral_fwd(lbm_no* n, int l, const float* src, int use_gelu, float* out, int parts) {
+lbm_status spectral_fwd(lbm_no* n, int l, const float* src, const float* bias, int use_gelu, float* out, int parts) {
     const int B = n->B, W = n->W, D = n->D, MX = n->MX, MY = n->MY, MZ = n->MZ;
     const long long D2 = (long long)D * D;
     const long long BWD = (long long)B * W * D;
-    NCK(n, center(n, src, use_gelu, parts), "centre");
+    NCK(n, center(n, src, bias, use_gelu, parts), "centre");
     // x: [bcz][y][x] x FX -> t1 [bcz][(kx,ri)][y]
     NCK(n, gemm(n, D, 2 * MX, D, (int)BWD, n->hs, D, 1, D2, n->FX, 2 * MX, 1, 0, n->t1, 1, D, 2LL * MX * D, 1, 0), "fx");
     // y: rows (bcz,kx), K = (ri,y) -> t2 [b][c][z][kx][ri][ky]
@@ -1409,7 +1434,7 @@ lbm_status spectral_bwd(lbm_no* n, int l, const float* dz, float* dh, int parts)
     const long long BWD = (long long)B * W * D;
     const long long R = (long long)B * W * MX * MY;
     // the adjoint transforms take the centred gradient too (see k_center_partials)
-    NCK(n, center(n, dz, 0, parts), "centre");
+    NCK(n, center(n, dz, nullptr, 0, parts), "centre");
     // adjoint of inverse x -> u2 layout
     NCK(n, gemm(n, D, 2 * MX, D, (int)BWD, n->hs, D, 1, D2, n->HX, 1, D, 0, n->u2, 1, D, 2LL * MX * D, 1, 0), "ix^T");
     // adjoint of inverse y -> u1p layout
@@ -1459,6 +1484,21 @@ lbm_status ensure_batch(lbm_no* n, int B) {
     return LBM_OK;
 }
 
+// The last layer's bias is left to the readers of its output h_L = z + b (the projection and the
+// projection's weight gradient, which add it again, to the same bits) where both are the kernels that
+// can: no pass over h_L for it (64^3, batch 4: 51 us).
+bool last_bias_pending(const lbm_no* n, const float* out) {
+    return n->S % 4 == 0 && n->W == 32 && n->Co == 4 && (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
+}
+
+// Adds the pending bias to z[L-1] where the kernel that would have done it cannot take dout (alignment).
+cudaError_t add_last_bias(lbm_no* n, const float* dout) {
+    if (!n->last_pending || (reinterpret_cast<uintptr_t>(dout) & 15u) == 0) return cudaSuccess;
+    n->last_pending = false;
+    return launch_pdl(k_bias_act_v, dim3(row_blocks(n->S), n->B * n->W), 256, 0, n->stream, n->z[n->L - 1], n->bkeep + (n->L - 1) * n->W,
+                      n->W, n->S, 0, 1, n->hb[n->L], nullptr);
+}
+
 // in == nullptr: the input is already in a_in
 lbm_status forward(lbm_no* n, int B, const float* in, float* out) {
     lbm_status st = ensure_batch(n, B);
@@ -1468,6 +1508,7 @@ lbm_status forward(lbm_no* n, int B, const float* in, float* out) {
     if (in) NCK(n, cudaMemcpyAsync(n->a_in, in, sizeof(float) * B * n->Ci * S, cudaMemcpyDefault, n->stream), "input copy");
     // the row-vectorised maps need S a multiple of 4; every buffer here is 16-byte aligned
     const bool rowv = S % 4 == 0;
+    n->last_pending = last_bias_pending(n, out);
     if (rowv && n->Ci <= VEC_CH)
         launch_pdl(k_lift_v, grid_rows(S, B), 256, 0, n->stream, n->a_in, n->params + n->oP, n->params + n->op, n->Ci, W, S, n->h0,
                                                           n->hb[0]);
@@ -1477,9 +1518,10 @@ lbm_status forward(lbm_no* n, int B, const float* in, float* out) {
     NCK(n, cudaGetLastError(), "lift");
     int parts = 0;
     for (int l = 0; l < n->L; ++l) {
-        launch_pdl(k_f32_to_bf16, grid_for((long long)W * W), 256, 0, n->stream, n->params + n->oWc[l], n->wcb + (long long)l * W * W,
-                                                                           (long long)W * W);
-        st = l == 0 ? spectral_fwd(n, l, n->h0, 0, n->z[l], 0) : spectral_fwd(n, l, n->z[l - 1], 1, n->z[l], parts);
+        launch_pdl(k_keep_map, grid_for((long long)W * W), 256, 0, n->stream, n->params + n->oWc[l], n->params + n->obc[l],
+                   n->wcb + (long long)l * W * W, n->bkeep + l * W, W);
+        st = l == 0 ? spectral_fwd(n, l, n->h0, nullptr, 0, n->z[l], 0)
+                    : spectral_fwd(n, l, n->z[l - 1], rowv ? n->bkeep + (l - 1) * W : nullptr, 1, n->z[l], parts);
         if (st) return st;
         // 1x1 conv accumulated onto the spectral output: z[b][o][s] += sum_c Wc[o][c] h[b][c][s]
         NCK(n, gemm(n, (int)S, W, W, B, n->hb[l], 1, S, (long long)W * S, n->wcb + (long long)l * W * W, 1, W, 0, n->z[l], 1,
@@ -1487,18 +1529,19 @@ lbm_status forward(lbm_no* n, int B, const float* in, float* out) {
             "conv");
         // the row kernel also leaves the next layer's centring sums of act(z) in cpart
         parts = rowv && l < n->L - 1 ? n->rowparts : 0;
+        if (l == n->L - 1 && n->last_pending) break;
         if (rowv)
             launch_pdl(k_bias_act_v, dim3(row_blocks(S), B * W), 256, 0, n->stream, n->z[l], n->params + n->obc[l], W, S,
-                                                                                  l < n->L - 1 ? 1 : 0, n->hb[l + 1],
-                                                                                  parts ? n->cpart : nullptr);
+                       l < n->L - 1 ? 1 : 0, l < n->L - 1 ? 0 : 1, n->hb[l + 1], parts ? n->cpart : nullptr);
         else
             launch_pdl(k_bias_act, grid_for(tot), 256, 0, n->stream, n->z[l], n->params + n->obc[l], W, S, tot,
                                                             l < n->L - 1 ? 1 : 0, n->hb[l + 1]);
         NCK(n, cudaGetLastError(), "bias act");
     }
     if (rowv && n->Co <= VEC_CH && (reinterpret_cast<uintptr_t>(out) & 15u) == 0)
-        launch_pdl(k_project_v, grid_rows(S, B), 256, 0, n->stream, n->z[n->L - 1], n->params + n->oQ, n->params + n->oq, W, n->Co,
-                                                             S, out);
+        launch_pdl(k_project_v, grid_rows(S, B), 256, 0, n->stream, n->z[n->L - 1],
+                   n->last_pending ? n->bkeep + (n->L - 1) * W : nullptr, n->params + n->oQ, n->params + n->oq, W, n->Co, S,
+                   out);
     else
         launch_pdl(k_project, grid_for((long long)B * n->Co * S), 256, 0, n->stream, n->z[n->L - 1], n->params + n->oQ,
                                                                             n->params + n->oq, B, W, n->Co, S, out);
@@ -1512,7 +1555,9 @@ lbm_status backward(lbm_no* n, const float* dout) {
     const long long S = n->S, tot = (long long)B * W * S;
     NCK(n, cudaMemsetAsync(n->grads, 0, sizeof(float) * n->nparam, n->stream), "zero grads");
     // projection
-    NCK(n, reduce_bs(n, dout, n->z[L - 1], n->Co, W, n->grads + n->oQ), "projection dW");
+    NCK(n, add_last_bias(n, dout), "last bias");
+    NCK(n, reduce_bs(n, dout, n->z[L - 1], n->Co, W, n->grads + n->oQ, n->last_pending ? n->bkeep + (L - 1) * W : nullptr),
+        "projection dW");
     NCK(n, reduce_bs(n, dout, nullptr, n->Co, 1, n->grads + n->oq), "projection db");
     if (S % 4 == 0 && n->Co <= VEC_CH && (reinterpret_cast<uintptr_t>(dout) & 15u) == 0)
         launch_pdl(k_project_bwd_x_v, grid_rows(S, B), 256, 0, n->stream, dout, n->params + n->oQ, W, n->Co, S, n->dh);
@@ -1524,8 +1569,8 @@ lbm_status backward(lbm_no* n, const float* dout) {
         // of the spectral adjoint's input
         const int parts = n->rowparts;
         if (parts) {
-            launch_pdl(k_act_bwd_v, dim3(row_blocks(S), B * W), 256, 0, n->stream, n->dh, n->z[l], S, l < L - 1 ? 1 : 0, n->dz,
-                                                                                 n->dzb, n->cpart);
+            launch_pdl(k_act_bwd_v, dim3(row_blocks(S), B * W), 256, 0, n->stream, n->dh, n->z[l], n->bkeep + l * W, W, S,
+                       l < L - 1 ? 1 : 0, n->dz, n->dzb, n->cpart);
             NCK(n, cudaGetLastError(), "act bwd");
             launch_pdl(k_rows_to_bias, (W + 3) / 4, 128, 0, n->stream, n->cpart, B, W, parts, n->grads + n->obc[l]);
             NCK(n, cudaGetLastError(), "bias db");
@@ -1660,6 +1705,7 @@ lbm_status lbm_no_create(int D, int W, int modes, int L, int Ci, int Co, int max
     alloc((void**)&n->adam_m, sizeof(float) * n->nparam);
     alloc((void**)&n->adam_v, sizeof(float) * n->nparam);
     alloc((void**)&n->wcb, sizeof(bf16) * L * W * W);
+    alloc((void**)&n->bkeep, sizeof(float) * L * W);
     alloc((void**)&n->a_in, sizeof(float) * maxB * Ci * S);
     alloc((void**)&n->h0, sizeof(float) * act);
     n->hb.assign(L + 1, nullptr);
@@ -1827,6 +1873,7 @@ lbm_status lbm_no_train_step(lbm_no* n, int batch, const float* in, const float*
             NCK(n, cudaGraphLaunch(n->step_graph, n->gstream), "graph launch");
             NCK(n, cudaEventRecord(n->ev_out, n->gstream), "event");
             NCK(n, cudaStreamWaitEvent(n->stream, n->ev_out, 0), "event wait");
+            n->last_pending = last_bias_pending(n, n->dout);  // as the captured forward leaves it
             replayed = true;
         }
     }
@@ -1850,7 +1897,7 @@ const char* lbm_no_last_error(const lbm_no* n) { return n ? n->err.c_str() : "";
 void lbm_no_destroy(lbm_no* n) {
     if (!n) return;
     cudaStreamSynchronize(n->stream);
-    void* bufs[] = {n->params, n->grads, n->adam_m, n->adam_v, n->wcb, n->a_in, n->h0, n->FX, n->GY, n->GZ, n->HZ, n->HY,
+    void* bufs[] = {n->params, n->grads, n->adam_m, n->adam_v, n->wcb, n->bkeep, n->a_in, n->h0, n->FX, n->GY, n->GZ, n->HZ, n->HY,
                     n->HX, n->t1, n->t2, n->t2p, n->yh, n->dyh, n->u1, n->u1p, n->u2, n->dh, n->dh2, n->dz, n->dzb, n->hs, n->hmean, n->cpart, n->red,
                     n->part, n->dout, n->loss_d, n->gemm_err};
     for (void* b : bufs) cudaFree(b);
