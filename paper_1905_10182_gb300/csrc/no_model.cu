@@ -28,13 +28,15 @@ namespace {
 typedef __nv_bfloat16 bf16;
 
 // ------------------------------------------------------------------------------ elementwise kernels
-// What a layer keeps of its 1x1 map for the backward pass: the weights in BF16 and the bias.
-__global__ void k_keep_map(const float* __restrict__ w, const float* __restrict__ b, bf16* __restrict__ wb, float* __restrict__ bk,
-                           int W) {
+// What the layers keep of their 1x1 maps for the backward pass: the weights in BF16 and the bias.  w, b:
+// the first layer's, the others `stride` parameters on; grid (blocks, layers).
+__global__ void k_keep_maps(const float* __restrict__ w, const float* __restrict__ b, long long stride, bf16* __restrict__ wb,
+                            float* __restrict__ bk, int W) {
     pdl_wait();
+    const int l = blockIdx.y;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < W * W; i += gridDim.x * blockDim.x) {
-        wb[i] = __float2bfloat16(w[i]);
-        if (i < W) bk[i] = b[i];
+        wb[(long long)l * W * W + i] = __float2bfloat16(w[l * stride + i]);
+        if (i < W) bk[l * W + i] = b[l * stride + i];
     }
 }
 
@@ -105,6 +107,16 @@ __global__ void k_bias_act(float* __restrict__ z, const float* __restrict__ bias
         z[idx] = v;
         hb[idx] = __float2bfloat16(use_gelu ? gelu(v) : v);
     }
+}
+
+// Zeroes the gradient vector outside the mode matrices: block 0 the parameters before the first one (the
+// lift), block l the ones from layer l - 1's 1x1 map on to the next mode matrix or the end.  wm, wc: offsets
+// of layer 0's mode matrix and 1x1 map, the other layers' `stride` on.
+__global__ void k_zero_dense(float* __restrict__ g, long long wm, long long wc, long long stride, int L, long long n) {
+    pdl_wait();
+    const int l = blockIdx.x;
+    const long long lo = l == 0 ? 0 : wc + (l - 1) * stride, hi = l == L ? n : wm + l * stride;
+    for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) g[i] = 0.0f;
 }
 
 // dz = dh * act'(z); BF16 copy for the GEMMs
@@ -725,7 +737,7 @@ __global__ void __launch_bounds__(512) k_sum_partials(const float* __restrict__ 
     const int k = blockIdx.x * 32 + lane;
     float a = 0.0f;
     if (k < K) {
-#pragma unroll 4
+#pragma unroll 16
         for (int p = warp; p < P; p += nw) a += part[(long long)p * K + k];
     }
     __shared__ float sh[16][32];
@@ -852,7 +864,8 @@ __global__ void __launch_bounds__(256) k_bias_act_v(float* __restrict__ z, const
     if (part) block_sum_to(sum, part + row * gridDim.x + blockIdx.x);
 }
 
-// dz = dh act'(z + bias) (FP32 and BF16; bias: W entries), row-vectorised; grid (row_blocks(S), B W).  part: the block's
+// dz = dh act'(z + bias) (FP32 and BF16; bias: W entries), row-vectorised; grid (row_blocks(S), B W).
+// Without the GELU dz is dh itself and only the BF16 copy is written.  part: the block's
 // FP64 sum of dz at part[row gridDim.x + blockIdx.x] (centring and bias gradient).
 __global__ void __launch_bounds__(256) k_act_bwd_v(const float* __restrict__ dh, const float* __restrict__ z,
                                                    const float* __restrict__ bias, int W, long long S, int use_gelu, float* __restrict__ dz, bf16* __restrict__ dzb,
@@ -872,7 +885,7 @@ __global__ void __launch_bounds__(256) k_act_bwd_v(const float* __restrict__ dh,
                 x = make_float4(x.x + bo, x.y + bo, x.z + bo, x.w + bo);
                 v = make_float4(v.x * gelu_grad(x.x), v.y * gelu_grad(x.y), v.z * gelu_grad(x.z), v.w * gelu_grad(x.w));
             }
-            reinterpret_cast<float4*>(dz)[i] = v;
+            if (use_gelu) reinterpret_cast<float4*>(dz)[i] = v;
             reinterpret_cast<uint2*>(dzb)[i] = pack_bf16x4(v);
             sum += v.x + v.y + v.z + v.w;
         }
@@ -908,27 +921,33 @@ __global__ void __launch_bounds__(256) k_lift_v(const float* __restrict__ a, con
     }
 }
 
-// out[b][k][s] = q[k] + sum_c Q[k][c] (h[b][c][s] + bias[c]) (Co <= VEC_CH; bias optional); grid (positions / 1024, B)
+// out[b][k][s] = q[k] + sum_c Q[k][c] (h[b][c][s] + bias[c]) (Co <= VEC_CH; bias with BIAS); CO: Co as a
+// constant, 0: read from Co; grid (positions / 1024, B).  Bound by HBM (h read once, 134 MB at 64^3, batch
+// 4); the channel loop must stay free of branches for its loads to be issued together.
+template <int CO, bool BIAS>
 __global__ void __launch_bounds__(256) k_project_v(const float* __restrict__ h, const float* __restrict__ bias,
-                                                   const float* __restrict__ Q, const float* __restrict__ q, int W, int Co, long long S, float* __restrict__ out) {
+                                                   const float* __restrict__ Q, const float* __restrict__ q, int W, int Co, long long S,
+                                                   float* __restrict__ out) {
     pdl_wait();
+    constexpr int K = CO > 0 ? CO : VEC_CH;
     const long long s4 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (s4 * 4 >= S) return;
     const long long b = blockIdx.y;
-    float4 v[VEC_CH];
+    float4 v[K];
 #pragma unroll
-    for (int k = 0; k < VEC_CH; ++k)
-        if (k < Co) v[k] = make_float4(q[k], q[k], q[k], q[k]);
+    for (int k = 0; k < K; ++k)
+        if (CO > 0 || k < Co) v[k] = make_float4(q[k], q[k], q[k], q[k]);
+#pragma unroll 8
     for (int c = 0; c < W; ++c) {
         float4 x = __ldg(reinterpret_cast<const float4*>(h + (b * W + c) * S) + s4);
-        if (bias) {
-            const float bo = bias[c];
+        if (BIAS) {
+            const float bo = __ldg(bias + c);
             x = make_float4(x.x + bo, x.y + bo, x.z + bo, x.w + bo);
         }
 #pragma unroll
-        for (int k = 0; k < VEC_CH; ++k)
-            if (k < Co) {
-                const float w = Q[k * W + c];
+        for (int k = 0; k < K; ++k)
+            if (CO > 0 || k < Co) {
+                const float w = __ldg(Q + k * W + c);
                 v[k].x += w * x.x;
                 v[k].y += w * x.y;
                 v[k].z += w * x.z;
@@ -936,8 +955,8 @@ __global__ void __launch_bounds__(256) k_project_v(const float* __restrict__ h, 
             }
     }
 #pragma unroll
-    for (int k = 0; k < VEC_CH; ++k)
-        if (k < Co) reinterpret_cast<float4*>(out + (b * Co + k) * S)[s4] = v[k];
+    for (int k = 0; k < K; ++k)
+        if (CO > 0 || k < Co) reinterpret_cast<float4*>(out + (b * Co + k) * S)[s4] = v[k];
 }
 
 // dh[b][c][s] = sum_k Q[k][c] dout[b][k][s] (Co <= VEC_CH); grid (positions / 1024, B)
@@ -1107,19 +1126,15 @@ cudaError_t permute(lbm_no* n, const bf16* in, bf16* out, const long long din[6]
 
 constexpr int REDUCE_CHUNKS = 64;  // chunks of the B * S positions in a gradient reduction
 
-// hs = bf16(act(src) - mean), hmean = the per-(sample, channel) means (see k_center_partials)
-// parts > 0: the row sums of act(src) are already in cpart, `parts` per row (written by the kernel
-// that produced src)
-// bias (row-vectorised kernels only): to be added to src
-cudaError_t center(lbm_no* n, const float* src, const float* bias, int use_gelu, int parts = 0) {
+// hs = bf16(act(src + bias) - mean), hmean = the per-(sample, channel) means (see k_center_partials)
+// parts > 0: the row sums of act(src + bias) are already in cpart, `parts` per row (written by the kernel
+// that produced src); bias only with the row-vectorised kernels
+cudaError_t center(lbm_no* n, const float* src, const float* bias, int use_gelu, int parts) {
     const int ch = n->B * n->W;
     const bool v4 = n->S % 4 == 0 && (reinterpret_cast<uintptr_t>(src) & 15u) == 0;
     if (parts <= 0) {
         parts = CENTER_PARTS;
-        if (v4)
-            launch_pdl(k_center_partials_v, ch * CENTER_PARTS, 256, 0, n->stream, src, n->S, use_gelu, n->cpart);
-        else
-            launch_pdl(k_center_partials, ch * CENTER_PARTS, 256, 0, n->stream, src, n->S, use_gelu, n->cpart);
+        launch_pdl(v4 ? k_center_partials_v : k_center_partials, ch * CENTER_PARTS, 256, 0, n->stream, src, n->S, use_gelu, n->cpart);
     }
     launch_pdl(k_center_means, (ch + 3) / 4, 128, 0, n->stream, n->cpart, ch, parts, n->S, n->hmean);
     if (v4)
@@ -1402,8 +1417,7 @@ lbm_status spectral_fwd(lbm_no* n, int l, const float* src, const float* bias, i
     const long long R = (long long)B * W * MX * MY;
     NCK(n, gemm(n, (int)R, 2 * MZ, 2 * D, 1, n->t2p, 2 * D, 1, 0, n->GZ, 2 * MZ, 1, 0, n->Xh[l], 2 * MZ, 1, 0, 0, 0), "fz");
     // the mean's mode: sum over the grid = S * mean
-    launch_pdl(k_add_dc, (B * W + 127) / 128, 128, 0, n->stream, n->Xh[l], n->hmean, B * W, (long long)MX * MY * 2 * MZ,
-                                                         (float)n->S);
+    launch_pdl(k_add_dc, (B * W + 127) / 128, 128, 0, n->stream, n->Xh[l], n->hmean, B * W, (long long)MX * MY * 2 * MZ, (float)n->S);
     NCK(n, cudaGetLastError(), "dc mode");
     MixDims md{B, W, MX, MY, MZ};
     const unsigned mix_grid = (unsigned)(((long long)MX * MY * MZ + 7) / 8);
@@ -1453,7 +1467,7 @@ lbm_status spectral_bwd(lbm_no* n, int l, const float* dz, float* dh, int parts)
     MixDims md{B, W, MX, MY, MZ};
     const unsigned mix_grid = (unsigned)(((long long)MX * MY * MZ + 7) / 8);
     if (mix32(n, n->params + n->oWm[l]) && mix32(n, n->grads + n->oWm[l])) {
-        // the gradient buffer was zeroed by backward() and this is the only writer of the block
+        // this is the only writer of the block of the gradient
         launch_pdl(k_mix_bwd_w32, mix_grid, 256, 0, n->stream, n->dyh, n->Xh[l], md, n->grads + n->oWm[l], 0);
         NCK(n, cudaGetLastError(), "mix dW");
         launch_pdl(k_mix_bwd_x32, mix_grid, 256, MIX_SMAT, n->stream, n->dyh, n->params + n->oWm[l], md, n->yh);
@@ -1517,9 +1531,10 @@ lbm_status forward(lbm_no* n, int B, const float* in, float* out) {
                                                     n->hb[0]);
     NCK(n, cudaGetLastError(), "lift");
     int parts = 0;
+    launch_pdl(k_keep_maps, dim3(grid_for((long long)W * W), n->L), 256, 0, n->stream, n->params + n->oWc[0], n->params + n->obc[0],
+               n->L > 1 ? n->oWc[1] - n->oWc[0] : 0LL, n->wcb, n->bkeep, W);
+    NCK(n, cudaGetLastError(), "keep maps");
     for (int l = 0; l < n->L; ++l) {
-        launch_pdl(k_keep_map, grid_for((long long)W * W), 256, 0, n->stream, n->params + n->oWc[l], n->params + n->obc[l],
-                   n->wcb + (long long)l * W * W, n->bkeep + l * W, W);
         st = l == 0 ? spectral_fwd(n, l, n->h0, nullptr, 0, n->z[l], 0)
                     : spectral_fwd(n, l, n->z[l - 1], rowv ? n->bkeep + (l - 1) * W : nullptr, 1, n->z[l], parts);
         if (st) return st;
@@ -1539,9 +1554,8 @@ lbm_status forward(lbm_no* n, int B, const float* in, float* out) {
         NCK(n, cudaGetLastError(), "bias act");
     }
     if (rowv && n->Co <= VEC_CH && (reinterpret_cast<uintptr_t>(out) & 15u) == 0)
-        launch_pdl(k_project_v, grid_rows(S, B), 256, 0, n->stream, n->z[n->L - 1],
-                   n->last_pending ? n->bkeep + (n->L - 1) * W : nullptr, n->params + n->oQ, n->params + n->oq, W, n->Co, S,
-                   out);
+        launch_pdl(n->last_pending ? k_project_v<4, true> : n->Co == 4 ? k_project_v<4, false> : k_project_v<0, false>, grid_rows(S, B), 256,
+                   0, n->stream, n->z[n->L - 1], n->bkeep + (n->L - 1) * W, n->params + n->oQ, n->params + n->oq, W, n->Co, S, out);
     else
         launch_pdl(k_project, grid_for((long long)B * n->Co * S), 256, 0, n->stream, n->z[n->L - 1], n->params + n->oQ,
                                                                             n->params + n->oq, B, W, n->Co, S, out);
@@ -1553,7 +1567,16 @@ lbm_status forward(lbm_no* n, int B, const float* in, float* out) {
 lbm_status backward(lbm_no* n, const float* dout) {
     const int B = n->B, W = n->W, L = n->L;
     const long long S = n->S, tot = (long long)B * W * S;
-    NCK(n, cudaMemsetAsync(n->grads, 0, sizeof(float) * n->nparam, n->stream), "zero grads");
+    // zero what is accumulated: everything, or, where the mixing kernels write the mode matrices' gradients
+    // (nearly all of the vector: 226 MB at 12 modes, width 32), the dense maps between them
+    bool modes_written = true;
+    for (int l = 0; l < L; ++l) modes_written = modes_written && mix32(n, n->params + n->oWm[l]) && mix32(n, n->grads + n->oWm[l]);
+    if (modes_written) {
+        launch_pdl(k_zero_dense, L + 1, 256, 0, n->stream, n->grads, n->oWm[0], n->oWc[0], L > 1 ? n->oWm[1] - n->oWm[0] : 0LL, L, n->nparam);
+        NCK(n, cudaGetLastError(), "zero grads");
+    } else {
+        NCK(n, cudaMemsetAsync(n->grads, 0, sizeof(float) * n->nparam, n->stream), "zero grads");
+    }
     // projection
     NCK(n, add_last_bias(n, dout), "last bias");
     NCK(n, reduce_bs(n, dout, n->z[L - 1], n->Co, W, n->grads + n->oQ, n->last_pending ? n->bkeep + (L - 1) * W : nullptr),
@@ -1613,7 +1636,7 @@ lbm_status backward(lbm_no* n, const float* dout) {
         NCK(n, gemm(n, (int)S, W, W, B, n->dzb, 1, S, (long long)W * S, n->wcb + (long long)l * W * W, W, 1, 0, n->dh2, 1, S,
                     (long long)W * S, 0, 0),
             "conv dX");
-        lbm_status st = spectral_bwd(n, l, n->dz, n->dh2, parts);
+        lbm_status st = spectral_bwd(n, l, parts && l == L - 1 ? n->dh : n->dz, n->dh2, parts);
         if (st) return st;
         std::swap(n->dh, n->dh2);
     }
@@ -1797,7 +1820,8 @@ lbm_status step_body(lbm_no* n, int batch) {
     if (st) return st;
     const long long cnt = (long long)batch * n->Co * n->S;
     NCK(n, cudaMemsetAsync(n->loss_d, 0, sizeof(double), n->stream), "loss reset");
-    launch_pdl(k_mse, grid_for(cnt), 256, 0, n->stream, out, n->tgt, cnt, n->dout, n->loss_d);
+    // few blocks: each ends in an FP64 atomic on the loss (4864 of them took 44 us)
+    launch_pdl(k_mse, std::min(grid_for(cnt), 152u * 4), 256, 0, n->stream, out, n->tgt, cnt, n->dout, n->loss_d);
     NCK(n, cudaGetLastError(), "loss");
     st = backward(n, n->dout);
     if (st) return st;
