@@ -28,6 +28,7 @@
 #include <string.h>
 
 #include "../../include/cmlbm.h"
+#include "no_act.cuh"
 #include "no_gemm.h"
 #include "pdl.cuh"
 
@@ -886,6 +887,239 @@ __global__ void __launch_bounds__(Shape<GROUPS>::threads, Shape<GROUPS>::blocks_
     }
 }
 
+// ---------------------------------------------------------------------------------------------
+// The 1x1 map with the activation (launch_map_act).  Apart, the map added to z through the copy engine's
+// reduce-add (50 us at 64^3, batch 4, HBM-bound) and the activation read z again (46 us, bound by the
+// issue of erff: 34 instructions per value); together 77 us.  The epilogue warps load the next tile's z
+// ahead of the activation of the current one.  Bound by that arithmetic on eight warps per SM (2 blocks: three
+// spill and take 91 us) and by the last round of its 1,024 runs of eight tiles on 304 blocks.
+//   Roles as in k_gemm_bf16_tma: warp 0 loads tiles of 128 positions x 32 channels of h (M-major), warp 1
+// issues two tcgen05.mma (K = 16, N = 32) per tile against the resident weights, warps 2-5 drain.  A lane
+// reads its accumulator row (one position, 32 channels); the warp turns the 32 x 32 block through shared
+// memory so that a lane holds four consecutive positions of eight channels: 16-byte accesses to z.
+//   Tiles: block `super` u takes the tiles at positions p 8192 + j 1024 + i 128, j = 0..7, (b, p, i) from u,
+// one after the other, and each lane sums the values of its positions over j in FP32 before the FP64 sum
+// over lanes: the order in which k_bias_act_v's threads sum, so the means come out the same.
+constexpr int MAP_STAGES = 6, MAP_A_BYTES = 2 * ATOM * MAP_W * 2, MAP_B_BYTES = MAP_W * 128;
+constexpr int MAP_THREADS = 192, MAP_BLOCKS = 2;
+constexpr int MAP_SMEM = SMEM_ALIGN + MAP_B_BYTES + MAP_STAGES * MAP_A_BYTES + 4 * 32 * 32 * 4;
+
+struct MapArgs {
+    float* z;
+    const float* bias;
+    __nv_bfloat16* hb;
+    double* part;
+    long long S;
+    int chunks;  // of 8192 positions per row
+    int supers;  // B chunks 8
+    int three;   // the map of h carries the batch
+    unsigned int* err;
+};
+
+__global__ void __launch_bounds__(MAP_THREADS, MAP_BLOCKS)
+    k_map_act(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, MapArgs g) {
+    constexpr uint32_t TMEM_COLS = 2 * MAP_W;
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t full[MAP_STAGES], empty[MAP_STAGES], tfull[2], tempty[2], drain, bres;
+    __shared__ uint32_t tmem_base;
+    __shared__ volatile int abort_flag;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t res = (smem_u32(smem_raw) + SMEM_ALIGN - 1) & ~(uint32_t)(SMEM_ALIGN - 1);
+    const uint32_t ring = res + MAP_B_BYTES, turn = ring + MAP_STAGES * MAP_A_BYTES;
+
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&tmem_base)),
+                     "r"(TMEM_COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    if (tid == 0) {
+        abort_flag = 0;
+        for (int s = 0; s < MAP_STAGES; ++s) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&full[s])) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&empty[s])) : "memory");
+        }
+        for (int a = 0; a < 2; ++a) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&tfull[a])) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;\n" ::"r"(smem_u32(&tempty[a])) : "memory");
+        }
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&drain)) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&bres)) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(&map_a)) : "memory");
+        asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(&map_b)) : "memory");
+    }
+    pdl_wait();
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    const uint32_t tmem = tmem_base;
+
+    // first position of tile j of super u; its sample and chunk
+    auto tile = [&](int u, int j, int& b, int& p, int& i) {
+        const int bp = u >> 3;
+        i = u & 7;
+        b = bp / g.chunks;
+        p = bp - b * g.chunks;
+        return p * 8192 + j * 1024 + i * 128;  // S < 2^31 - 8192 (launch_map_act)
+    };
+
+    if (warp == 0 && lane == 0) {
+        // ---- TMA producer
+        const uint32_t wbar = smem_u32(&bres);
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(wbar), "r"(MAP_B_BYTES) : "memory");
+        tma_load(res, &map_b, 0, 0, 0, false, wbar);
+        uint32_t it = 0, s = 0, ph = 0;
+        for (int u = blockIdx.x; u < g.supers && !abort_flag; u += gridDim.x)
+            for (int j = 0; j < 8; ++j, ++it, s = (s + 1 == MAP_STAGES) ? (ph ^= 1u, 0u) : s + 1) {
+                int b, p, i;
+                const int m0 = tile(u, j, b, p, i);
+                if (m0 >= g.S) break;
+                if (!wait_or_abort(smem_u32(&empty[s]), ph ^ 1, &abort_flag)) {
+                    abort_flag = 1;
+                    break;
+                }
+                const uint32_t bar = smem_u32(&full[s]), sa = ring + s * MAP_A_BYTES;
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(MAP_A_BYTES) : "memory");
+                tma_load(sa, &map_a, m0, 0, b, g.three, bar);
+                tma_load(sa + MAP_A_BYTES / 2, &map_a, m0 + ATOM, 0, b, g.three, bar);
+            }
+        // every copy issued has landed before the block can exit
+        volatile int never = 0;
+        for (uint32_t j = 0; j < MAP_STAGES && j < it; ++j) {
+            const uint32_t last = it - 1 - ((it - 1 + MAP_STAGES - j) % MAP_STAGES);
+            if (!wait_or_abort(smem_u32(&full[j]), (last / MAP_STAGES) & 1, &never)) atomicOr(g.err, 1u);
+        }
+        if (!wait_or_abort(wbar, 0, &never)) atomicOr(g.err, 1u);
+    } else if (warp == 1 && lane == 0) {
+        // ---- MMA issuer
+        const uint32_t idesc = instr_desc(TM, MAP_W) | (1u << 15);  // A M-major
+        bool ok = wait_or_abort(smem_u32(&bres), 0, &abort_flag);
+        if (!ok) abort_flag = 1;
+        uint32_t s = 0, ph = 0, lt = 0;
+        for (int u = blockIdx.x; ok && u < g.supers && !abort_flag; u += gridDim.x)
+            for (int j = 0; j < 8; ++j, ++lt, s = (s + 1 == MAP_STAGES) ? (ph ^= 1u, 0u) : s + 1) {
+                int b, p, i;
+                if (tile(u, j, b, p, i) >= g.S) break;
+                const uint32_t a = lt & 1, ause = lt >> 1;
+                if (!wait_or_abort(smem_u32(&tempty[a]), (ause & 1) ^ 1, &abort_flag) ||
+                    !wait_or_abort(smem_u32(&full[s]), ph, &abort_flag)) {
+                    ok = false;
+                    abort_flag = 1;
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                const uint32_t sa = ring + s * MAP_A_BYTES, d = tmem + a * MAP_W;
+#pragma unroll
+                for (int k = 0; k < MAP_W / 16; ++k)
+                    asm volatile(
+                        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+                        "l"(sw128_desc(sa + 2048u * k, MAP_A_BYTES / 2, 1024)), "l"(sw128_desc(res + 32u * k, 16, 1024)), "r"(idesc),
+                        "r"(k > 0 ? 1u : 0u)
+                        : "memory");
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(smem_u32(&empty[s]))
+                             : "memory");
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(smem_u32(&tfull[a]))
+                             : "memory");
+            }
+        // no MMA of this thread may still run when the tensor memory is freed
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(smem_u32(&drain)) : "memory");
+        volatile int never = 0;
+        if (!wait_or_abort(smem_u32(&drain), 0, &never)) atomicOr(g.err, 1u);
+    } else if (warp >= 2) {
+        // ---- epilogue: lane = four positions (4 (lane mod 8) ...) of channels lane / 8 + 4 k, k = 0..7
+        const int q = warp & 3, c0 = lane >> 3, x0 = (lane & 7) * 4;
+        const uint32_t buf = turn + (uint32_t)(warp - 2) * 4096;
+        float bo[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) bo[k] = g.bias[c0 + 4 * k];
+        // offset of the lane's first values of a tile, -1 past the row's end
+        auto offset = [&](int u, int j) -> long long {
+            int b, p, i;
+            if (u >= g.supers) return -1;
+            const int m0 = tile(u, j, b, p, i);
+            return m0 < g.S ? ((long long)b * MAP_W + c0) * g.S + m0 + q * 32 + x0 : -1;
+        };
+        uint32_t lt = 0;
+        long long at = offset(blockIdx.x, 0), held = -1;  // the tile to do, and the one whose z is in old
+        float4 old[8];
+        auto load = [&](long long o) {
+            held = o;
+            if (o >= 0)
+#pragma unroll
+                for (int k = 0; k < 8; ++k) old[k] = *reinterpret_cast<const float4*>(g.z + o + 4 * k * g.S);
+        };
+        for (int u = blockIdx.x; u < g.supers && !abort_flag; u += gridDim.x) {
+            float sum[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) sum[k] = 0.0f;
+            if (held != at) load(at);
+            for (int j = 0; at >= 0; ++j, ++lt) {
+                const uint32_t a = lt & 1, ause = lt >> 1;
+                if (!wait_or_abort(smem_u32(&tfull[a]), ause & 1, &abort_flag)) {
+                    abort_flag = 1;
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + a * MAP_W;
+                __syncwarp();  // the last tile's reads of buf are done
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf) {
+                    uint32_t v[16];
+                    tmem_ld16(taddr + 16 * hf, v);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+                    for (int c = 0; c < 16; ++c)
+                        asm volatile("st.shared.b32 [%0], %1;\n" ::"r"(buf + (uint32_t)((16 * hf + c) * 128 + lane * 4)), "r"(v[c])
+                                     : "memory");
+                }
+                asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+                __syncwarp();
+                if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(&tempty[a])) : "memory");
+                // this tile's z + map, then the loads of the next tile's z ahead of this one's activation
+                float4 w[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];\n"
+                                 : "=f"(w[k].x), "=f"(w[k].y), "=f"(w[k].z), "=f"(w[k].w)
+                                 : "r"(buf + (uint32_t)((c0 + 4 * k) * 128 + x0 * 4))
+                                 : "memory");
+                    w[k] = make_float4(old[k].x + w[k].x, old[k].y + w[k].y, old[k].z + w[k].z, old[k].w + w[k].w);
+                }
+                const long long here = at, next = j < 7 ? offset(u, j + 1) : -1;
+                load(next >= 0 ? next : offset(u + (int)gridDim.x, 0));
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    *reinterpret_cast<float4*>(g.z + here + 4 * k * g.S) = w[k];
+                    const float4 h = make_float4(gelu(w[k].x + bo[k]), gelu(w[k].y + bo[k]), gelu(w[k].z + bo[k]), gelu(w[k].w + bo[k]));
+                    *reinterpret_cast<uint2*>(g.hb + here + 4 * k * g.S) = pack_bf16x4(h);
+                    sum[k] += h.x + h.y + h.z + h.w;
+                }
+                at = next;
+            }
+            at = offset(u + (int)gridDim.x, 0);
+            const int bp = u >> 3, b = bp / g.chunks, p = bp - b * g.chunks;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                double d = sum[k];
+#pragma unroll
+                for (int off = 4; off > 0; off >>= 1) d += __shfl_down_sync(0xFFFFFFFFu, d, off, 8);
+                if ((lane & 7) == 0)
+                    g.part[((long long)b * MAP_W + c0 + 4 * k) * (g.chunks * 32) + p * 32 + (u & 7) * 4 + q] = d;
+            }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    if (tid == 0 && abort_flag) atomicOr(g.err, 1u);
+    if (warp == 1) {
+        __syncwarp();
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+    }
+}
+
 }  // namespace tma
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -1152,6 +1386,31 @@ __global__ void k_gemm_zero_c(GemmArgs g, int batch) {
 }
 
 }  // namespace
+
+cudaError_t launch_map_act(const __nv_bfloat16* h, const __nv_bfloat16* Wc, const float* bias, int B, long long S, float* z,
+                           __nv_bfloat16* hb, double* part, unsigned int* err, cudaStream_t st) {
+    if (S % 128 != 0 || S >= (1LL << 31) - 8192 || !aligned16(z) || !aligned16(hb)) return cudaErrorNotSupported;
+    CUtensorMap ma, mb;
+    int mn, three, mn_b, three_b;
+    if (!operand_map(&ma, h, (int)S, MAP_W, B, 1, S, (long long)MAP_W * S, TM, 1, MAP_W, &mn, &three) || !mn) return cudaErrorNotSupported;
+    if (!operand_map(&mb, Wc, MAP_W, MAP_W, 1, MAP_W, 1, 0, MAP_W, 1, TK, &mn_b, &three_b) || mn_b) return cudaErrorNotSupported;
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(tma::k_map_act, cudaFuncAttributeMaxDynamicSharedMemorySize, tma::MAP_SMEM);
+    if (attr != cudaSuccess) return attr;
+    static const int sms = sm_count();
+    tma::MapArgs a;
+    a.z = z;
+    a.bias = bias;
+    a.hb = hb;
+    a.part = part;
+    a.S = S;
+    a.chunks = map_parts(S) / 32;
+    if ((long long)B * a.chunks * 8 >= (1LL << 31)) return cudaErrorNotSupported;
+    a.supers = B * a.chunks * 8;
+    a.three = three;
+    a.err = err;
+    return launch_pdl(tma::k_map_act, std::min(a.supers, sms * tma::MAP_BLOCKS), tma::MAP_THREADS, tma::MAP_SMEM, st, ma, mb, a);
+}
 
 cudaError_t launch_gemm_bf16(const GemmArgs& g_in, int batch, cudaStream_t st) {
     if (g_in.M <= 0 || g_in.N <= 0 || g_in.K < 0 || batch <= 0) return cudaErrorInvalidValue;

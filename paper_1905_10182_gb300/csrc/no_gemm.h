@@ -37,4 +37,13 @@ struct GemmArgs {
 
 cudaError_t launch_gemm_bf16(const GemmArgs& g, int batch, cudaStream_t st);
 
+// The 1x1 map of a hidden layer of width 32 with what follows it, in one pass over the activations:
+//   z[b][o][s] += sum_c Wc[o][c] h[b][c][s];   v = act(z + bias[o]);   hb[b][o][s] = bf16(v)
+// and the sums of v per row: part[(b 32 + o) map_parts(S) + k], the row's parts in FP64.  h, Wc and hb BF16,
+// act = GELU.  cudaErrorNotSupported where the kernel does not apply (S no multiple of 128, alignment).
+constexpr int MAP_W = 32;
+inline int map_parts(long long S) { return (int)((S + 8191) / 8192) * 32; }
+cudaError_t launch_map_act(const __nv_bfloat16* h, const __nv_bfloat16* Wc, const float* bias, int B, long long S, float* z,
+                           __nv_bfloat16* hb, double* part, unsigned int* err, cudaStream_t st);
+
 }  // namespace cmlbm

@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "../../include/cmlbm.h"
+#include "no_act.cuh"
 #include "no_gemm.h"
 #include "pdl.cuh"
 
@@ -89,7 +90,6 @@ __global__ void k_project_bwd_x(const float* __restrict__ dout, const float* __r
     }
 }
 
-__device__ __forceinline__ float gelu(float x) { return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f)); }
 __device__ __forceinline__ float gelu_grad(float x) {
     const float cdf = 0.5f * (1.0f + erff(x * 0.70710678118654752f));
     const float pdf = 0.39894228040143268f * expf(-0.5f * x * x);
@@ -138,11 +138,6 @@ __global__ void k_act_bwd(const float* __restrict__ dh, const float* __restrict_
 // numbers.  The mean's mode is added back in FP32 (k_add_dc).  Three passes: partial sums over
 // CENTER_PARTS chunks per channel (FP32 per thread, FP64 per block), the means in a fixed order,
 // then the element-wise centring.
-__device__ __forceinline__ uint2 pack_bf16x4(float4 v) {
-    const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
-    return make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
-}
-
 constexpr int CENTER_PARTS = 16;
 
 __global__ void __launch_bounds__(256) k_center_partials(const float* __restrict__ src, long long S, int use_gelu,
@@ -1538,6 +1533,16 @@ lbm_status forward(lbm_no* n, int B, const float* in, float* out) {
         st = l == 0 ? spectral_fwd(n, l, n->h0, nullptr, 0, n->z[l], 0)
                     : spectral_fwd(n, l, n->z[l - 1], rowv ? n->bkeep + (l - 1) * W : nullptr, 1, n->z[l], parts);
         if (st) return st;
+        // a hidden layer's map and activation in one pass, which also leaves the next layer's centring sums
+        if (l < n->L - 1 && rowv && W == MAP_W) {
+            const cudaError_t e = launch_map_act(n->hb[l], n->wcb + (long long)l * W * W, n->bkeep + l * W, B, S, n->z[l], n->hb[l + 1],
+                                                 n->cpart, n->gemm_err, n->stream);
+            if (e == cudaSuccess) {
+                parts = map_parts(S);
+                continue;
+            }
+            if (e != cudaErrorNotSupported) NCK(n, e, "map and activation");
+        }
         // 1x1 conv accumulated onto the spectral output: z[b][o][s] += sum_c Wc[o][c] h[b][c][s]
         NCK(n, gemm(n, (int)S, W, W, B, n->hb[l], 1, S, (long long)W * S, n->wcb + (long long)l * W * W, 1, W, 0, n->z[l], 1,
                     S, (long long)W * S, 0, 1),
@@ -1754,7 +1759,7 @@ lbm_status lbm_no_create(int D, int W, int modes, int L, int Ci, int Co, int max
     alloc((void**)&n->hs, sizeof(bf16) * act);
     alloc((void**)&n->hmean, sizeof(float) * maxB * W);
     n->rowparts = n->S % 4 == 0 ? row_blocks(n->S) : 0;
-    alloc((void**)&n->cpart, sizeof(double) * maxB * W * std::max(CENTER_PARTS, n->rowparts));
+    alloc((void**)&n->cpart, sizeof(double) * maxB * W * std::max(CENTER_PARTS, W == MAP_W ? map_parts(S) : n->rowparts));
     alloc((void**)&n->red, sizeof(float) * std::max(REDUCE_CHUNKS, PAIR_CHUNKS) * std::max(std::max(W * Ci, Co * W), W));
     alloc((void**)&n->part, sizeof(float) * maxB * ((S + KSPLIT - 1) / KSPLIT + 1) * W * W);
     alloc((void**)&n->dout, sizeof(float) * maxB * Co * S);
