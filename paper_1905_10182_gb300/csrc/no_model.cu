@@ -526,19 +526,21 @@ __device__ __forceinline__ void unstage_block(bf16* __restrict__ out, const MixD
     __syncthreads();
 }
 
-// A mode's 32 x 32 complex matrix (8 KB, rows o of 64 floats) into shared memory rows padded to
-// MIX_PITCH floats, by the warp with cp.async (16 bytes per lane and copy, coalesced 512-byte
-// reads): lanes reading one 16-byte chunk of 8 different rows, or 32 consecutive 8-byte words of
-// one row, then meet no bank conflict.
-constexpr int MIX_PITCH = 2 * MIX_W + 4;
-constexpr int MIX_SMAT = MIX_MODES * MIX_W * MIX_PITCH * (int)sizeof(float);  // 69,632 B of dynamic shared memory
+// A mode's 32 x 32 complex matrix (8 KB, rows o of 64 floats) into shared memory, by the warp with
+// cp.async (16 bytes per lane and copy, coalesced 512-byte reads): 16-byte chunk c4 of row o at place
+// c4 ^ (o mod 8) of the row, so that lanes reading one chunk of 8 different rows, or 32 consecutive 8-byte
+// words of one row, meet no bank conflict.  With rows padded instead, and the outputs staged apart from
+// the inputs, two blocks fit an SM; now three do.
+constexpr int MIX_PITCH = 2 * MIX_W;
+constexpr int MIX_SMAT = MIX_MODES * MIX_W * MIX_PITCH * (int)sizeof(float);  // 65,536 B of dynamic shared memory
+__device__ __forceinline__ int mix_chunk(int o, int c4) { return o * MIX_PITCH + ((c4 ^ (o & 7)) << 2); }
 
 __device__ __forceinline__ void load_mode_matrix(float* sw, const float* __restrict__ w, int lane) {
     const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(sw));
 #pragma unroll
     for (int i = 0; i < MIX_W / 2; ++i) {
         const int q = i * 32 + lane, o = q >> 4, c4 = q & 15;  // 16-byte chunk c4 of row o
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(base + (uint32_t)((o * MIX_PITCH + c4 * 4) * 4)),
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(base + (uint32_t)(mix_chunk(o, c4) * 4)),
                      "l"(w + q * 4)
                      : "memory");
     }
@@ -555,7 +557,7 @@ __global__ void __launch_bounds__(256) k_mix_fwd32(const float* __restrict__ X, 
     pdl_wait();
     extern __shared__ __align__(16) float smat[];  // MIX_MODES matrices, MIX_W rows of MIX_PITCH
     __shared__ __align__(16) float sbuf[MIX_MODES][MIX_BUF];
-    __shared__ __align__(16) bf16 so[MIX_S * MIX_W * 2][MIX_MODES];
+    bf16 (*so)[MIX_MODES] = reinterpret_cast<bf16 (*)[MIX_MODES]>(sbuf);  // the outputs take the inputs' place
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long m = (long long)blockIdx.x * MIX_MODES + warp;  // modes fill whole blocks
     int kx, ky, kz;
@@ -563,7 +565,6 @@ __global__ void __launch_bounds__(256) k_mix_fwd32(const float* __restrict__ X, 
     const int kz0 = kz - warp;
     float* sw = smat + warp * MIX_W * MIX_PITCH;
     load_mode_matrix(sw, Wm + widx(d, kx, ky, kz, 0, 0), lane);
-    const float* wrow = sw + lane * MIX_PITCH;  // row o = lane
     const float* sv = sbuf[warp];
     for (int b0 = 0; b0 < d.B; b0 += MIX_S) {
         const int nb = min(MIX_S, d.B - b0);
@@ -574,8 +575,8 @@ __global__ void __launch_bounds__(256) k_mix_fwd32(const float* __restrict__ X, 
         for (int j = 0; j < MIX_S; ++j) yr[j] = yi[j] = 0.0f;
 #pragma unroll
         for (int c = 0; c < MIX_W; ++c) {
-            // two channels per 16-byte read (conflict-free across 8 lanes with the padded rows)
-            const float4 wq = *reinterpret_cast<const float4*>(wrow + 4 * (c >> 1));
+            // two channels per 16-byte read
+            const float4 wq = *reinterpret_cast<const float4*>(sw + mix_chunk(lane, c >> 1));  // row o = lane
             const float wr = (c & 1) ? wq.z : wq.x, wi = (c & 1) ? wq.w : wq.y;
             const float4 x01 = *reinterpret_cast<const float4*>(sv + c * 2 * MIX_S);
             const float4 x23 = *reinterpret_cast<const float4*>(sv + c * 2 * MIX_S + 4);
@@ -586,6 +587,7 @@ __global__ void __launch_bounds__(256) k_mix_fwd32(const float* __restrict__ X, 
                 yi[j] += wr * xi[j] + wi * xr[j];
             }
         }
+        __syncthreads();
 #pragma unroll
         for (int j = 0; j < MIX_S; ++j) {
             so[(j * MIX_W + lane) * 2][warp] = __float2bfloat16(yr[j]);
@@ -600,7 +602,7 @@ __global__ void __launch_bounds__(256) k_mix_bwd_x32(const float* __restrict__ d
     pdl_wait();
     extern __shared__ __align__(16) float smat[];  // MIX_MODES matrices, MIX_W rows of MIX_PITCH
     __shared__ __align__(16) float sbuf[MIX_MODES][MIX_BUF];
-    __shared__ __align__(16) bf16 so[MIX_S * MIX_W * 2][MIX_MODES];
+    bf16 (*so)[MIX_MODES] = reinterpret_cast<bf16 (*)[MIX_MODES]>(sbuf);  // the outputs take the inputs' place
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long m = (long long)blockIdx.x * MIX_MODES + warp;
     int kx, ky, kz;
@@ -608,7 +610,6 @@ __global__ void __launch_bounds__(256) k_mix_bwd_x32(const float* __restrict__ d
     const int kz0 = kz - warp;
     float* sw = smat + warp * MIX_W * MIX_PITCH;
     load_mode_matrix(sw, Wm + widx(d, kx, ky, kz, 0, 0), lane);
-    const float* wcol = sw + 2 * lane;  // column c = lane: W[o][c] at wcol[o MIX_PITCH]
     const float* sv = sbuf[warp];
     for (int b0 = 0; b0 < d.B; b0 += MIX_S) {
         const int nb = min(MIX_S, d.B - b0);
@@ -619,7 +620,7 @@ __global__ void __launch_bounds__(256) k_mix_bwd_x32(const float* __restrict__ d
         for (int j = 0; j < MIX_S; ++j) xr[j] = xi[j] = 0.0f;
 #pragma unroll
         for (int o = 0; o < MIX_W; ++o) {
-            const float2 wo = *reinterpret_cast<const float2*>(wcol + o * MIX_PITCH);
+            const float2 wo = *reinterpret_cast<const float2*>(sw + mix_chunk(o, lane >> 1) + 2 * (lane & 1));  // column c = lane
             const float wr = wo.x, wi = wo.y;
             const float4 y01 = *reinterpret_cast<const float4*>(sv + o * 2 * MIX_S);
             const float4 y23 = *reinterpret_cast<const float4*>(sv + o * 2 * MIX_S + 4);
@@ -630,6 +631,7 @@ __global__ void __launch_bounds__(256) k_mix_bwd_x32(const float* __restrict__ d
                 xi[j] += -wi * yr[j] + wr * yi[j];
             }
         }
+        __syncthreads();
 #pragma unroll
         for (int j = 0; j < MIX_S; ++j) {
             so[(j * MIX_W + lane) * 2][warp] = __float2bfloat16(xr[j]);
