@@ -148,6 +148,7 @@ KParams make_params(const lbm_ctx* c) {
     // population store does not fit in L2 (a store that fits is read from L2 anyway)
     const double store_bytes = 27.0 * (double)c->N * (double)elem_size(c->storage);
     p.pf = store_bytes > (double)c->l2 ? 2 * c->sms : 0;
+    p.rev = 2.0 * store_bytes > (double)c->l2;
     set_numbering(p);
     return p;
 }

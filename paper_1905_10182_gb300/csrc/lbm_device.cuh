@@ -113,6 +113,7 @@ struct KParams {
     int ho;                // 1: second-order Hermite truncation of f^eq and/or F_i (models M4, M5)
     float ce, cf;          // weights of hermite2_correction (1 / 0 and 1/2 / 0)
     int pf;                // stream-collide: L2 prefetch distance in blocks of the launch (0: off)
+    int rev;               // odd steps walk the grid backwards, see step_backwards
     FastDiv pf_gx, pf_ny;  // division by a row's blocks and by the rows of a plane
     uint32_t nodes;        // active nodes (nx ny planes), below 2^31
     FastDiv dnx;           // division by nx
@@ -144,6 +145,19 @@ __device__ __forceinline__ bool node_of(const KParams& p, int& x, int& y, int& z
     return x < p.nx;
 }
 
+// Odd steps of a large store (p.rev) walk the grid backwards: each step then begins where the step before it
+// ended, with that part of the store still in the 129 MB of L2, to be read and overwritten without HBM.  Per
+// step, forwards -> backwards: FP32 96^3 25.7 -> 22.5 us, 112^3 50.1 -> 41.2, 128^3 69.1 -> 64.9, 256^3
+// 526.5 -> 522.6; FP16 128^3 39.8 -> 36.0, 256^3 294.6 -> 292.5; 128^3 with a magnetic field 133.5 -> 126.5.
+// A store that L2 holds with room to spare has nothing to gain and reads a little more from the far half of
+// L2: FP32 32^3 2.70 -> 2.78 us, 64^3 7.56 -> 7.63, so p.rev is 0 up to half of L2 (FP16 96^3 and 112^3, 48
+// and 76 MB, are the same both ways).  Not with the Shan-Chen force, whose psi pass between the steps walks
+// backwards itself.
+template <bool ODD, int FK>
+__device__ __forceinline__ bool step_backwards(const KParams& p) {
+    return ODD && FK != FK_SHAN_CHEN && p.rev;
+}
+
 // launch grid of node_of: the ghost planes of a z slab get no threads
 inline dim3 node_grid(const KParams& p, bool flat) {
     if (flat) return dim3((p.nodes + BLOCK_X - 1) / BLOCK_X);
@@ -163,18 +177,20 @@ inline void set_numbering(KParams& p) {
 // direction i = opp(k)); one thread per 128-byte line of them issues a prefetch.  This keeps more
 // DRAM requests in flight than the gathers alone, which are latency-bound at 16-20 warps per SM.
 template <typename S, bool ODD, bool FLAT>
-__device__ __forceinline__ void k1_prefetch(const KParams& p, const S* f) {
+__device__ __forceinline__ void k1_prefetch(const KParams& p, const S* f, bool rev) {
     constexpr uint32_t LPR = BLOCK_X * sizeof(S) / 128;  // lines per row segment
     const uint32_t t = threadIdx.x;
     if (t >= 27 * LPR) return;
     const uint32_t k = t / LPR, dx = (t - k * LPR) * (128 / sizeof(S));
+    // the block p.pf places on in launch order (below 0 wraps to past the end)
+    const uint32_t gx = gridDim.x, blocks = gx * gridDim.y * gridDim.z;
+    const uint32_t me = blockIdx.x + gx * (blockIdx.y + gridDim.y * blockIdx.z);
+    const uint32_t b = rev ? blocks - 1 - me - (uint32_t)p.pf : me + (uint32_t)p.pf;
+    if (b >= blocks) return;
     int xs, yk, zk;
     if (FLAT) {  // a segment that runs into the next row is taken to continue in place
-        if (!node_at(p, (blockIdx.x + (uint32_t)p.pf) * BLOCK_X + dx, xs, yk, zk)) return;
+        if (!node_at(p, b * BLOCK_X + dx, xs, yk, zk)) return;
     } else {
-        const uint32_t gx = gridDim.x;
-        const uint32_t b = blockIdx.x + gx * (blockIdx.y + gridDim.y * blockIdx.z) + (uint32_t)p.pf;
-        if (b >= gx * gridDim.y * gridDim.z) return;
         const uint32_t r = p.pf_gx.div(b);
         const uint32_t zb = p.pf_ny.div(r);
         yk = (int)(r - zb * (uint32_t)p.ny);

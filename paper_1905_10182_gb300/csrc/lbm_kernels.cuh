@@ -27,9 +27,10 @@ __device__ __forceinline__ void check_node(const KParams& p, const Macro& m) {
 template <typename S, bool ODD, bool LINKS, int FK, bool TRACE, bool HO, bool FLAT, bool OFF32>
 __global__ void __launch_bounds__(BLOCK_X, (sizeof(S) == 4 || ODD ? 4 : 5)) k_stream_collide(KParams p, S* __restrict__ f) {
     pdl_wait();
-    if (p.pf) k1_prefetch<S, ODD, FLAT>(p, f);
+    const bool rev = step_backwards<ODD, FK>(p);
+    if (p.pf) k1_prefetch<S, ODD, FLAT>(p, f, rev);
     int x, y, z;
-    if (!node_of<FLAT>(p, x, y, z)) return;
+    if (!node_of<FLAT>(p, x, y, z, rev)) return;
     const Nbr nb(x, y, z, p);
     uint32_t link = 0;
     if (LINKS) {

@@ -137,7 +137,7 @@ template <bool ODD, bool LINKS, bool FLAT>
 __global__ void __launch_bounds__(BLOCK_X, 5) k_mhd_step(KParams p, MhdArgs q, float* __restrict__ f) {
     pdl_wait();
     int x, y, z;
-    if (!node_of<FLAT>(p, x, y, z)) return;
+    if (!node_of<FLAT>(p, x, y, z, step_backwards<ODD, FK_CONST>(p))) return;
     const Nbr nb(x, y, z, p);
     const uint32_t link = LINKS ? p.links[nb.self()] : 0u;
     float h[21];
