@@ -305,8 +305,8 @@ def kernel_source_hash(batch=False):
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_1905_10182_gb300", "csrc")
     for name in sorted(os.listdir(csrc)):
-        if (batch and name in ("lbm_device.cuh", "lbm_batch.cu")) or (not batch and (
-                name in ("lbm_device.cuh", "lbm_kernels.cuh", "lbm_x2.cuh") or
+        if (batch and name in ("lbm_device.cuh", "lbm_vec.cuh", "lbm_batch.cu")) or (not batch and (
+                name in ("lbm_device.cuh", "lbm_vec.cuh", "lbm_kernels.cuh", "lbm_x2.cuh") or
                 (name.startswith("lbm_k_") and name.endswith(".cu")))):
             text = open(os.path.join(csrc, name), encoding="utf-8").read()
             text = re.sub(r"/\*.*?\*/", " ", text, flags=re.S)

@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <cstdint>
 
 #include "pdl.cuh"
 
@@ -11,8 +12,9 @@ namespace cmlbm {
 struct KParams;
 
 // A caller's array that the kernels may read or write where it lies: device memory of device `dev` (host,
-// managed and other devices' memory goes through a copy).
+// managed and other devices' memory, and floats off their 4-byte alignment, go through a copy).
 inline bool in_place(const void* p, int dev) {
+    if (reinterpret_cast<uintptr_t>(p) & 3) return false;
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();

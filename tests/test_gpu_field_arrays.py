@@ -61,3 +61,21 @@ def test_batch():
             fields.append(host)
         got.append(fields)
     assert all(np.array_equal(a, c) for a, c in zip(*got))
+
+
+def test_unaligned_device_arrays():
+    """Device pointers off the 4-byte alignment are copied."""
+    L, (nx, ny, nz) = nat.lib(), SHAPES[0]
+    N, host = nx * ny * nz, _fields(*SHAPES[0])
+    raw = torch.zeros(4, 4 * N + 4, dtype=torch.uint8, device="cuda")
+    raw[:, 2:-2] = torch.stack([torch.from_numpy(f.reshape(-1).view(np.uint8)) for f in host]).cuda()
+    s, ref = Solver(nx, ny, nz, nu=0.04), Solver(nx, ny, nz, nu=0.04)
+    b = BatchSolver([dict(nx=nx, ny=ny, nz=nz, nu=0.04)])
+    ref.set_state(*host)
+    for put, get, h in ((L.lbm_set_state, L.lbm_macroscopic, (s._h,)), (L.lbm_batch_set_state, L.lbm_batch_macroscopic, (b._h, 0))):
+        assert put(*h, *(raw[k].data_ptr() + 2 for k in range(4))) == 0
+        out = torch.zeros_like(raw)
+        assert get(*h, *(out[k].data_ptr() + 2 for k in range(4))) == 0
+        out = out.cpu().numpy()
+        assert np.array_equal(out[:, 2:-2].copy().view(np.float32).reshape(4, nz, ny, nx), np.stack(ref.macroscopic()))
+        assert not out[:, :2].any() and not out[:, -2:].any()
