@@ -113,11 +113,11 @@ struct KParams {
     int ho;                // 1: second-order Hermite truncation of f^eq and/or F_i (models M4, M5)
     float ce, cf;          // weights of hermite2_correction (1 / 0 and 1/2 / 0)
     int pf;                // stream-collide: L2 prefetch distance in blocks of the launch (0: off)
-    int rev;               // odd steps walk the grid backwards, see step_backwards
     FastDiv pf_gx, pf_ny;  // division by a row's blocks and by the rows of a plane
     uint32_t nodes;        // active nodes (nx ny planes), below 2^31
     FastDiv dnx;           // division by nx
     int flat;              // node numbering of the kernels with one thread per node, see node_of
+    int rev;               // odd steps walk the grid backwards, see can_reverse
 };
 
 // One thread per node.  FLAT = false: a row of blocks for each row of the grid (blockIdx = x block, y, z;
@@ -152,11 +152,10 @@ __device__ __forceinline__ bool node_of(const KParams& p, int& x, int& y, int& z
 // A store that L2 holds with room to spare has nothing to gain and reads a little more from the far half of
 // L2: FP32 32^3 2.70 -> 2.78 us, 64^3 7.56 -> 7.63, so p.rev is 0 up to half of L2 (FP16 96^3 and 112^3, 48
 // and 76 MB, are the same both ways).  Not with the Shan-Chen force, whose psi pass between the steps walks
-// backwards itself.
+// backwards itself.  An instantiation of its own: chosen inside the kernel it cost every odd step (32^3 2.70
+// -> 2.76 us, 512^3 0.2 %).
 template <bool ODD, int FK>
-__device__ __forceinline__ bool step_backwards(const KParams& p) {
-    return ODD && FK != FK_SHAN_CHEN && p.rev;
-}
+constexpr bool can_reverse = ODD && FK != FK_SHAN_CHEN;
 
 // launch grid of node_of: the ghost planes of a z slab get no threads
 inline dim3 node_grid(const KParams& p, bool flat) {
@@ -176,8 +175,8 @@ inline void set_numbering(KParams& p) {
 // BLOCK_X nodes (on an odd step plane k comes from the row shifted by c_k, the source x - c_i of
 // direction i = opp(k)); one thread per 128-byte line of them issues a prefetch.  This keeps more
 // DRAM requests in flight than the gathers alone, which are latency-bound at 16-20 warps per SM.
-template <typename S, bool ODD, bool FLAT>
-__device__ __forceinline__ void k1_prefetch(const KParams& p, const S* f, bool rev) {
+template <typename S, bool ODD, bool FLAT, bool REV>
+__device__ __forceinline__ void k1_prefetch(const KParams& p, const S* f) {
     constexpr uint32_t LPR = BLOCK_X * sizeof(S) / 128;  // lines per row segment
     const uint32_t t = threadIdx.x;
     if (t >= 27 * LPR) return;
@@ -185,7 +184,7 @@ __device__ __forceinline__ void k1_prefetch(const KParams& p, const S* f, bool r
     // the block p.pf places on in launch order (below 0 wraps to past the end)
     const uint32_t gx = gridDim.x, blocks = gx * gridDim.y * gridDim.z;
     const uint32_t me = blockIdx.x + gx * (blockIdx.y + gridDim.y * blockIdx.z);
-    const uint32_t b = rev ? blocks - 1 - me - (uint32_t)p.pf : me + (uint32_t)p.pf;
+    const uint32_t b = REV ? blocks - 1 - me - (uint32_t)p.pf : me + (uint32_t)p.pf;
     if (b >= blocks) return;
     int xs, yk, zk;
     if (FLAT) {  // a segment that runs into the next row is taken to continue in place

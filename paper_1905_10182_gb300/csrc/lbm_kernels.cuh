@@ -24,13 +24,12 @@ __device__ __forceinline__ void check_node(const KParams& p, const Macro& m) {
 // K1: one fused AA stream-collide step.  TRACE replaces the collision by the identity, which
 // turns the step into pure streaming with bounce-back (used to check indices bit-exactly).
 // HO: the second-order Hermite truncations (models M4, M5 of Sec. III) instead of the complete ones.
-template <typename S, bool ODD, bool LINKS, int FK, bool TRACE, bool HO, bool FLAT, bool OFF32>
+template <typename S, bool ODD, bool LINKS, int FK, bool TRACE, bool HO, bool FLAT, bool OFF32, bool REV>
 __global__ void __launch_bounds__(BLOCK_X, (sizeof(S) == 4 || ODD ? 4 : 5)) k_stream_collide(KParams p, S* __restrict__ f) {
     pdl_wait();
-    const bool rev = step_backwards<ODD, FK>(p);
-    if (p.pf) k1_prefetch<S, ODD, FLAT>(p, f, rev);
+    if (p.pf) k1_prefetch<S, ODD, FLAT, REV>(p, f);
     int x, y, z;
-    if (!node_of<FLAT>(p, x, y, z, rev)) return;
+    if (!node_of<FLAT>(p, x, y, z, REV)) return;
     const Nbr nb(x, y, z, p);
     uint32_t link = 0;
     if (LINKS) {
@@ -166,39 +165,47 @@ static cudaError_t launch_step_t(const KParams& p, S* f, int fk, bool trace, cud
         if (!trace && p.nx % 2 == 0 && (reinterpret_cast<uintptr_t>(f) & 3) == 0) {
             const dim3 grid2 = x2_grid(p);
             const PairDims pd = make_pair_dims(p);
+#define CMLBM_X2(FK)                                                                                              \
+    launch_pdl(p.rev ? k_stream_collide_x2<S, ODD, FK, HO, can_reverse<ODD, FK>> : k_stream_collide_x2<S, ODD, FK, HO, false>, \
+               grid2, X2_BLOCK, 0, st, p, pd, f)
             switch (fk) {
-            case FK_CONST: return launch_pdl(k_stream_collide_x2<S, ODD, FK_CONST, HO>, grid2, X2_BLOCK, 0, st, p, pd, f);
-            case FK_KOLMOGOROV: return launch_pdl(k_stream_collide_x2<S, ODD, FK_KOLMOGOROV, HO>, grid2, X2_BLOCK, 0, st, p, pd, f);
-            case FK_FIELD: return launch_pdl(k_stream_collide_x2<S, ODD, FK_FIELD, HO>, grid2, X2_BLOCK, 0, st, p, pd, f);
-            case FK_SHAN_CHEN: return launch_pdl(k_stream_collide_x2<S, ODD, FK_SHAN_CHEN, HO>, grid2, X2_BLOCK, 0, st, p, pd, f);
+            case FK_CONST: return CMLBM_X2(FK_CONST);
+            case FK_KOLMOGOROV: return CMLBM_X2(FK_KOLMOGOROV);
+            case FK_FIELD: return CMLBM_X2(FK_FIELD);
+            case FK_SHAN_CHEN: return CMLBM_X2(FK_SHAN_CHEN);
             default: return cudaErrorInvalidValue;
             }
+#undef CMLBM_X2
         }
     }
     if constexpr (sizeof(S) == 4 && !LINKS) {
         // FP32 storage, the same (byte offsets within a plane are 32-bit).  Measured against the one-node
-        // kernel: store in L2 64^3 10.9 -> 7.6 us, 128x128x48 25.2 -> 20.2; store beyond L2 (p.pf) 192^3
-        // 241 -> 227 us, where the one-node kernel's rows leave lanes idle (nx no multiple of 128); but
-        // 256^3 528 -> 534 and 512^3 4.20 -> 4.31 ms: there both run at the copy rate and the pair
-        // kernel's odd step pays for its 4-byte stores.  With the Shan-Chen stencil the pair wins at
-        // every size (128^3: psi pass and step 109 -> 101 us).
-        const bool rows_full = p.pf != 0 && p.nx % BLOCK_X == 0 && fk != FK_SHAN_CHEN;
+        // kernel: 64^3 10.9 -> 7.6 us, 128x128x48 25.2 -> 20.2, 128x128x80 40.4 -> 37.6, 128^3 65.3 -> 62.6,
+        // 192^3 (rows of 1.5 blocks) 241 -> 227, 256^3 523.7 -> 520.4, 512x256x256 1063.5 -> 1061.8; with the
+        // Shan-Chen stencil 128^3 (psi pass and step) 109 -> 101.  Once L2 holds next to nothing of the
+        // store and the one-node kernel's rows are full, both run at the copy rate and the pair kernel's
+        // odd step pays for its 4-byte stores (512^3 4175 -> 4198 us; crossing between 2^25 and 2^27 nodes).
+        const bool rows_full = p.N > (1LL << 26) && p.nx % BLOCK_X == 0 && fk != FK_SHAN_CHEN;
         if (!trace && !rows_full && p.nx % 2 == 0 && (reinterpret_cast<uintptr_t>(f) & 7) == 0 && p.N < (1LL << 30)) {
             const dim3 grid2 = x2_grid(p);
             const PairDims pd = make_pair_dims(p);
+#define CMLBM_X2(FK)                                                                                              \
+    launch_pdl(p.rev ? k_stream_collide_x2f<ODD, FK, HO, can_reverse<ODD, FK>> : k_stream_collide_x2f<ODD, FK, HO, false>, \
+               grid2, X2_BLOCK, 0, st, p, pd, f)
             switch (fk) {
-            case FK_CONST: return launch_pdl(k_stream_collide_x2f<ODD, FK_CONST, HO>, grid2, X2_BLOCK, 0, st, p, pd, f);
-            case FK_KOLMOGOROV: return launch_pdl(k_stream_collide_x2f<ODD, FK_KOLMOGOROV, HO>, grid2, X2_BLOCK, 0, st, p, pd, f);
-            case FK_FIELD: return launch_pdl(k_stream_collide_x2f<ODD, FK_FIELD, HO>, grid2, X2_BLOCK, 0, st, p, pd, f);
-            case FK_SHAN_CHEN: return launch_pdl(k_stream_collide_x2f<ODD, FK_SHAN_CHEN, HO>, grid2, X2_BLOCK, 0, st, p, pd, f);
+            case FK_CONST: return CMLBM_X2(FK_CONST);
+            case FK_KOLMOGOROV: return CMLBM_X2(FK_KOLMOGOROV);
+            case FK_FIELD: return CMLBM_X2(FK_FIELD);
+            case FK_SHAN_CHEN: return CMLBM_X2(FK_SHAN_CHEN);
             default: return cudaErrorInvalidValue;
             }
+#undef CMLBM_X2
         }
     }
     if (trace) {
         // free streaming is only offered for FP32 storage (bit-exact index checks)
         if constexpr (std::is_same<S, float>::value && !HO)
-            return launch_pdl(k_stream_collide<S, ODD, LINKS, FK_CONST, true, false, false, false>, node_grid(p, false), BLOCK_X, 0,
+            return launch_pdl(k_stream_collide<S, ODD, LINKS, FK_CONST, true, false, false, false, false>, node_grid(p, false), BLOCK_X, 0,
                               st, p, f);
         else
             return cudaErrorInvalidValue;
@@ -210,10 +217,12 @@ static cudaError_t launch_step_t(const KParams& p, S* f, int fk, bool trace, cud
     const bool off64 = LINKS && 27 * p.N >= (1LL << 32);
     const bool flat = p.flat != 0 || off64;
     const dim3 grid = node_grid(p, flat);
+#define CMLBM_K1R(FK, REV)                                                                                  \
+    (off64 ? k_stream_collide<S, ODD, LINKS, FK, false, HO, true, false, REV>                               \
+     : flat ? k_stream_collide<S, ODD, LINKS, FK, false, HO, true, LINKS, REV>                              \
+            : k_stream_collide<S, ODD, LINKS, FK, false, HO, false, LINKS, REV>)
 #define CMLBM_K1(FK)                                                                                        \
-    launch_pdl(off64 ? k_stream_collide<S, ODD, LINKS, FK, false, HO, true, false>                          \
-               : flat ? k_stream_collide<S, ODD, LINKS, FK, false, HO, true, LINKS>                         \
-                      : k_stream_collide<S, ODD, LINKS, FK, false, HO, false, LINKS>, grid, BLOCK_X, 0, st, p, f)
+    launch_pdl(p.rev ? CMLBM_K1R(FK, (can_reverse<ODD, FK>)) : CMLBM_K1R(FK, false), grid, BLOCK_X, 0, st, p, f)
     switch (fk) {
     case FK_CONST: return CMLBM_K1(FK_CONST);
     case FK_KOLMOGOROV: return CMLBM_K1(FK_KOLMOGOROV);
@@ -224,6 +233,7 @@ static cudaError_t launch_step_t(const KParams& p, S* f, int fk, bool trace, cud
     default: return cudaErrorInvalidValue;
     }
 #undef CMLBM_K1
+#undef CMLBM_K1R
 }
 
 template <typename S, bool ODD, bool HO>

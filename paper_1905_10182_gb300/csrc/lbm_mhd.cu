@@ -133,11 +133,11 @@ struct MhdArgs {
     float bw[3];
 };
 
-template <bool ODD, bool LINKS, bool FLAT>
+template <bool ODD, bool LINKS, bool FLAT, bool REV>
 __global__ void __launch_bounds__(BLOCK_X, 5) k_mhd_step(KParams p, MhdArgs q, float* __restrict__ f) {
     pdl_wait();
     int x, y, z;
-    if (!node_of<FLAT>(p, x, y, z, step_backwards<ODD, FK_CONST>(p))) return;
+    if (!node_of<FLAT>(p, x, y, z, REV)) return;
     const Nbr nb(x, y, z, p);
     const uint32_t link = LINKS ? p.links[nb.self()] : 0u;
     float h[21];
@@ -255,11 +255,13 @@ cudaError_t launch_mhd_step(const KParams& p, void* f, float* hm, float omega_m,
                             cudaStream_t st) {
     const MhdArgs q = args(hm, omega_m, bw);
     float* ff = static_cast<float*>(f);
-    const auto kernel =
-        p.flat ? (odd ? (p.links ? k_mhd_step<true, true, true> : k_mhd_step<true, false, true>)
-                      : (p.links ? k_mhd_step<false, true, true> : k_mhd_step<false, false, true>))
-               : (odd ? (p.links ? k_mhd_step<true, true, false> : k_mhd_step<true, false, false>)
-                      : (p.links ? k_mhd_step<false, true, false> : k_mhd_step<false, false, false>));
+    // [flat][links]: even steps, odd steps, odd steps backwards
+    static constexpr decltype(&k_mhd_step<false, false, false, false>) kernels[2][2][3] = {
+        {{k_mhd_step<false, false, false, false>, k_mhd_step<true, false, false, false>, k_mhd_step<true, false, false, true>},
+         {k_mhd_step<false, true, false, false>, k_mhd_step<true, true, false, false>, k_mhd_step<true, true, false, true>}},
+        {{k_mhd_step<false, false, true, false>, k_mhd_step<true, false, true, false>, k_mhd_step<true, false, true, true>},
+         {k_mhd_step<false, true, true, false>, k_mhd_step<true, true, true, false>, k_mhd_step<true, true, true, true>}}};
+    const auto kernel = kernels[p.flat != 0][p.links != nullptr][odd ? (p.rev ? 2 : 1) : 0];
     return launch_pdl(kernel, node_grid(p, p.flat != 0), BLOCK_X, 0, st, p, q, ff);
 }
 

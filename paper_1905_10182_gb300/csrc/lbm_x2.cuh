@@ -230,15 +230,15 @@ inline dim3 x2_grid(const KParams& p) {
 // otherwise a line may cover the start of the next row, and the prefetch only misses part of it).
 // Distance: p.pf blocks for 16-bit storage, 3/4 of it for FP32, whose blocks hold twice the bytes
 // (256^3, one step at 1/2, 3/4, 1 and 3/2 of p.pf: FP32 536, 534, 537, 552 us, FP16 296, 294, 294, 294).
-template <typename S, bool ODD>
-__device__ __forceinline__ void x2_prefetch(const KParams& p, const PairDims& pd, const S* f, bool rev) {
+template <typename S, bool ODD, bool REV>
+__device__ __forceinline__ void x2_prefetch(const KParams& p, const PairDims& pd, const S* f) {
     const uint32_t ahead = sizeof(S) == 4 ? (uint32_t)p.pf * 3 / 4 : (uint32_t)p.pf;
     constexpr uint32_t LPW = 64 * sizeof(S) / 128, LPB = LPW * (X2_BLOCK / 32);  // lines per warp and per block, of a plane
 #pragma unroll
     for (uint32_t t = threadIdx.x; t < 27 * LPB; t += X2_BLOCK) {
         const uint32_t k = t / LPB, w = t - k * LPB;
         // the block `ahead` places on in launch order (below 0 wraps to past the end)
-        const uint32_t b = rev ? gridDim.x - 1 - blockIdx.x - ahead : blockIdx.x + ahead;
+        const uint32_t b = REV ? gridDim.x - 1 - blockIdx.x - ahead : blockIdx.x + ahead;
         const uint32_t G = b * X2_BLOCK + w * (32 / LPW);
         if (b >= gridDim.x || G >= pd.pairs) return;
         const uint32_t row = pd.np.div(G);
@@ -347,13 +347,12 @@ __device__ __forceinline__ void check_pair(const KParams& p, const Macro2& m) {
     }
 }
 
-template <typename S, bool ODD, int FK, bool HO>
+template <typename S, bool ODD, int FK, bool HO, bool REV>
 __global__ void __launch_bounds__(X2_BLOCK, (ODD ? 4 : 5))
     k_stream_collide_x2(KParams p, PairDims pd, S* __restrict__ f) {
     pdl_wait();
-    const bool rev = step_backwards<ODD, FK>(p);
-    if (p.pf) x2_prefetch<S, ODD>(p, pd, f, rev);
-    const uint32_t G = (rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * X2_BLOCK + threadIdx.x;
+    if (p.pf) x2_prefetch<S, ODD, REV>(p, pd, f);
+    const uint32_t G = (REV ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * X2_BLOCK + threadIdx.x;
     if (G >= pd.pairs) return;
     const PairMap pm = map_pair(p, pd, G);
     const uint32_t nx = p.nx, ny = p.ny, nz = p.nz;
@@ -443,13 +442,12 @@ __device__ __forceinline__ void cp_async4(uint32_t s, const char* g) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(s), "l"(g) : "memory");
 }
 
-template <bool ODD, int FK, bool HO>
+template <bool ODD, int FK, bool HO, bool REV>
 __global__ void __launch_bounds__(X2_BLOCK, 5) k_stream_collide_x2f(KParams p, PairDims pd, float* __restrict__ f) {
     __shared__ float2 stage[27][X2_BLOCK];
     pdl_wait();
-    const bool rev = step_backwards<ODD, FK>(p);
-    if (p.pf) x2_prefetch<float, ODD>(p, pd, f, rev);
-    const uint32_t G = (rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * X2_BLOCK + threadIdx.x;
+    if (p.pf) x2_prefetch<float, ODD, REV>(p, pd, f);
+    const uint32_t G = (REV ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * X2_BLOCK + threadIdx.x;
     if (G >= pd.pairs) return;
     const uint32_t nx = p.nx, ny = p.ny, nz = p.nz;
     const uint64_t PB = (uint64_t)p.N * sizeof(float);
