@@ -458,6 +458,50 @@ lbm_status ensure_scratch(lbm_batch* b) {
 // parity of domain k's store: active domains share the batch parity, retired ones are natural
 int domain_parity(const lbm_batch* b, int k) { return b->active[k] ? b->parity : 0; }
 
+// Puts the equilibrium state of src (rho, u) into domain k.  Returns without waiting for the stream.
+lbm_status launch_state(lbm_batch* b, int k, const float* (&src)[4]) {
+    const long long N = b->dom[k].N;
+    for (int j = 0; j < 4; ++j) {
+        if (in_place(src[j], b->device)) continue;
+        const lbm_status st = ensure_scratch(b);
+        if (st) return st;
+        BCK(b, cudaMemcpyAsync(b->scratch + j * N, src[j], sizeof(float) * N, cudaMemcpyDefault, b->stream), "set_state copy");
+        src[j] = b->scratch + j * N;
+    }
+    BCK(b, launch_init_equilibrium<float>(domain_params(b, k), b->pool + b->dom[k].f_off, src[0], src[1], src[2], src[3], b->stream),
+        "set_state");
+    return LBM_OK;
+}
+
+// rho and u of domain k into outs (null: left out).  Returns without waiting for the stream.
+lbm_status launch_fields(lbm_batch* b, int k, float* const (&outs)[4]) {
+    const long long N = b->dom[k].N;
+    float* dst[4];
+    for (int j = 0; j < 4; ++j) {
+        dst[j] = outs[j];
+        if (outs[j] && in_place(outs[j], b->device)) continue;
+        const lbm_status st = ensure_scratch(b);
+        if (st) return st;
+        dst[j] = b->scratch + j * N;
+    }
+    BCK(b, launch_macroscopic<float>(domain_params(b, k), b->pool + b->dom[k].f_off, domain_parity(b, k), FK_CONST, dst[0], dst[1],
+                                     dst[2], dst[3], b->stream),
+        "macroscopic");
+    for (int j = 0; j < 4; ++j)
+        if (outs[j] && outs[j] != dst[j])
+            BCK(b, cudaMemcpyAsync(outs[j], dst[j], sizeof(float) * N, cudaMemcpyDefault, b->stream), "macroscopic copy");
+    return LBM_OK;
+}
+
+// Waits for the stream, also when st is an error of work issued to it: the caller's arrays are its own
+// again when the call returns, and the scratch is free for the next.
+lbm_status settle(lbm_batch* b, lbm_status st, const char* what) {
+    const cudaError_t e = cudaStreamSynchronize(b->stream);
+    if (st) return st;
+    BCK(b, e, what);
+    return LBM_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -693,43 +737,16 @@ lbm_status lbm_batch_run(lbm_batch* b, double tol, long long max_steps, int chec
 lbm_status lbm_batch_set_state(lbm_batch* b, int k, const float* rho, const float* ux, const float* uy, const float* uz) {
     if (!b || k < 0 || k >= b->ndom || !rho || !ux || !uy || !uz) return LBM_ERR_ARG;
     if (b->active[k] && b->parity) return bfail(b, LBM_ERR_STATE, "set_state needs the batch at even parity");
-    const long long N = b->dom[k].N;
     const float* src[4] = {rho, ux, uy, uz};
     std::lock_guard<std::mutex> lock(b->scratch_mutex);
-    for (int j = 0; j < 4; ++j) {
-        if (in_place(src[j], b->device)) continue;
-        const lbm_status st = ensure_scratch(b);
-        if (st) return st;
-        BCK(b, cudaMemcpyAsync(b->scratch + j * N, src[j], sizeof(float) * N, cudaMemcpyDefault, b->stream), "set_state copy");
-        src[j] = b->scratch + j * N;
-    }
-    BCK(b, launch_init_equilibrium<float>(domain_params(b, k), b->pool + b->dom[k].f_off, src[0], src[1], src[2], src[3], b->stream),
-        "set_state");
-    BCK(b, cudaStreamSynchronize(b->stream), "set_state sync");
-    return LBM_OK;
+    return settle(b, launch_state(b, k, src), "set_state sync");
 }
 
 lbm_status lbm_batch_macroscopic(lbm_batch* b, int k, float* rho, float* ux, float* uy, float* uz) {
     if (!b || k < 0 || k >= b->ndom) return LBM_ERR_ARG;
-    const long long N = b->dom[k].N;
-    float* outs[4] = {rho, ux, uy, uz};
-    float* dst[4];
+    float* const outs[4] = {rho, ux, uy, uz};
     std::lock_guard<std::mutex> lock(b->scratch_mutex);
-    for (int j = 0; j < 4; ++j) {
-        dst[j] = outs[j];
-        if (outs[j] && in_place(outs[j], b->device)) continue;
-        const lbm_status st = ensure_scratch(b);
-        if (st) return st;
-        dst[j] = b->scratch + j * N;
-    }
-    BCK(b, launch_macroscopic<float>(domain_params(b, k), b->pool + b->dom[k].f_off, domain_parity(b, k), FK_CONST, dst[0], dst[1],
-                                     dst[2], dst[3], b->stream),
-        "macroscopic");
-    for (int j = 0; j < 4; ++j)
-        if (outs[j] && outs[j] != dst[j])
-            BCK(b, cudaMemcpyAsync(outs[j], dst[j], sizeof(float) * N, cudaMemcpyDefault, b->stream), "macroscopic copy");
-    BCK(b, cudaStreamSynchronize(b->stream), "macroscopic sync");
-    return LBM_OK;
+    return settle(b, launch_fields(b, k, outs), "macroscopic sync");
 }
 
 lbm_status lbm_batch_get_populations(lbm_batch* b, int k, float* g) {

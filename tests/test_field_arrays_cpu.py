@@ -1,0 +1,79 @@
+"""Field arrays handed to the C ABI, on a host CUDA runtime (fake_runtime.py): what the calls do when a copy
+fails."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import fake_runtime
+from paper_1905_10182_gb300 import _native as nat
+
+SHAPES = [(13, 9, 7), (20, 11, 6)]
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    return fake_runtime.build(tmp_path_factory.mktemp("host"))
+
+
+@pytest.fixture
+def batch(lib):
+    lib.fake_reset()
+    arr = (nat.LbmDomain * len(SHAPES))()
+    for a, s in zip(arr, SHAPES):
+        a.nx, a.ny, a.nz, a.nu, a.walls_y = *s, 0.05, 1
+    h = ctypes.c_void_p()
+    assert lib.lbm_batch_create(arr, len(SHAPES), 1.0, None, ctypes.byref(h)) == nat.LBM_OK
+    yield h
+    lib.lbm_batch_destroy(h)
+
+
+def host(n):
+    return [np.zeros(n, dtype=np.float32) for _ in range(4)]
+
+
+def ptrs(arrays):
+    return [a.ctypes.data if isinstance(a, np.ndarray) else a for a in arrays]
+
+
+@pytest.fixture
+def domain(lib):
+    lib.fake_reset()
+    d = nat.LbmDesc()
+    d.nx, d.ny, d.nz, d.nu, d.rho0 = *SHAPES[0], 0.05, 1.0
+    h = ctypes.c_void_p()
+    assert lib.lbm_create(ctypes.byref(d), ctypes.byref(h)) == nat.LBM_OK
+    yield h
+    lib.lbm_destroy(h)
+
+
+@pytest.fixture
+def alloc(lib):
+    made = []
+
+    def f(n):
+        made.append(lib.fake_alloc(n))
+        return made[-1]
+    yield f
+    for p in made:
+        lib.cudaFree(p)
+
+
+def call(lib, kind, which, handle, arrays):
+    if kind == "batch":
+        return getattr(lib, "lbm_batch_" + which)(handle, 0, *ptrs(arrays))
+    return getattr(lib, "lbm_" + which)(handle, *ptrs(arrays))
+
+
+@pytest.mark.parametrize("which", ["set_state", "macroscopic"])
+@pytest.mark.parametrize("kind", ["batch", "domain"])
+@pytest.mark.parametrize("fails,nth", [("cudaMemcpyAsync", 1), ("cudaMemcpyAsync", 2), ("cudaMemcpyAsync", 3), ("launch", 1)])
+def test_nothing_runs_after_an_error(lib, request, kind, which, fails, nth, alloc):
+    """The arrays are the caller's again when the call returns, with an error too: no copy and no kernel may
+    still be reading or writing them.  The first array lies in device memory, the others need copies."""
+    handle = request.getfixturevalue(kind)
+    n = int(np.prod(SHAPES[0]))
+    arrays = [alloc(4 * n)] + host(n)[1:]
+    lib.fake_fail(fails.encode(), nth)
+    assert call(lib, kind, which, handle, arrays) == nat.LBM_ERR_CUDA
+    assert lib.fake_pending() == 0
