@@ -269,7 +269,8 @@ struct lbm_batch {
     double* h_res = nullptr;
     int tile_capacity = 0;
     int device = 0;
-    float* scratch = nullptr;  // 4 planes of the largest domain, made for the first array that is not in device memory
+    float* scratch = nullptr;  // 4 planes of scratch_nodes nodes, made for the first array that is not in device memory
+    uint32_t scratch_nodes = 0;
     std::mutex scratch_mutex;  // held by the call that uses it
 
     // launch shape (autotuned)
@@ -445,13 +446,23 @@ KParams domain_params(const lbm_batch* b, int k) {
     return p;
 }
 
-// Scratch for fields that are not in device memory, kept for the batch's life: allocated and freed in
-// each call it cost 0.15 ms and a device-wide synchronisation per domain (40 domains set and read: 12 ms).
-lbm_status ensure_scratch(lbm_batch* b) {
-    if (b->scratch) return LBM_OK;
-    uint32_t most = 0;
-    for (const BatchDomain& d : b->dom) most = std::max(most, d.N);
-    BCK(b, cudaMalloc(&b->scratch, sizeof(float) * 4 * most), "cudaMalloc(fields)");
+// Scratch for fields of a domain of N nodes that are not in device memory, kept for the batch's life: allocated
+// and freed in each call it cost 0.15 ms and a device-wide synchronisation per domain (40 domains set and
+// read: 12 ms).  Made for the largest domain, or for this one where there is no memory for that.
+lbm_status ensure_scratch(lbm_batch* b, uint32_t N) {
+    if (b->scratch_nodes >= N) return LBM_OK;
+    cudaFree(b->scratch);
+    b->scratch = nullptr;
+    b->scratch_nodes = 0;
+    uint32_t nodes = 0;
+    for (const BatchDomain& d : b->dom) nodes = std::max(nodes, d.N);
+    if (cudaMalloc(&b->scratch, 4 * sizeof(float) * nodes) != cudaSuccess) {
+        cudaGetLastError();
+        nodes = N;
+        b->scratch = nullptr;
+        BCK(b, cudaMalloc(&b->scratch, 4 * sizeof(float) * nodes), "cudaMalloc(fields)");
+    }
+    b->scratch_nodes = nodes;
     return LBM_OK;
 }
 
@@ -463,7 +474,7 @@ lbm_status launch_state(lbm_batch* b, int k, const float* (&src)[4]) {
     const long long N = b->dom[k].N;
     for (int j = 0; j < 4; ++j) {
         if (in_place(src[j], b->device)) continue;
-        const lbm_status st = ensure_scratch(b);
+        const lbm_status st = ensure_scratch(b, (uint32_t)N);
         if (st) return st;
         BCK(b, cudaMemcpyAsync(b->scratch + j * N, src[j], sizeof(float) * N, cudaMemcpyDefault, b->stream), "set_state copy");
         src[j] = b->scratch + j * N;
@@ -480,7 +491,7 @@ lbm_status launch_fields(lbm_batch* b, int k, float* const (&outs)[4]) {
     for (int j = 0; j < 4; ++j) {
         dst[j] = outs[j];
         if (outs[j] && in_place(outs[j], b->device)) continue;
-        const lbm_status st = ensure_scratch(b);
+        const lbm_status st = ensure_scratch(b, (uint32_t)N);
         if (st) return st;
         dst[j] = b->scratch + j * N;
     }

@@ -1,5 +1,5 @@
 """Field arrays handed to the C ABI, on a host CUDA runtime (fake_runtime.py): what the calls do when a copy
-fails."""
+fails or memory is short."""
 import ctypes
 
 import numpy as np
@@ -77,3 +77,23 @@ def test_nothing_runs_after_an_error(lib, request, kind, which, fails, nth, allo
     lib.fake_fail(fails.encode(), nth)
     assert call(lib, kind, which, handle, arrays) == nat.LBM_ERR_CUDA
     assert lib.fake_pending() == 0
+
+
+def test_batch_scratch_where_memory_is_short(lib, batch):
+    """A call on host arrays needs four planes of its own domain, not of the largest one."""
+    small, large = (int(np.prod(s)) for s in SHAPES)
+    free = 16 * small + 64
+    assert free < 16 * large
+    lib.fake_limit(lib.fake_used() + free)
+    a, b = host(small), host(large)
+    for _ in range(2):
+        assert lib.lbm_batch_set_state(batch, 0, *ptrs(a)) == nat.LBM_OK
+        assert lib.lbm_batch_macroscopic(batch, 0, *ptrs(a)) == nat.LBM_OK
+    assert lib.lbm_batch_set_state(batch, 1, *ptrs(b)) == nat.LBM_ERR_OOM
+    assert lib.lbm_batch_set_state(batch, 0, *ptrs(a)) == nat.LBM_OK
+    lib.fake_limit(1 << 40)
+    assert lib.lbm_batch_macroscopic(batch, 1, *ptrs(b)) == nat.LBM_OK
+    made = lib.fake_calls(b"cudaMalloc")
+    for k, f in ((0, a), (1, b)):  # then kept
+        assert lib.lbm_batch_set_state(batch, k, *ptrs(f)) == nat.LBM_OK
+    assert lib.fake_calls(b"cudaMalloc") == made
