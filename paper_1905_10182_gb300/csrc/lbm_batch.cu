@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "../../include/cmlbm.h"
+#include "lbm_arrays.h"
 #include "lbm_device.cuh"
 #include "lbm_launch.h"
 
@@ -473,7 +474,7 @@ int domain_parity(const lbm_batch* b, int k) { return b->active[k] ? b->parity :
 lbm_status launch_state(lbm_batch* b, int k, const float* (&src)[4]) {
     const long long N = b->dom[k].N;
     for (int j = 0; j < 4; ++j) {
-        if (in_place(src[j], b->device)) continue;
+        if (in_place(src[j], sizeof(float) * N, b->device)) continue;
         const lbm_status st = ensure_scratch(b, (uint32_t)N);
         if (st) return st;
         BCK(b, cudaMemcpyAsync(b->scratch + j * N, src[j], sizeof(float) * N, cudaMemcpyDefault, b->stream), "set_state copy");
@@ -488,9 +489,9 @@ lbm_status launch_state(lbm_batch* b, int k, const float* (&src)[4]) {
 lbm_status launch_fields(lbm_batch* b, int k, float* const (&outs)[4]) {
     const long long N = b->dom[k].N;
     float* dst[4];
+    direct_outputs(outs, sizeof(float) * N, b->device, b->pool + b->dom[k].f_off, sizeof(float) * 27 * N, dst);
     for (int j = 0; j < 4; ++j) {
-        dst[j] = outs[j];
-        if (outs[j] && in_place(outs[j], b->device)) continue;
+        if (dst[j]) continue;
         const lbm_status st = ensure_scratch(b, (uint32_t)N);
         if (st) return st;
         dst[j] = b->scratch + j * N;

@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "../../include/cmlbm.h"
+#include "lbm_arrays.h"
 #include "lbm_device.cuh"
 #include "lbm_launch.h"
 
@@ -100,6 +101,7 @@ lbm_status cuda_fail(lbm_ctx* c, cudaError_t e, const char* what) {
     } while (0)
 
 size_t elem_size(int storage) { return storage == LBM_FP32 ? 4 : 2; }
+size_t store_bytes(const lbm_ctx* c) { return (size_t)27 * (size_t)c->N * elem_size(c->storage); }
 
 bool valid_dims(const lbm_desc* d) {
     if (!d || d->nx < 1 || d->ny < 1 || d->nz < 1) return false;
@@ -146,9 +148,9 @@ KParams make_params(const lbm_ctx* c) {
     p.ho = (c->eq_order == 2 || c->force_order == 2) ? 1 : 0;
     // the stream-collide kernels prefetch the rows of the block two per SM ahead, when the
     // population store does not fit in L2 (a store that fits is read from L2 anyway)
-    const double store_bytes = 27.0 * (double)c->N * (double)elem_size(c->storage);
-    p.pf = store_bytes > (double)c->l2 ? 2 * c->sms : 0;
-    p.rev = 2.0 * store_bytes > (double)c->l2;
+    const size_t bytes = store_bytes(c);
+    p.pf = bytes > (size_t)c->l2 ? 2 * c->sms : 0;
+    p.rev = 2 * bytes > (size_t)c->l2;
     set_numbering(p);
     return p;
 }
@@ -268,9 +270,7 @@ lbm_status run_macro(lbm_ctx* c, float* const* out = nullptr) {
 // rho and u into outs (null: left out).  Returns without waiting for the stream.
 lbm_status launch_fields(lbm_ctx* c, float* const (&outs)[4]) {
     float* there[4] = {};
-    if (!c->hm && !c->cgb)
-        for (int k = 0; k < 4; ++k)
-            if (outs[k] && in_place(outs[k], c->device)) there[k] = outs[k];
+    if (!c->hm && !c->cgb) direct_outputs(outs, sizeof(float) * c->NL, c->device, c->f, store_bytes(c), there);
     const lbm_status st = run_macro(c, there);
     if (st) return st;
     for (int k = 0; k < 4; ++k)
@@ -279,11 +279,12 @@ lbm_status launch_fields(lbm_ctx* c, float* const (&outs)[4]) {
 }
 
 // Puts the equilibrium state of src (rho, u) into the store.  Device arrays are read where they lie (copied
-// first, they cost 32 B per node more: 512^3 0.65 ms).  Returns without waiting for the stream.
+// first, they cost 32 B per node more: 512^3 0.65 ms), unless they lie in the store, which the kernel
+// overwrites.  Returns without waiting for the stream.
 lbm_status launch_state(lbm_ctx* c, const float* (&src)[4]) {
     const long long NL = c->NL;
     for (int k = 0; k < 4; ++k) {
-        if (in_place(src[k], c->device)) continue;
+        if (in_place(src[k], sizeof(float) * NL, c->device) && !overlap(src[k], sizeof(float) * NL, c->f, store_bytes(c))) continue;
         const lbm_status st = ensure_macro(c);
         if (st) return st;
         CK(c, copy_in(c->macro + k * NL, src[k], sizeof(float) * NL, c->stream), "state copy");
@@ -898,7 +899,7 @@ lbm_status lbm_save(lbm_ctx* c, const char* path) {
     h.force_order = c->force_order;
     ckpt_force(c, h.F);
     h.G = c->G;
-    h.store_bytes = (uint64_t)27 * (uint64_t)c->N * elem_size(c->storage);
+    h.store_bytes = store_bytes(c);
     std::vector<char> buf(h.store_bytes);
     CK(c, cudaMemcpyAsync(buf.data(), c->f, h.store_bytes, cudaMemcpyDeviceToHost, c->stream), "checkpoint copy");
     CK(c, cudaStreamSynchronize(c->stream), "checkpoint sync");
@@ -918,7 +919,7 @@ lbm_status lbm_load(lbm_ctx* c, const char* path) {
     CkptHeader h;
     bool ok = std::fread(&h, sizeof(h), 1, fp) == 1 && std::memcmp(h.magic, "CMLBMCK1", 8) == 0 && h.version == 1;
     if (ok && (h.nx != c->nx || h.ny != c->ny || h.nz != c->nz || h.storage != c->storage || h.slab != c->slab ||
-               h.walls_y != c->walls_y || h.store_bytes != (uint64_t)27 * (uint64_t)c->N * elem_size(c->storage))) {
+               h.walls_y != c->walls_y || h.store_bytes != store_bytes(c))) {
         std::fclose(fp);
         return fail(c, LBM_ERR_STATE, "checkpoint grid, storage or boundaries differ from the context");
     }

@@ -11,18 +11,6 @@ namespace cmlbm {
 
 struct KParams;
 
-// A caller's array that the kernels may read or write where it lies: device memory of device `dev` (host,
-// managed and other devices' memory, and floats off their 4-byte alignment, go through a copy).
-inline bool in_place(const void* p, int dev) {
-    if (reinterpret_cast<uintptr_t>(p) & 3) return false;
-    cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return a.type == cudaMemoryTypeDevice && a.device == dev;
-}
-
 template <typename S, bool ODD, bool HO>
 cudaError_t launch_step_parity(const KParams& p, void* f, int fk, int trace, cudaStream_t st);
 // ho: the second-order Hermite truncation variants (instantiated in lbm_k_*_ho_*.cu)
