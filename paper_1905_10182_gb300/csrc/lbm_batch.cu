@@ -94,7 +94,7 @@ __device__ __forceinline__ void batch_scatter(float* __restrict__ f, uint32_t N,
 // latency.
 template <bool ODD, int SCHED>
 __global__ void __launch_bounds__(256, 2) k_batch_step(const BatchDomain* __restrict__ dom, const BatchTile* __restrict__ tiles,
-                                                    const int* __restrict__ ntiles_p, float* __restrict__ pool,
+                                                    const int* __restrict__ ntiles_p, float* pool,
                                                     const uint32_t* __restrict__ links, unsigned int* flag, float rho0) {
     pdl_wait();
     const int ntiles = *ntiles_p;

@@ -144,7 +144,7 @@ __device__ __forceinline__ void gather_two(const float* __restrict__ fr, const f
 // this pass ends, each with that part of the stores still in L2 (64x256x64: fields and step 150 -> 139 us;
 // forwards where the stores fit, 48x100x48 27.2 -> 26.7 us).
 template <bool ODD, bool LINKS, bool FLAT>
-__global__ void __launch_bounds__(BLOCK_X) k_cg_fields(KParams p, CgArgs q, const float* __restrict__ fr) {
+__global__ void __launch_bounds__(BLOCK_X) k_cg_fields(KParams p, CgArgs q, const float* fr) {
     pdl_wait();
     int x, y, z;
     if (!node_of<FLAT>(p, x, y, z, q.rev != 0)) return;
@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(BLOCK_X) k_cg_fields(KParams p, CgArgs q, cons
 }
 
 template <bool ODD, bool LINKS, bool FLAT>
-__global__ void __launch_bounds__(BLOCK_X, 4) k_cg_step(KParams p, CgArgs q, float* __restrict__ fr) {
+__global__ void __launch_bounds__(BLOCK_X, 4) k_cg_step(KParams p, CgArgs q, float* fr) {
     pdl_wait();
     int x, y, z;
     if (!node_of<FLAT>(p, x, y, z)) return;

@@ -25,7 +25,7 @@ __device__ __forceinline__ void check_node(const KParams& p, const Macro& m) {
 // turns the step into pure streaming with bounce-back (used to check indices bit-exactly).
 // HO: the second-order Hermite truncations (models M4, M5 of Sec. III) instead of the complete ones.
 template <typename S, bool ODD, bool LINKS, int FK, bool TRACE, bool HO, bool FLAT, bool OFF32, bool REV>
-__global__ void __launch_bounds__(BLOCK_X, (sizeof(S) == 4 || ODD ? 4 : 5)) k_stream_collide(KParams p, S* __restrict__ f) {
+__global__ void __launch_bounds__(BLOCK_X, (sizeof(S) == 4 || ODD ? 4 : 5)) k_stream_collide(KParams p, S* f) {
     pdl_wait();
     if (p.pf) k1_prefetch<S, ODD, FLAT, REV>(p, f);
     int x, y, z;
@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(BLOCK_X, (sizeof(S) == 4 || ODD ? 4 : 5)) k_st
 // pass ended and ends where the next one starts, so both hand-overs find the most recently
 // touched part of the store (up to the 129 MB of L2) still in L2.
 template <typename S, bool ODD, bool LINKS>
-__global__ void __launch_bounds__(BLOCK_X) k_psi(KParams p, const S* __restrict__ f, float* __restrict__ psi) {
+__global__ void __launch_bounds__(BLOCK_X) k_psi(KParams p, const S* f, float* __restrict__ psi) {
     pdl_wait();
     const int x = (gridDim.x - 1 - blockIdx.x) * BLOCK_X + threadIdx.x;
     const int y = gridDim.y - 1 - blockIdx.y, z = gridDim.z - 1 - blockIdx.z + p.z0;

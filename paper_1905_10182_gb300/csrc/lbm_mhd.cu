@@ -134,7 +134,7 @@ struct MhdArgs {
 };
 
 template <bool ODD, bool LINKS, bool FLAT, bool REV>
-__global__ void __launch_bounds__(BLOCK_X, 5) k_mhd_step(KParams p, MhdArgs q, float* __restrict__ f) {
+__global__ void __launch_bounds__(BLOCK_X, 5) k_mhd_step(KParams p, MhdArgs q, float* f) {
     pdl_wait();
     int x, y, z;
     if (!node_of<FLAT>(p, x, y, z, REV)) return;

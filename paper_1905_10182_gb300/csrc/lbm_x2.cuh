@@ -281,15 +281,15 @@ __device__ __forceinline__ void shan_chen_x2(const KParams& p, const uint32_t (&
 #pragma unroll
         for (int dy = -1; dy <= 1; ++dy) {
             const float* r = p.psi + zo[dz + 1] + yo[dy + 1];
-            const float2 L = __ldg(reinterpret_cast<const float2*>(r + xl));
-            const float2 c = __ldg(reinterpret_cast<const float2*>(r + x0));
+            const float2 L = *reinterpret_cast<const float2*>(r + xl);
+            const float2 c = *reinterpret_cast<const float2*>(r + x0);
             V2 m, z0, pl;  // psi(x - 1), psi(x), psi(x + 1) of the pair's two nodes
             if (ODD) {
                 m = V2{L};
                 z0 = V2{make_float2(L.y, c.x)};
                 pl = V2{c};
             } else {
-                const float2 R = __ldg(reinterpret_cast<const float2*>(r + xr));
+                const float2 R = *reinterpret_cast<const float2*>(r + xr);
                 m = V2{make_float2(L.y, c.x)};
                 z0 = V2{c};
                 pl = V2{make_float2(c.y, R.x)};
@@ -349,7 +349,7 @@ __device__ __forceinline__ void check_pair(const KParams& p, const Macro2& m) {
 
 template <typename S, bool ODD, int FK, bool HO, bool REV>
 __global__ void __launch_bounds__(X2_BLOCK, (ODD ? 4 : 5))
-    k_stream_collide_x2(KParams p, PairDims pd, S* __restrict__ f) {
+    k_stream_collide_x2(KParams p, PairDims pd, S* f) {
     pdl_wait();
     if (p.pf) x2_prefetch<S, ODD, REV>(p, pd, f);
     const uint32_t G = (REV ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * X2_BLOCK + threadIdx.x;
@@ -443,7 +443,7 @@ __device__ __forceinline__ void cp_async4(uint32_t s, const char* g) {
 }
 
 template <bool ODD, int FK, bool HO, bool REV>
-__global__ void __launch_bounds__(X2_BLOCK, 5) k_stream_collide_x2f(KParams p, PairDims pd, float* __restrict__ f) {
+__global__ void __launch_bounds__(X2_BLOCK, 5) k_stream_collide_x2f(KParams p, PairDims pd, float* f) {
     __shared__ float2 stage[27][X2_BLOCK];
     pdl_wait();
     if (p.pf) x2_prefetch<float, ODD, REV>(p, pd, f);
@@ -547,7 +547,7 @@ __device__ __forceinline__ V2 ld_pair_straddle(const char* a, const char* b) {
 // order like k_psi.  The sum over the 27 values runs in the order of k_psi, so psi is the same to
 // the bit.
 template <typename S, bool ODD>
-__global__ void __launch_bounds__(X2_BLOCK) k_psi_x2(KParams p, PairDims pd, const S* __restrict__ f,
+__global__ void __launch_bounds__(X2_BLOCK) k_psi_x2(KParams p, PairDims pd, const S* f,
                                                       float* __restrict__ psi) {
     pdl_wait();
     const uint32_t G = (gridDim.x - 1 - blockIdx.x) * X2_BLOCK + threadIdx.x;

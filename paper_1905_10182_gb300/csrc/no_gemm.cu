@@ -122,7 +122,7 @@ __device__ __forceinline__ void stage_tile(uint8_t* dst, const __nv_bfloat16* __
                 if (row < R && kk < K) {
                     const __nv_bfloat16* p = src + (long long)row * sr + kk;
                     if (kk + 8 <= K) {
-                        v[t] = __ldg(reinterpret_cast<const uint4*>(p));
+                        v[t] = *reinterpret_cast<const uint4*>(p);
                     } else {
                         __align__(16) __nv_bfloat16 tmp[8];
 #pragma unroll
@@ -153,7 +153,7 @@ __device__ __forceinline__ void stage_tile(uint8_t* dst, const __nv_bfloat16* __
             if (row + 8 <= R && kk + 8 <= K) {
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    const uint4 t = __ldg(reinterpret_cast<const uint4*>(src + row + (long long)(kk + j) * sk));
+                    const uint4 t = *reinterpret_cast<const uint4*>(src + row + (long long)(kk + j) * sk);
                     w[j][0] = t.x;
                     w[j][1] = t.y;
                     w[j][2] = t.z;

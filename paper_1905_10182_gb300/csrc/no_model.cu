@@ -31,7 +31,7 @@ typedef __nv_bfloat16 bf16;
 // ------------------------------------------------------------------------------ elementwise kernels
 // What the layers keep of their 1x1 maps for the backward pass: the weights in BF16 and the bias.  w, b:
 // the first layer's, the others `stride` parameters on; grid (blocks, layers).
-__global__ void k_keep_maps(const float* __restrict__ w, const float* __restrict__ b, long long stride, bf16* __restrict__ wb,
+__global__ void k_keep_maps(const float* w, const float* b, long long stride, bf16* __restrict__ wb,
                             float* __restrict__ bk, int W) {
     pdl_wait();
     const int l = blockIdx.y;
@@ -42,8 +42,8 @@ __global__ void k_keep_maps(const float* __restrict__ w, const float* __restrict
 }
 
 // out[b][c][s] = sum_i P[c][i] a[b][i][s] + p[c]  (FP32 and BF16 copies)
-__global__ void k_lift(const float* __restrict__ a, const float* __restrict__ P, const float* __restrict__ p, int B, int Ci,
-                       int W, long long S, float* __restrict__ h, bf16* __restrict__ hb) {
+__global__ void k_lift(const float* a, const float* P, const float* p, int B, int Ci, int W,
+                       long long S, float* __restrict__ h, bf16* __restrict__ hb) {
     pdl_wait();
     const long long total = (long long)B * W * S;
     for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
@@ -59,7 +59,7 @@ __global__ void k_lift(const float* __restrict__ a, const float* __restrict__ P,
 }
 
 // out[b][o][s] = sum_c Q[o][c] h[b][c][s] + q[o]
-__global__ void k_project(const float* __restrict__ h, const float* __restrict__ Q, const float* __restrict__ q, int B, int W,
+__global__ void k_project(const float* h, const float* Q, const float* q, int B, int W,
                           int Co, long long S, float* __restrict__ out) {
     pdl_wait();
     const long long total = (long long)B * Co * S;
@@ -75,7 +75,7 @@ __global__ void k_project(const float* __restrict__ h, const float* __restrict__
 }
 
 // dh[b][c][s] = sum_o Q[o][c] dout[b][o][s]
-__global__ void k_project_bwd_x(const float* __restrict__ dout, const float* __restrict__ Q, int B, int W, int Co, long long S,
+__global__ void k_project_bwd_x(const float* dout, const float* Q, int B, int W, int Co, long long S,
                                 float* __restrict__ dh) {
     pdl_wait();
     const long long total = (long long)B * W * S;
@@ -97,7 +97,7 @@ __device__ __forceinline__ float gelu_grad(float x) {
 }
 
 // z[b][o][s] += bias[o]; h = act(z) (BF16 copy for the next GEMMs)
-__global__ void k_bias_act(float* __restrict__ z, const float* __restrict__ bias, int W, long long S, long long total,
+__global__ void k_bias_act(float* z, const float* bias, int W, long long S, long long total,
                            int use_gelu, bf16* __restrict__ hb) {
     pdl_wait();
     for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
@@ -112,7 +112,7 @@ __global__ void k_bias_act(float* __restrict__ z, const float* __restrict__ bias
 // Zeroes the gradient vector outside the mode matrices: block 0 the parameters before the first one (the
 // lift), block l the ones from layer l - 1's 1x1 map on to the next mode matrix or the end.  wm, wc: offsets
 // of layer 0's mode matrix and 1x1 map, the other layers' `stride` on.
-__global__ void k_zero_dense(float* __restrict__ g, long long wm, long long wc, long long stride, int L, long long n) {
+__global__ void k_zero_dense(float* g, long long wm, long long wc, long long stride, int L, long long n) {
     pdl_wait();
     const int l = blockIdx.x;
     const long long lo = l == 0 ? 0 : wc + (l - 1) * stride, hi = l == L ? n : wm + l * stride;
@@ -120,7 +120,7 @@ __global__ void k_zero_dense(float* __restrict__ g, long long wm, long long wc, 
 }
 
 // dz = dh * act'(z); BF16 copy for the GEMMs
-__global__ void k_act_bwd(const float* __restrict__ dh, const float* __restrict__ z, long long total, int use_gelu,
+__global__ void k_act_bwd(const float* dh, const float* z, long long total, int use_gelu,
                           float* __restrict__ dz, bf16* __restrict__ dzb) {
     pdl_wait();
     for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
@@ -140,7 +140,7 @@ __global__ void k_act_bwd(const float* __restrict__ dh, const float* __restrict_
 // then the element-wise centring.
 constexpr int CENTER_PARTS = 16;
 
-__global__ void __launch_bounds__(256) k_center_partials(const float* __restrict__ src, long long S, int use_gelu,
+__global__ void __launch_bounds__(256) k_center_partials(const float* src, long long S, int use_gelu,
                                                          double* __restrict__ part) {
     pdl_wait();
     const int bc = blockIdx.x / CENTER_PARTS, p = blockIdx.x % CENTER_PARTS;
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(256) k_center_partials(const float* __restrict
 
 // The same partition, four values per load (S a multiple of 4, rows 16-byte aligned): part p of
 // a row covers the float4 groups [p per4, (p + 1) per4).
-__global__ void __launch_bounds__(256) k_center_partials_v(const float* __restrict__ src, long long S, int use_gelu,
+__global__ void __launch_bounds__(256) k_center_partials_v(const float* src, long long S, int use_gelu,
                                                            double* __restrict__ part) {
     pdl_wait();
     const int bc = blockIdx.x / CENTER_PARTS, p = blockIdx.x % CENTER_PARTS;
@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(256) k_center_partials_v(const float* __restri
     float acc = 0.0f;
 #pragma unroll 4
     for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-        const float4 v = __ldg(x + i);
+        const float4 v = x[i];
         if (use_gelu) {
             acc += gelu(v.x);
             acc += gelu(v.y);
@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(256) k_center_partials_v(const float* __restri
 
 // one warp per channel: mean[bc] = (sum of its parts) / S, the parts split over the lanes and the
 // lanes' sums combined by a shuffle tree (FP64)
-__global__ void k_center_means(const double* __restrict__ part, int channels, int parts, long long S, float* __restrict__ mean) {
+__global__ void k_center_means(const double* part, int channels, int parts, long long S, float* __restrict__ mean) {
     pdl_wait();
     const int bc = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (bc >= channels) return;
@@ -212,7 +212,7 @@ __global__ void k_center_means(const double* __restrict__ part, int channels, in
 
 // db[o] += sum over samples and parts of the per-row partial sums part[(b W + o) parts + p]; one
 // warp per o
-__global__ void k_rows_to_bias(const double* __restrict__ part, int B, int W, int parts, float* __restrict__ db) {
+__global__ void k_rows_to_bias(const double* part, int B, int W, int parts, float* db) {
     pdl_wait();
     const int o = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (o >= W) return;
@@ -240,39 +240,50 @@ __device__ __forceinline__ void block_sum_to(float v, double* out) {
 }
 
 // grid (chunks, channels): each block strides over its channel's S values
-__global__ void k_center_apply(const float* __restrict__ src, long long S, int use_gelu, const float* __restrict__ mean,
+__global__ void k_center_apply(const float* src, long long S, int use_gelu, const float* mean,
                                bf16* __restrict__ out) {
     pdl_wait();
     const long long base = (long long)blockIdx.y * S;
     const float m = mean[blockIdx.y];
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < S; i += (long long)gridDim.x * blockDim.x) {
         const float v = src[base + i];
-        out[base + i] = __float2bfloat16((use_gelu ? gelu(v) : v) - m);
+        out[base + i] = __float2bfloat16(__fsub_rn(use_gelu ? gelu(v) : v, m));
     }
 }
 
-// bias (optional, W entries): added to src first
-__global__ void __launch_bounds__(256) k_center_apply_v(const float* __restrict__ src, const float* __restrict__ bias, int W,
-                                                        long long S, int use_gelu, const float* __restrict__ mean,
-                                                        bf16* __restrict__ out) {
+constexpr int APPLY_PER = 4;  // float4 groups in flight per thread
+
+// bias (optional, W entries): added to src first.  Bound by HBM with the GELU's instructions close behind; the
+// loads of APPLY_PER groups are issued before the first store, which a load cannot pass (one group at a time
+// the forward call at 64^3, batch 4 took 1100 us instead of 1065).
+__global__ void __launch_bounds__(256) k_center_apply_v(const float* src, const float* bias, int W, long long S, int use_gelu,
+                                                        const float* mean, bf16* __restrict__ out) {
     pdl_wait();
     const long long base = (long long)blockIdx.y * S;
     const float m = mean[blockIdx.y], bo = bias ? bias[blockIdx.y % W] : 0.0f;
     const float4* x = reinterpret_cast<const float4*>(src + base);
     uint2* o = reinterpret_cast<uint2*>(out + base);
-#pragma unroll 4
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < S / 4; i += (long long)gridDim.x * blockDim.x) {
-        float4 v = __ldg(x + i);
-        if (bias) v = make_float4(v.x + bo, v.y + bo, v.z + bo, v.w + bo);
-        if (use_gelu) v = make_float4(gelu(v.x), gelu(v.y), gelu(v.z), gelu(v.w));
-        o[i] = pack_bf16x4(make_float4(v.x - m, v.y - m, v.z - m, v.w - m));
+    const long long n4 = S / 4, step = (long long)gridDim.x * blockDim.x;
+    for (long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x; i0 < n4; i0 += APPLY_PER * step) {
+        float4 q[APPLY_PER];
+#pragma unroll
+        for (int j = 0; j < APPLY_PER; ++j)
+            if (i0 + j * step < n4) q[j] = x[i0 + j * step];
+#pragma unroll
+        for (int j = 0; j < APPLY_PER; ++j) {
+            if (i0 + j * step >= n4) break;
+            float4 v = q[j];
+            if (bias) v = make_float4(v.x + bo, v.y + bo, v.z + bo, v.w + bo);
+            if (use_gelu) v = make_float4(gelu(v.x), gelu(v.y), gelu(v.z), gelu(v.w));
+            // the activation is rounded before the mean is taken off, whatever the compiler makes of the branch
+            o[i0 + j * step] = pack_bf16x4(make_float4(__fsub_rn(v.x, m), __fsub_rn(v.y, m), __fsub_rn(v.z, m), __fsub_rn(v.w, m)));
+        }
     }
 }
 
 // Mode (0, 0, 0), real part, of each (sample, channel) row block of a mode array laid out
 // [b][c][kx][ky][ri][kz]: += scale * mean[b * W + c].
-__global__ void k_add_dc(float* __restrict__ modes, const float* __restrict__ mean, int rows, long long stride,
-                         float scale) {
+__global__ void k_add_dc(float* modes, const float* mean, int rows, long long stride, float scale) {
     pdl_wait();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < rows) modes[(long long)k * stride] += scale * mean[k];
@@ -283,7 +294,7 @@ struct Perm6 {
     long long din[6];
     int perm[6];
 };
-__global__ void k_permute6(const bf16* __restrict__ in, bf16* __restrict__ out, Perm6 P, long long total) {
+__global__ void k_permute6(const bf16* in, bf16* __restrict__ out, Perm6 P, long long total) {
     pdl_wait();
     long long sin[6];
     sin[5] = 1;
@@ -305,7 +316,7 @@ __global__ void k_permute6(const bf16* __restrict__ in, bf16* __restrict__ out, 
 // [kx][ky][ri][z].  One block per (b c, kx) moves the D x 2 MY sub-slab of that kx through shared
 // memory (rows padded by two elements against bank conflicts), reading and writing 16-byte
 // vectors; needs D and 2 MY multiples of 8 and 16-byte aligned buffers.
-__global__ void __launch_bounds__(256) k_to_zlast(const bf16* __restrict__ in, bf16* __restrict__ out, int D, int MX,
+__global__ void __launch_bounds__(256) k_to_zlast(const bf16* in, bf16* __restrict__ out, int D, int MX,
                                                   int MY) {
     pdl_wait();
     extern __shared__ bf16 sm[];  // [z][ri * MY + ky]
@@ -316,7 +327,7 @@ __global__ void __launch_bounds__(256) k_to_zlast(const bf16* __restrict__ in, b
     const int nv = L / 8;
     for (int e = threadIdx.x; e < D * nv; e += blockDim.x) {
         const int z = e / nv, v = e % nv;
-        const uint4 q = __ldg(reinterpret_cast<const uint4*>(src + (long long)z * MX * L + v * 8));
+        const uint4 q = *reinterpret_cast<const uint4*>(src + (long long)z * MX * L + v * 8);
         const bf16* h = reinterpret_cast<const bf16*>(&q);
 #pragma unroll
         for (int k = 0; k < 8; ++k) sm[z * R + v * 8 + k] = h[k];
@@ -334,7 +345,7 @@ __global__ void __launch_bounds__(256) k_to_zlast(const bf16* __restrict__ in, b
     }
 }
 
-__global__ void __launch_bounds__(256) k_from_zlast(const bf16* __restrict__ in, bf16* __restrict__ out, int D, int MX,
+__global__ void __launch_bounds__(256) k_from_zlast(const bf16* in, bf16* __restrict__ out, int D, int MX,
                                                     int MY) {
     pdl_wait();
     extern __shared__ bf16 sm[];  // [ky 2 + ri][z]
@@ -345,7 +356,7 @@ __global__ void __launch_bounds__(256) k_from_zlast(const bf16* __restrict__ in,
     const int nz = D / 8;
     for (int e = threadIdx.x; e < L * nz; e += blockDim.x) {
         const int qd = e / nz, z0 = (e % nz) * 8;
-        const uint4 q = __ldg(reinterpret_cast<const uint4*>(src + (long long)qd * D + z0));
+        const uint4 q = *reinterpret_cast<const uint4*>(src + (long long)qd * D + z0);
         const bf16* h = reinterpret_cast<const bf16*>(&q);
 #pragma unroll
         for (int k = 0; k < 8; ++k) sm[qd * R + z0 + k] = h[k];
@@ -389,8 +400,7 @@ __device__ __forceinline__ void mode_of(const MixDims& d, long long m, int& kx, 
 }
 
 // Y[b][o] = sum_c W[o][c] X[b][c] (complex), Y in BF16 for the inverse transforms
-__global__ void __launch_bounds__(256) k_mix_fwd(const float* __restrict__ X, const float* __restrict__ Wm, MixDims d,
-                                                 bf16* __restrict__ Y) {
+__global__ void __launch_bounds__(256) k_mix_fwd(const float* X, const float* Wm, MixDims d, bf16* __restrict__ Y) {
     pdl_wait();
     const long long m = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (m >= (long long)d.MX * d.MY * d.MZ) return;
@@ -423,8 +433,7 @@ __global__ void __launch_bounds__(256) k_mix_fwd(const float* __restrict__ X, co
 }
 
 // dX[b][c] = sum_o conj(W[o][c]) dY[b][o] (BF16 out); lanes over c read W[o][c] coalesced
-__global__ void __launch_bounds__(256) k_mix_bwd_x(const float* __restrict__ dY, const float* __restrict__ Wm,
-                                                   MixDims d, bf16* __restrict__ dX) {
+__global__ void __launch_bounds__(256) k_mix_bwd_x(const float* dY, const float* Wm, MixDims d, bf16* __restrict__ dX) {
     pdl_wait();
     const long long m = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (m >= (long long)d.MX * d.MY * d.MZ) return;
@@ -457,8 +466,7 @@ __global__ void __launch_bounds__(256) k_mix_bwd_x(const float* __restrict__ dY,
 }
 
 // dW[o][c] += sum_b dY[b][o] conj(X[b][c]); lanes over c write dW coalesced
-__global__ void __launch_bounds__(256) k_mix_bwd_w(const float* __restrict__ dY, const float* __restrict__ X, MixDims d,
-                                                   float* __restrict__ dW) {
+__global__ void __launch_bounds__(256) k_mix_bwd_w(const float* dY, const float* X, MixDims d, float* dW) {
     pdl_wait();
     const long long m = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (m >= (long long)d.MX * d.MY * d.MZ) return;
@@ -491,28 +499,36 @@ __global__ void __launch_bounds__(256) k_mix_bwd_w(const float* __restrict__ dY,
 constexpr int MIX_W = 32, MIX_S = 4, MIX_MODES = 8;
 constexpr int MIX_BUF = MIX_W * 2 * MIX_S;  // floats per mode and sample chunk
 
-// sbuf[w][(ch MIX_S + j) 2 + ri] <- v[b0 + j][ch][kx][ky][ri][kz0 + w] (zeros for j >= nb)
-__device__ __forceinline__ void stage_block(const float* __restrict__ V, const MixDims& d, int b0, int nb, int kx, int ky,
-                                            int kz0, float (*sbuf)[MIX_BUF]) {
-    for (int r = threadIdx.x; r < MIX_S * MIX_W * 2; r += blockDim.x) {
-        const int j = r / (MIX_W * 2), ch = (r >> 1) % MIX_W, ri = r & 1;
-        float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
-        if (j < nb) {
-            const float4* p = reinterpret_cast<const float4*>(V + xidx(d, b0 + j, ch, kx, ky, ri, kz0));
-            lo = __ldg(p);
-            hi = __ldg(p + 1);
-        }
-        const int off = (ch * MIX_S + j) * 2 + ri;
-        sbuf[0][off] = lo.x;
-        sbuf[1][off] = lo.y;
-        sbuf[2][off] = lo.z;
-        sbuf[3][off] = lo.w;
-        sbuf[4][off] = hi.x;
-        sbuf[5][off] = hi.y;
-        sbuf[6][off] = hi.z;
-        sbuf[7][off] = hi.w;
+// A thread's run of the block's coefficients, v[b0 + j][ch][kx][ky][ri][kz0 .. + 7] of its (j, ch, ri) (zeros
+// for j >= nb), and their places sbuf[w][(ch MIX_S + j) 2 + ri].  Loaded apart from the staging so that the
+// loads can be issued ahead of the matrix copies.
+struct MixRun {
+    float4 lo, hi;
+};
+constexpr int MIX_THREADS = MIX_S * MIX_W * 2;  // a run for each
+
+__device__ __forceinline__ MixRun load_run(const float* V, const MixDims& d, int b0, int kx, int ky, int kz0) {
+    const int r = threadIdx.x, j = r / (MIX_W * 2), ch = (r >> 1) % MIX_W, ri = r & 1;
+    MixRun q;
+    q.lo = q.hi = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (b0 + j < d.B) {
+        const float4* p = reinterpret_cast<const float4*>(V + xidx(d, b0 + j, ch, kx, ky, ri, kz0));
+        q.lo = p[0];
+        q.hi = p[1];
     }
-    __syncthreads();
+    return q;
+}
+__device__ __forceinline__ void stage_run(const MixRun& q, float (*sbuf)[MIX_BUF]) {
+    const int r = threadIdx.x, j = r / (MIX_W * 2), ch = (r >> 1) % MIX_W, ri = r & 1;
+    const int off = (ch * MIX_S + j) * 2 + ri;
+    sbuf[0][off] = q.lo.x;
+    sbuf[1][off] = q.lo.y;
+    sbuf[2][off] = q.lo.z;
+    sbuf[3][off] = q.lo.w;
+    sbuf[4][off] = q.hi.x;
+    sbuf[5][off] = q.hi.y;
+    sbuf[6][off] = q.hi.z;
+    sbuf[7][off] = q.hi.w;
 }
 
 // out[b0 + j][ch][kx][ky][ri][kz0 .. + 7] <- so[(j MIX_W + ch) 2 + ri][mode], one 16-byte store per run
@@ -535,7 +551,7 @@ constexpr int MIX_PITCH = 2 * MIX_W;
 constexpr int MIX_SMAT = MIX_MODES * MIX_W * MIX_PITCH * (int)sizeof(float);  // 65,536 B of dynamic shared memory
 __device__ __forceinline__ int mix_chunk(int o, int c4) { return o * MIX_PITCH + ((c4 ^ (o & 7)) << 2); }
 
-__device__ __forceinline__ void load_mode_matrix(float* sw, const float* __restrict__ w, int lane) {
+__device__ __forceinline__ void load_mode_matrix(float* sw, const float* w, int lane) {
     const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(sw));
 #pragma unroll
     for (int i = 0; i < MIX_W / 2; ++i) {
@@ -552,8 +568,7 @@ __device__ __forceinline__ void wait_mode_matrix() {
     __syncwarp();
 }
 
-__global__ void __launch_bounds__(256) k_mix_fwd32(const float* __restrict__ X, const float* __restrict__ Wm, MixDims d,
-                                                   bf16* __restrict__ Y) {
+__global__ void __launch_bounds__(MIX_THREADS) k_mix_fwd32(const float* X, const float* Wm, MixDims d, bf16* __restrict__ Y) {
     pdl_wait();
     extern __shared__ __align__(16) float smat[];  // MIX_MODES matrices, MIX_W rows of MIX_PITCH
     __shared__ __align__(16) float sbuf[MIX_MODES][MIX_BUF];
@@ -564,11 +579,14 @@ __global__ void __launch_bounds__(256) k_mix_fwd32(const float* __restrict__ X, 
     mode_of(d, m, kx, ky, kz);
     const int kz0 = kz - warp;
     float* sw = smat + warp * MIX_W * MIX_PITCH;
+    MixRun run = load_run(X, d, 0, kx, ky, kz0);
     load_mode_matrix(sw, Wm + widx(d, kx, ky, kz, 0, 0), lane);
     const float* sv = sbuf[warp];
     for (int b0 = 0; b0 < d.B; b0 += MIX_S) {
         const int nb = min(MIX_S, d.B - b0);
-        stage_block(X, d, b0, nb, kx, ky, kz0, sbuf);
+        if (b0 > 0) run = load_run(X, d, b0, kx, ky, kz0);
+        stage_run(run, sbuf);
+        __syncthreads();
         if (b0 == 0) wait_mode_matrix();
         float yr[MIX_S], yi[MIX_S];
 #pragma unroll
@@ -597,8 +615,7 @@ __global__ void __launch_bounds__(256) k_mix_fwd32(const float* __restrict__ X, 
     }
 }
 
-__global__ void __launch_bounds__(256) k_mix_bwd_x32(const float* __restrict__ dY, const float* __restrict__ Wm,
-                                                     MixDims d, bf16* __restrict__ dX) {
+__global__ void __launch_bounds__(MIX_THREADS) k_mix_bwd_x32(const float* dY, const float* Wm, MixDims d, bf16* __restrict__ dX) {
     pdl_wait();
     extern __shared__ __align__(16) float smat[];  // MIX_MODES matrices, MIX_W rows of MIX_PITCH
     __shared__ __align__(16) float sbuf[MIX_MODES][MIX_BUF];
@@ -609,11 +626,14 @@ __global__ void __launch_bounds__(256) k_mix_bwd_x32(const float* __restrict__ d
     mode_of(d, m, kx, ky, kz);
     const int kz0 = kz - warp;
     float* sw = smat + warp * MIX_W * MIX_PITCH;
+    MixRun run = load_run(dY, d, 0, kx, ky, kz0);
     load_mode_matrix(sw, Wm + widx(d, kx, ky, kz, 0, 0), lane);
     const float* sv = sbuf[warp];
     for (int b0 = 0; b0 < d.B; b0 += MIX_S) {
         const int nb = min(MIX_S, d.B - b0);
-        stage_block(dY, d, b0, nb, kx, ky, kz0, sbuf);
+        if (b0 > 0) run = load_run(dY, d, b0, kx, ky, kz0);
+        stage_run(run, sbuf);
+        __syncthreads();
         if (b0 == 0) wait_mode_matrix();
         float xr[MIX_S], xi[MIX_S];
 #pragma unroll
@@ -641,11 +661,9 @@ __global__ void __launch_bounds__(256) k_mix_bwd_x32(const float* __restrict__ d
     }
 }
 
-// dW[o][c] (+)= sum_b dY[b][o] conj(X[b][c]), lane = c: both staged by the block, samples four at
+// dW[o][c] = sum_b dY[b][o] conj(X[b][c]), lane = c: both staged by the block, samples four at
 // a time with the 32 (o) complex sums in registers; each o a coalesced 256-byte row of the warp.
-// `add`: accumulate onto dW, else overwrite.
-__global__ void __launch_bounds__(256) k_mix_bwd_w32(const float* __restrict__ dY, const float* __restrict__ X, MixDims d,
-                                                     float* __restrict__ dW, int add) {
+__global__ void __launch_bounds__(MIX_THREADS, 2) k_mix_bwd_w32(const float* dY, const float* X, MixDims d, float* __restrict__ dW) {
     pdl_wait();
     __shared__ __align__(16) float sy[MIX_MODES][MIX_BUF];
     __shared__ __align__(16) float sx[MIX_MODES][MIX_BUF];
@@ -659,8 +677,10 @@ __global__ void __launch_bounds__(256) k_mix_bwd_w32(const float* __restrict__ d
     for (int o = 0; o < MIX_W; ++o) gr[o] = gi[o] = 0.0f;
     for (int b0 = 0; b0 < d.B; b0 += MIX_S) {
         const int nb = min(MIX_S, d.B - b0);
-        stage_block(X, d, b0, nb, kx, ky, kz0, sx);
-        stage_block(dY, d, b0, nb, kx, ky, kz0, sy);
+        const MixRun x = load_run(X, d, b0, kx, ky, kz0), y = load_run(dY, d, b0, kx, ky, kz0);
+        stage_run(x, sx);
+        stage_run(y, sy);
+        __syncthreads();
         const float4 x01 = *reinterpret_cast<const float4*>(&sx[warp][lane * 2 * MIX_S]);
         const float4 x23 = *reinterpret_cast<const float4*>(&sx[warp][lane * 2 * MIX_S + 4]);
         const float xr[MIX_S] = {x01.x, x01.z, x23.x, x23.z}, xi[MIX_S] = {x01.y, x01.w, x23.y, x23.w};
@@ -680,15 +700,7 @@ __global__ void __launch_bounds__(256) k_mix_bwd_w32(const float* __restrict__ d
     }
     float2* w2 = reinterpret_cast<float2*>(dW + widx(d, kx, ky, kz, 0, lane));
 #pragma unroll
-    for (int o = 0; o < MIX_W; ++o) {
-        float2 v = make_float2(gr[o], gi[o]);
-        if (add) {
-            const float2 p = w2[o * MIX_W];
-            v.x += p.x;
-            v.y += p.y;
-        }
-        w2[o * MIX_W] = v;
-    }
+    for (int o = 0; o < MIX_W; ++o) w2[o * MIX_W] = make_float2(gr[o], gi[o]);
 }
 
 
@@ -696,7 +708,7 @@ __global__ void __launch_bounds__(256) k_mix_bwd_w32(const float* __restrict__ d
 // part[chunk][i * Cy + j] = sum over the chunk of X[b][i][s] * Y[b][j][s] (X alone if Y is null).
 // FP32 per thread (a few hundred terms at most), FP64 across the block; the chunks are summed in a
 // fixed order afterwards (k_sum_partials), so gradients are reproducible run to run.
-__global__ void k_reduce_bs(const float* __restrict__ X, const float* __restrict__ Y, int B, int Cx, int Cy, long long S,
+__global__ void k_reduce_bs(const float* X, const float* Y, int B, int Cx, int Cy, long long S,
                             int chunks, float* __restrict__ part) {
     pdl_wait();
     const int pairs = Cx * Cy;
@@ -728,7 +740,7 @@ __global__ void k_reduce_bs(const float* __restrict__ X, const float* __restrict
 // sum of partial blocks: out[k] += sum_p part[p][k]
 // out[k] += sum_p part[p][k]: a block takes 32 consecutive k (lanes) and splits the partials among
 // its 16 warps (warp w: p = w, w + 16, ...); the warps' sums are then added in warp order.
-__global__ void __launch_bounds__(512) k_sum_partials(const float* __restrict__ part, int P, int K, float* __restrict__ out) {
+__global__ void __launch_bounds__(512) k_sum_partials(const float* part, int P, int K, float* out) {
     pdl_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int k = blockIdx.x * 32 + lane;
@@ -748,7 +760,7 @@ __global__ void __launch_bounds__(512) k_sum_partials(const float* __restrict__ 
 }
 
 // mean squared error over all elements; dout = 2 (out - t) / n; loss accumulated in FP64
-__global__ void k_mse(const float* __restrict__ out, const float* __restrict__ t, long long n, float* __restrict__ dout,
+__global__ void k_mse(const float* out, const float* t, long long n, float* __restrict__ dout,
                       double* __restrict__ loss) {
     pdl_wait();
     double acc = 0.0;
@@ -775,8 +787,7 @@ __device__ __forceinline__ void adam1(float& p, float g, float& m, float& v, flo
 }
 
 // The same update four parameters per access (n4 = n / 4 float4 groups; the tail goes to k_adam).
-__global__ void __launch_bounds__(256) k_adam_v(float4* __restrict__ p, const float4* __restrict__ g, float4* __restrict__ m,
-                                                float4* __restrict__ v, long long n4, const float* __restrict__ sc, float b1,
+__global__ void __launch_bounds__(256) k_adam_v(float4* p, const float4* g, float4* m, float4* v, long long n4, const float* sc, float b1,
                                                 float b2, float eps) {
     pdl_wait();
     const float lr = sc[0], c1 = sc[1], c2 = sc[2];
@@ -793,15 +804,14 @@ __global__ void __launch_bounds__(256) k_adam_v(float4* __restrict__ p, const fl
     }
 }
 
-__global__ void k_set_adam_scalars(float* __restrict__ sc, float lr, float c1, float c2) {
+__global__ void k_set_adam_scalars(float* sc, float lr, float c1, float c2) {
     pdl_wait();
     sc[0] = lr;
     sc[1] = c1;
     sc[2] = c2;
 }
 
-__global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v, long long n,
-                       const float* __restrict__ sc, float b1, float b2, float eps) {
+__global__ void k_adam(float* p, const float* g, float* m, float* v, long long n, const float* sc, float b1, float b2, float eps) {
     pdl_wait();
     const float lr = sc[0], c1 = sc[1], c2 = sc[2];
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -835,7 +845,7 @@ inline int row_blocks(long long S) { return (int)((S / 4 + 256 * ROW_PER - 1) / 
 // float4 groups per thread.  Without keep the readers of z add the bias again, which gives the same
 // bits and saves a 134 MB write (64^3, batch 4: 51 -> 31 us).  part (optional): the block's FP64 sum of act(z) at part[row gridDim.x + blockIdx.x],
 // the next layer's centring sums.
-__global__ void __launch_bounds__(256) k_bias_act_v(float* __restrict__ z, const float* __restrict__ bias, int W, long long S,
+__global__ void __launch_bounds__(256) k_bias_act_v(float* z, const float* bias, int W, long long S,
                                                     int use_gelu, int keep, bf16* __restrict__ hb, double* __restrict__ part) {
     pdl_wait();
     const long long row = blockIdx.y, S4 = S / 4;
@@ -864,34 +874,47 @@ __global__ void __launch_bounds__(256) k_bias_act_v(float* __restrict__ z, const
 // dz = dh act'(z + bias) (FP32 and BF16; bias: W entries), row-vectorised; grid (row_blocks(S), B W).
 // Without the GELU dz is dh itself and only the BF16 copy is written.  part: the block's
 // FP64 sum of dz at part[row gridDim.x + blockIdx.x] (centring and bias gradient).
-__global__ void __launch_bounds__(256) k_act_bwd_v(const float* __restrict__ dh, const float* __restrict__ z,
-                                                   const float* __restrict__ bias, int W, long long S, int use_gelu, float* __restrict__ dz, bf16* __restrict__ dzb,
-                                                   double* __restrict__ part) {
+__global__ void __launch_bounds__(256) k_act_bwd_v(const float* dh, const float* z, const float* bias, int W, long long S, int use_gelu,
+                                                   float* __restrict__ dz, bf16* __restrict__ dzb, double* __restrict__ part) {
     pdl_wait();
     const long long row = blockIdx.y, S4 = S / 4;
     const float bo = bias[row % W];
     float sum = 0.0f;
+    constexpr int PER = ROW_PER / 2;  // groups loaded before the first store, which a load cannot pass (training
+                                      // step at 64^3, batch 4: 3065 us one at a time, 3020 in twos, 3003 in fours)
 #pragma unroll
-    for (int j = 0; j < ROW_PER; ++j) {
-        const long long s4 = ((long long)blockIdx.x * ROW_PER + j) * blockDim.x + threadIdx.x;
-        if (s4 < S4) {
-            const long long i = row * S4 + s4;
-            float4 v = __ldg(reinterpret_cast<const float4*>(dh) + i);
-            if (use_gelu) {
-                float4 x = __ldg(reinterpret_cast<const float4*>(z) + i);
-                x = make_float4(x.x + bo, x.y + bo, x.z + bo, x.w + bo);
-                v = make_float4(v.x * gelu_grad(x.x), v.y * gelu_grad(x.y), v.z * gelu_grad(x.z), v.w * gelu_grad(x.w));
+    for (int j0 = 0; j0 < ROW_PER; j0 += PER) {
+        float4 g[PER], x[PER];
+        const long long s0 = ((long long)blockIdx.x * ROW_PER + j0) * blockDim.x + threadIdx.x;
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            const long long s4 = s0 + j * blockDim.x;
+            if (s4 < S4) {
+                g[j] = reinterpret_cast<const float4*>(dh)[row * S4 + s4];
+                if (use_gelu) x[j] = reinterpret_cast<const float4*>(z)[row * S4 + s4];
             }
-            if (use_gelu) reinterpret_cast<float4*>(dz)[i] = v;
-            reinterpret_cast<uint2*>(dzb)[i] = pack_bf16x4(v);
-            sum += v.x + v.y + v.z + v.w;
+        }
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            const long long s4 = s0 + j * blockDim.x;
+            if (s4 < S4) {
+                const long long i = row * S4 + s4;
+                float4 v = g[j];
+                if (use_gelu) {
+                    const float4 a = make_float4(x[j].x + bo, x[j].y + bo, x[j].z + bo, x[j].w + bo);
+                    v = make_float4(v.x * gelu_grad(a.x), v.y * gelu_grad(a.y), v.z * gelu_grad(a.z), v.w * gelu_grad(a.w));
+                    reinterpret_cast<float4*>(dz)[i] = v;
+                }
+                reinterpret_cast<uint2*>(dzb)[i] = pack_bf16x4(v);
+                sum += v.x + v.y + v.z + v.w;
+            }
         }
     }
     if (part) block_sum_to(sum, part + row * gridDim.x + blockIdx.x);
 }
 
 // h[b][c][s] = p[c] + sum_i P[c][i] a[b][i][s] (Ci <= VEC_CH), h also as BF16; grid (positions / 1024, B)
-__global__ void __launch_bounds__(256) k_lift_v(const float* __restrict__ a, const float* __restrict__ P, const float* __restrict__ p,
+__global__ void __launch_bounds__(256) k_lift_v(const float* a, const float* P, const float* p,
                                                 int Ci, int W, long long S, float* __restrict__ h, bf16* __restrict__ hb) {
     pdl_wait();
     const long long s4 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -900,7 +923,7 @@ __global__ void __launch_bounds__(256) k_lift_v(const float* __restrict__ a, con
     float4 x[VEC_CH];
 #pragma unroll
     for (int i = 0; i < VEC_CH; ++i)
-        if (i < Ci) x[i] = __ldg(reinterpret_cast<const float4*>(a + (b * Ci + i) * S) + s4);
+        if (i < Ci) x[i] = reinterpret_cast<const float4*>(a + (b * Ci + i) * S)[s4];
     for (int c = 0; c < W; ++c) {
         const float pc = p[c];
         float4 v = make_float4(pc, pc, pc, pc);
@@ -922,9 +945,8 @@ __global__ void __launch_bounds__(256) k_lift_v(const float* __restrict__ a, con
 // constant, 0: read from Co; grid (positions / 1024, B).  Bound by HBM (h read once, 134 MB at 64^3, batch
 // 4); the channel loop must stay free of branches for its loads to be issued together.
 template <int CO, bool BIAS>
-__global__ void __launch_bounds__(256) k_project_v(const float* __restrict__ h, const float* __restrict__ bias,
-                                                   const float* __restrict__ Q, const float* __restrict__ q, int W, int Co, long long S,
-                                                   float* __restrict__ out) {
+__global__ void __launch_bounds__(256) k_project_v(const float* h, const float* bias, const float* Q, const float* q, int W, int Co,
+                                                   long long S, float* __restrict__ out) {
     pdl_wait();
     constexpr int K = CO > 0 ? CO : VEC_CH;
     const long long s4 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -936,15 +958,15 @@ __global__ void __launch_bounds__(256) k_project_v(const float* __restrict__ h, 
         if (CO > 0 || k < Co) v[k] = make_float4(q[k], q[k], q[k], q[k]);
 #pragma unroll 8
     for (int c = 0; c < W; ++c) {
-        float4 x = __ldg(reinterpret_cast<const float4*>(h + (b * W + c) * S) + s4);
+        float4 x = reinterpret_cast<const float4*>(h + (b * W + c) * S)[s4];
         if (BIAS) {
-            const float bo = __ldg(bias + c);
+            const float bo = bias[c];
             x = make_float4(x.x + bo, x.y + bo, x.z + bo, x.w + bo);
         }
 #pragma unroll
         for (int k = 0; k < K; ++k)
             if (CO > 0 || k < Co) {
-                const float w = __ldg(Q + k * W + c);
+                const float w = Q[k * W + c];
                 v[k].x += w * x.x;
                 v[k].y += w * x.y;
                 v[k].z += w * x.z;
@@ -957,7 +979,7 @@ __global__ void __launch_bounds__(256) k_project_v(const float* __restrict__ h, 
 }
 
 // dh[b][c][s] = sum_k Q[k][c] dout[b][k][s] (Co <= VEC_CH); grid (positions / 1024, B)
-__global__ void __launch_bounds__(256) k_project_bwd_x_v(const float* __restrict__ dout, const float* __restrict__ Q, int W, int Co,
+__global__ void __launch_bounds__(256) k_project_bwd_x_v(const float* dout, const float* Q, int W, int Co,
                                                          long long S, float* __restrict__ dh) {
     pdl_wait();
     const long long s4 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -966,7 +988,7 @@ __global__ void __launch_bounds__(256) k_project_bwd_x_v(const float* __restrict
     float4 g[VEC_CH];
 #pragma unroll
     for (int k = 0; k < VEC_CH; ++k)
-        if (k < Co) g[k] = __ldg(reinterpret_cast<const float4*>(dout + (b * Co + k) * S) + s4);
+        if (k < Co) g[k] = reinterpret_cast<const float4*>(dout + (b * Co + k) * S)[s4];
     for (int c = 0; c < W; ++c) {
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
@@ -1148,7 +1170,7 @@ cudaError_t center(lbm_no* n, const float* src, const float* bias, int use_gelu,
 // part[chunk][i Cy + j] as k_reduce_bs.  grid (chunks, big channels); S a multiple of 4.
 constexpr int RED_SMALL = 8;
 
-__global__ void __launch_bounds__(256) k_reduce_pairs(const float* __restrict__ big, const float* __restrict__ small, int Cb,
+__global__ void __launch_bounds__(256) k_reduce_pairs(const float* big, const float* small, int Cb,
                                                       int Cs, int B, long long S, int chunks, int big_is_x, int Cy,
                                                       float* __restrict__ part) {
     pdl_wait();
@@ -1166,11 +1188,11 @@ __global__ void __launch_bounds__(256) k_reduce_pairs(const float* __restrict__ 
             const float4* yp = reinterpret_cast<const float4*>(small + b * Cs * S);
 #pragma unroll 2
             for (long long g = g0 + threadIdx.x; g < g1; g += blockDim.x) {
-                const float4 x = __ldg(xp + g);
+                const float4 x = xp[g];
 #pragma unroll
                 for (int k = 0; k < RED_SMALL; ++k)
                     if (k < Cs) {
-                        const float4 y = __ldg(yp + k * S4 + g);
+                        const float4 y = yp[k * S4 + g];
                         acc[k] = fmaf(x.x, y.x, acc[k]);
                         acc[k] = fmaf(x.y, y.y, acc[k]);
                         acc[k] = fmaf(x.z, y.z, acc[k]);
@@ -1180,7 +1202,7 @@ __global__ void __launch_bounds__(256) k_reduce_pairs(const float* __restrict__ 
         } else {
 #pragma unroll 4
             for (long long g = g0 + threadIdx.x; g < g1; g += blockDim.x) {
-                const float4 x = __ldg(xp + g);
+                const float4 x = xp[g];
                 acc[0] += x.x;
                 acc[0] += x.y;
                 acc[0] += x.z;
@@ -1219,8 +1241,8 @@ __global__ void __launch_bounds__(256) k_reduce_pairs(const float* __restrict__ 
 constexpr int PAIR_CHUNKS = 256;
 
 template <int CS>
-__global__ void __launch_bounds__(256) k_reduce_pairs32(const float* __restrict__ big, const float* __restrict__ bias,
-                                                        const float* __restrict__ small, int B, long long S, int big_is_x, int Cy, float* __restrict__ part) {
+__global__ void __launch_bounds__(256) k_reduce_pairs32(const float* big, const float* bias, const float* small, int B, long long S,
+                                                        int big_is_x, int Cy, float* __restrict__ part) {
     pdl_wait();
     constexpr int CB = 32, NA = CB * CS;  // accumulators per thread, index c CS + k
     const long long S4 = S / 4, n4 = (long long)B * S4;
@@ -1236,10 +1258,10 @@ __global__ void __launch_bounds__(256) k_reduce_pairs32(const float* __restrict_
         for (long long g = g0 + threadIdx.x; g < g1; g += blockDim.x) {
             float4 y[CS];
 #pragma unroll
-            for (int k = 0; k < CS; ++k) y[k] = __ldg(sp + k * S4 + g);
+            for (int k = 0; k < CS; ++k) y[k] = sp[k * S4 + g];
 #pragma unroll
             for (int c = 0; c < CB; ++c) {
-                float4 x = __ldg(bp + c * S4 + g);
+                float4 x = bp[c * S4 + g];
                 if (bias) {
                     const float bo = bias[c];
                     x = make_float4(x.x + bo, x.y + bo, x.z + bo, x.w + bo);
@@ -1419,7 +1441,7 @@ lbm_status spectral_fwd(lbm_no* n, int l, const float* src, const float* bias, i
     MixDims md{B, W, MX, MY, MZ};
     const unsigned mix_grid = (unsigned)(((long long)MX * MY * MZ + 7) / 8);
     if (mix32(n, n->params + n->oWm[l]))
-        launch_pdl(k_mix_fwd32, mix_grid, 256, MIX_SMAT, n->stream, n->Xh[l], n->params + n->oWm[l], md, n->yh);
+        launch_pdl(k_mix_fwd32, mix_grid, MIX_THREADS, MIX_SMAT, n->stream, n->Xh[l], n->params + n->oWm[l], md, n->yh);
     else
         launch_pdl(k_mix_fwd, mix_grid, 256, 0, n->stream, n->Xh[l], n->params + n->oWm[l], md, n->yh);
     NCK(n, cudaGetLastError(), "mix");
@@ -1465,9 +1487,9 @@ lbm_status spectral_bwd(lbm_no* n, int l, const float* dz, float* dh, int parts)
     const unsigned mix_grid = (unsigned)(((long long)MX * MY * MZ + 7) / 8);
     if (mix32(n, n->params + n->oWm[l]) && mix32(n, n->grads + n->oWm[l])) {
         // this is the only writer of the block of the gradient
-        launch_pdl(k_mix_bwd_w32, mix_grid, 256, 0, n->stream, n->dyh, n->Xh[l], md, n->grads + n->oWm[l], 0);
+        launch_pdl(k_mix_bwd_w32, mix_grid, MIX_THREADS, 0, n->stream, n->dyh, n->Xh[l], md, n->grads + n->oWm[l]);
         NCK(n, cudaGetLastError(), "mix dW");
-        launch_pdl(k_mix_bwd_x32, mix_grid, 256, MIX_SMAT, n->stream, n->dyh, n->params + n->oWm[l], md, n->yh);
+        launch_pdl(k_mix_bwd_x32, mix_grid, MIX_THREADS, MIX_SMAT, n->stream, n->dyh, n->params + n->oWm[l], md, n->yh);
     } else {
         launch_pdl(k_mix_bwd_w, mix_grid, 256, 0, n->stream, n->dyh, n->Xh[l], md, n->grads + n->oWm[l]);
         NCK(n, cudaGetLastError(), "mix dW");
