@@ -1136,12 +1136,9 @@ int stage_mode(const void* base, long long sr, long long sk, long long sb, int b
 template <int TN>
 cudaError_t launch_tn(const GemmArgs& g, int batch, cudaStream_t st) {
     constexpr int smem = 2 * (TM * TK * 2 + TN * TK * 2);
-    static bool attr_set = false;  // the attribute is per device function; setting it twice is harmless
-    if (!attr_set) {
-        const cudaError_t e = cudaFuncSetAttribute(k_gemm_bf16_tc<TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static std::atomic<uint64_t> opted{0};
+    const cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(&k_gemm_bf16_tc<TN>), smem, opted);
+    if (e != cudaSuccess) return e;
     const dim3 grid((g.N + TN - 1) / TN, (g.M + TM - 1) / TM, batch);
     if (grid.y > 65535 || grid.z > 65535) return cudaErrorInvalidValue;
     launch_pdl(k_gemm_bf16_tc<TN>, grid, THREADS, smem, st, g);
@@ -1257,25 +1254,24 @@ bool c_map(CUtensorMap* map, const GemmArgs& g, int batch, int* row, int* three)
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Streaming multiprocessors of the current device (at least 1).
 int sm_count() {
+    static std::atomic<int> known[64];  // by device; 0: not asked yet
     int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        n = 0;
-    return n > 0 ? n : 1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
+    if ((n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) return 1;
+    known[dev].store(n, std::memory_order_relaxed);
+    return n;
 }
 
 template <int TN, int GROUPS>
 cudaError_t launch_tma_tn(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mc, tma::Args a, cudaStream_t st) {
     using Sh = tma::Shape<GROUPS>;
-    static bool attr_set = false;
-    if (!attr_set) {
-        const cudaError_t e = cudaFuncSetAttribute(tma::k_gemm_bf16_tma<TN, GROUPS>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, tma::smem_bytes<GROUPS>());
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
-    static const int sms = sm_count();
-    const long long slots = (long long)sms * Sh::blocks_per_sm;
+    static std::atomic<uint64_t> opted{0};
+    const cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(&tma::k_gemm_bf16_tma<TN, GROUPS>), tma::smem_bytes<GROUPS>(), opted);
+    if (e != cudaSuccess) return e;
+    const long long slots = (long long)sm_count() * Sh::blocks_per_sm;
     const long long grid = a.tiles < slots ? a.tiles : slots;
     launch_pdl(tma::k_gemm_bf16_tma<TN, GROUPS>, (unsigned)grid, Sh::threads, tma::smem_bytes<GROUPS>(), st, ma, mb, mc, a);
     return cudaGetLastError();
@@ -1394,10 +1390,9 @@ cudaError_t launch_map_act(const __nv_bfloat16* h, const __nv_bfloat16* Wc, cons
     int mn, three, mn_b, three_b;
     if (!operand_map(&ma, h, (int)S, MAP_W, B, 1, S, (long long)MAP_W * S, TM, 1, MAP_W, &mn, &three) || !mn) return cudaErrorNotSupported;
     if (!operand_map(&mb, Wc, MAP_W, MAP_W, 1, MAP_W, 1, 0, MAP_W, 1, TK, &mn_b, &three_b) || mn_b) return cudaErrorNotSupported;
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(tma::k_map_act, cudaFuncAttributeMaxDynamicSharedMemorySize, tma::MAP_SMEM);
-    if (attr != cudaSuccess) return attr;
-    static const int sms = sm_count();
+    static std::atomic<uint64_t> opted{0};
+    const cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(&tma::k_map_act), tma::MAP_SMEM, opted);
+    if (e != cudaSuccess) return e;
     tma::MapArgs a;
     a.z = z;
     a.bias = bias;
@@ -1409,7 +1404,7 @@ cudaError_t launch_map_act(const __nv_bfloat16* h, const __nv_bfloat16* Wc, cons
     a.supers = B * a.chunks * 8;
     a.three = three;
     a.err = err;
-    return launch_pdl(tma::k_map_act, std::min(a.supers, sms * tma::MAP_BLOCKS), tma::MAP_THREADS, tma::MAP_SMEM, st, ma, mb, a);
+    return launch_pdl(tma::k_map_act, std::min(a.supers, sm_count() * tma::MAP_BLOCKS), tma::MAP_THREADS, tma::MAP_SMEM, st, ma, mb, a);
 }
 
 cudaError_t launch_gemm_bf16(const GemmArgs& g_in, int batch, cudaStream_t st) {

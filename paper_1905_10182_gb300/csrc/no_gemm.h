@@ -4,7 +4,23 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
+#include <cstdint>
+
 namespace cmlbm {
+
+// Raises the kernel's limit of dynamic shared memory to `bytes` on the current device, once per device
+// (`done`: a bit for each where it is raised).  A failure is not kept: the next call tries again.
+inline cudaError_t opt_in_smem(const void* kernel, int bytes, std::atomic<uint64_t>& done) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const uint64_t bit = dev < 64 ? 1ull << dev : 0;
+    if (done.load(std::memory_order_relaxed) & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
+    return e;
+}
 
 // C[b] (+)= alpha * A[b] x B[b].  Element (m, k) of A[b] is A[b * sab + m * sam + k * sak], likewise
 // B (k, n) and C (m, n).  A and B are BF16; C is FP32, or BF16 when out_bf16 is set.  beta != 0

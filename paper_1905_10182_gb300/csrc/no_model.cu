@@ -1401,12 +1401,9 @@ lbm_status upload_dft(lbm_no* n) {
 
 // the width-32 mixing kernels take MIX_SMAT bytes of dynamic shared memory (beyond the default 48 KB)
 cudaError_t mix32_attrs() {
-    static const cudaError_t e = [] {
-        cudaError_t r = cudaFuncSetAttribute(k_mix_fwd32, cudaFuncAttributeMaxDynamicSharedMemorySize, MIX_SMAT);
-        if (r == cudaSuccess) r = cudaFuncSetAttribute(k_mix_bwd_x32, cudaFuncAttributeMaxDynamicSharedMemorySize, MIX_SMAT);
-        return r;
-    }();
-    return e;
+    static std::atomic<uint64_t> fwd{0}, bwd{0};
+    const cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(&k_mix_fwd32), MIX_SMAT, fwd);
+    return e != cudaSuccess ? e : opt_in_smem(reinterpret_cast<const void*>(&k_mix_bwd_x32), MIX_SMAT, bwd);
 }
 
 // the width-32 mixing kernels apply: W = 32 and the mode matrices 16-byte aligned

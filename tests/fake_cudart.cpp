@@ -21,6 +21,7 @@ struct Block {
 struct Launch {
     std::string kernel;
     std::vector<void*> pointers;  // the pointer arguments from the third on (after KParams and the store)
+    unsigned blocks;
 };
 std::map<char*, Block> blocks;
 std::map<const void*, std::string> names;
@@ -45,10 +46,11 @@ bool inside(const void* p, size_t n) {
     const auto* b = find(p);
     return !b || (char*)p + n <= b->first + b->second.bytes;
 }
-cudaError_t launch(const void* fn, void** args) {
+cudaError_t launch(const void* fn, dim3 grid, void** args) {
     if ((last = tick("launch")) != cudaSuccess) return last;
     Launch l;
     l.kernel = names.count(fn) ? names[fn] : "?";
+    l.blocks = grid.x * grid.y * grid.z;
     // fields kernels: (KParams, store, four arrays)
     if (l.kernel.find("k_init_equilibrium") != std::string::npos || l.kernel.find("k_macroscopic") != std::string::npos)
         for (int k = 2; k < 6; ++k) l.pointers.push_back(*(void**)args[k]);
@@ -99,6 +101,12 @@ API void* fake_pointer(const char* kernel, int k) {  // of the last launch of th
     for (size_t i = launches.size(); i-- > 0;)
         if (launches[i].kernel.find(kernel) != std::string::npos) return launches[i].pointers[k];
     return nullptr;
+}
+
+API int fake_blocks(const char* kernel) {  // of the last launch of the kernel
+    for (size_t i = launches.size(); i-- > 0;)
+        if (launches[i].kernel.find(kernel) != std::string::npos) return (int)launches[i].blocks;
+    return 0;
 }
 
 // ---- the runtime
@@ -166,9 +174,9 @@ API cudaError_t cudaGetDriverEntryPointByVersion(const char* name, void** fn, un
 // as on the device: a launch beyond the kernel's default 48 KB of dynamic shared memory needs the opt-in there
 API cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* fn, void** args) {
     if (c->dynamicSmemBytes > 48 * 1024 && attributes[{fn, device}] < (int)c->dynamicSmemBytes) return last = cudaErrorInvalidValue;
-    return launch(fn, args);
+    return launch(fn, c->gridDim, args);
 }
-API cudaError_t cudaLaunchKernel(const void* fn, dim3, dim3, void** args, size_t, cudaStream_t) { return launch(fn, args); }
+API cudaError_t cudaLaunchKernel(const void* fn, dim3 g, dim3, void** args, size_t, cudaStream_t) { return launch(fn, g, args); }
 API cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void*, int, size_t, unsigned) { *n = 2; return cudaSuccess; }
 API cudaError_t cudaGetSymbolAddress(void** p, const void*) { static char room[1 << 20]; *p = room; return cudaSuccess; }
 API cudaError_t cudaEventCreate(cudaEvent_t*) { return cudaSuccess; }
@@ -197,7 +205,7 @@ API cudaError_t __cudaPopCallConfiguration(dim3* g, dim3* b, size_t* m, void* s)
     return cudaSuccess;
 }
 API cudaError_t __cudaGetKernel(cudaKernel_t* k, const void* fn) { *k = (cudaKernel_t)fn; return cudaSuccess; }
-API cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void** args, size_t, cudaStream_t) { return launch((const void*)k, args); }
+API cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 g, dim3, void** args, size_t, cudaStream_t) { return launch((const void*)k, g, args); }
 API void** __cudaRegisterFatBinary(void*) { static void* h; return &h; }
 API void __cudaRegisterFatBinaryEnd(void**) {}
 API void __cudaUnregisterFatBinary(void**) {}

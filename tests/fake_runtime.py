@@ -29,7 +29,7 @@ def build(folder):
         fn.argtypes, fn.restype = getattr(real, name).argtypes, getattr(real, name).restype
     L.fake_alloc.argtypes, L.fake_alloc.restype = [ctypes.c_size_t], P
     L.fake_pointer.argtypes, L.fake_pointer.restype = [ctypes.c_char_p, ctypes.c_int], P
-    L.fake_launches.argtypes = L.fake_calls.argtypes = [ctypes.c_char_p]
+    L.fake_launches.argtypes = L.fake_calls.argtypes = L.fake_blocks.argtypes = [ctypes.c_char_p]
     L.fake_fail.argtypes = [ctypes.c_char_p, ctypes.c_int]
     L.fake_limit.argtypes = [ctypes.c_longlong]
     L.fake_used.restype = ctypes.c_longlong
