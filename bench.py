@@ -57,10 +57,10 @@ WORKLOADS = {
                               text="Rayleigh-Taylor instability, colour-gradient two-phase model, 64x256x64 "
                                    "(W=64, walls in y), At=0.5, Re=512, sqrt(gW)=0.04"),
 }
-# two-phase step, algorithmic bytes: both colours read and written once (432 + 432 B) and the
+# two-phase step, algorithmic bytes: both colours (2 x 27 floats, 216 B) read and written once and the
 # phase fields written and read back (8 + 8 B).  The field pass reads the colours a second time
-# (432 B), a cost of this two-pass design that is not counted.
-CG_BYTES_PER_NODE = 880
+# (216 B, 664 in all), a cost of this two-pass design that is not counted.
+CG_BYTES_PER_NODE = 2 * 216 + 16
 
 
 def grid_shape(wl):
