@@ -25,7 +25,7 @@ __device__ __forceinline__ void check_node(const KParams& p, const Macro& m) {
 // turns the step into pure streaming with bounce-back (used to check indices bit-exactly).
 // HO: the second-order Hermite truncations (models M4, M5 of Sec. III) instead of the complete ones.
 template <typename S, bool ODD, bool LINKS, int FK, bool TRACE, bool HO, bool FLAT, bool OFF32, bool REV>
-__global__ void __launch_bounds__(BLOCK_X, (sizeof(S) == 4 || ODD ? 4 : 5)) k_stream_collide(KParams p, S* f) {
+__global__ void __launch_bounds__(BLOCK_X, (sizeof(S) == 4 || (ODD && (!LINKS || OFF32)) ? 4 : 5)) k_stream_collide(KParams p, S* f) {
     pdl_wait();
     if (p.pf) k1_prefetch<S, ODD, FLAT, REV>(p, f);
     int x, y, z;
@@ -210,17 +210,24 @@ static cudaError_t launch_step_t(const KParams& p, S* f, int fk, bool trace, cud
         else
             return cudaErrorInvalidValue;
     }
-    // links: 32-bit element offsets for the bounce-back choice (aa_gather) where 27 N allows them: an odd
+    // Links: 32-bit element offsets for the bounce-back choice (aa_gather) where 27 N allows them: an odd
     // step of a 93x47x81 channel 24.1 us and 1,200 instructions per warp with both 64-bit addresses, 17 us
-    // with them (the whole run 17.0 -> 13.9 us per step, 256x128x128 197 -> 177 us).  Larger domains number
-    // their nodes through and form both addresses.
+    // with them (the whole run 17.0 -> 13.9 us per step, 256x128x128 197 -> 177 us).  An even step has no
+    // choice to make; with 32-bit offsets FP32 gains a little (300^3 967 -> 952 us), 16-bit storage loses (86
+    // registers and five blocks per SM instead of 70 and seven: FP16 512^3 3652 -> 3996, 128^3 53 -> 60).
+    constexpr bool off32 = LINKS && (ODD || sizeof(S) == 4);
+    // Larger domains form both addresses.  Their nodes are numbered through (FP32 640x512x512 7894 -> 7808 us
+    // per step, 600x560x500 7983 -> 7805, FP16 600x560x500 6652 -> 6542), but for 16-bit storage where the
+    // rows are full (FP16 640x512x512 with walls 6079 -> 6023); their odd 16-bit steps run at five blocks per
+    // SM (6686 -> 6444 with a mask).  Backwards gains nothing at 64 times L2 and more.
     const bool off64 = LINKS && 27 * p.N >= (1LL << 32);
-    const bool flat = p.flat != 0 || off64;
+    const bool flat = off64 ? p.flat || sizeof(S) == 4 || p.nx % BLOCK_X != 0 : p.flat != 0;
     const dim3 grid = node_grid(p, flat);
 #define CMLBM_K1R(FK, REV)                                                                                  \
-    (off64 ? k_stream_collide<S, ODD, LINKS, FK, false, HO, true, false, REV>                               \
-     : flat ? k_stream_collide<S, ODD, LINKS, FK, false, HO, true, LINKS, REV>                              \
-            : k_stream_collide<S, ODD, LINKS, FK, false, HO, false, LINKS, REV>)
+    (off64 ? (flat ? k_stream_collide<S, ODD, LINKS, FK, false, HO, true, false, false>                     \
+                   : k_stream_collide<S, ODD, LINKS, FK, false, HO, sizeof(S) == 4, false, false>)          \
+     : flat ? k_stream_collide<S, ODD, LINKS, FK, false, HO, true, off32, REV>                              \
+            : k_stream_collide<S, ODD, LINKS, FK, false, HO, false, off32, REV>)
 #define CMLBM_K1(FK)                                                                                        \
     launch_pdl(p.rev ? CMLBM_K1R(FK, (can_reverse<ODD, FK>)) : CMLBM_K1R(FK, false), grid, BLOCK_X, 0, st, p, f)
     switch (fk) {

@@ -19,8 +19,33 @@ def code(path):
 
 
 FILES = sorted(glob.glob(os.path.join(buildlib.CSRC, "*.cu")) + glob.glob(os.path.join(buildlib.CSRC, "*.cuh")))
-KERNEL = re.compile(r"__global__\s+void\s+(?:__launch_bounds__\((?:[^()]|\((?:[^()]|\([^()]*\))*\))*\)\s*)?(k_\w+)\s*\((.*?)\)\s*\{(.*?)\n\}", re.S)
-KERNELS = {m.group(1): m.groups()[1:] for f in FILES for m in KERNEL.finditer(code(f))}
+
+
+def past(text, i):
+    """The place after the bracket that closes the one at i."""
+    depth = 0
+    for j in range(i, len(text)):
+        depth += {"(": 1, "{": 1, ")": -1, "}": -1}.get(text[j], 0)
+        if depth == 0:
+            return j + 1
+
+
+def kernels(text):
+    """name -> (parameters, body) of the kernels in the source."""
+    found = {}
+    for m in re.finditer(r"__global__\s+void\s+", text):
+        i = m.end()
+        if text.startswith("__launch_bounds__", i):
+            i = past(text, text.index("(", i))
+        name = re.match(r"\s*(\w+)\s*", text[i:])
+        args = i + name.end()
+        end = past(text, args)
+        if text[end:].lstrip().startswith("{"):
+            found[name.group(1)] = (text[args:end], text[end:past(text, text.index("{", end))])
+    return found
+
+
+KERNELS = {k: v for f in FILES for k, v in kernels(code(f)).items()}
 
 
 def launched():
