@@ -184,7 +184,9 @@ static cudaError_t launch_step_t(const KParams& p, S* f, int fk, bool trace, cud
         // 192^3 (rows of 1.5 blocks) 241 -> 227, 256^3 523.7 -> 520.4, 512x256x256 1063.5 -> 1061.8; with the
         // Shan-Chen stencil 128^3 (psi pass and step) 109 -> 101.  Once L2 holds next to nothing of the
         // store and the one-node kernel's rows are full, both run at the copy rate and the pair kernel's
-        // odd step pays for its 4-byte stores (512^3 4175 -> 4198 us; crossing between 2^25 and 2^27 nodes).
+        // odd step pays for its 4-byte stores: 512x512x256 2133 -> 2143 us, 512x512x320 2641 -> 2661, 512^3
+        // 4175 -> 4198, 768x512x512 6243 -> 6273.  Rows of blocks that are only nearly full leave the pair
+        // kernel ahead: 500^3 3961 -> 3911, 510^3 4183 -> 4150, 600^3 6806 -> 6727, 1000x512x512 8305 -> 8277.
         const bool rows_full = p.N > (1LL << 26) && p.nx % BLOCK_X == 0 && fk != FK_SHAN_CHEN;
         if (!trace && !rows_full && p.nx % 2 == 0 && (reinterpret_cast<uintptr_t>(f) & 7) == 0 && p.N < (1LL << 30)) {
             const dim3 grid2 = x2_grid(p);

@@ -1,13 +1,15 @@
-// Stream-collide with two nodes per thread for 16-bit population storage on fully periodic grids
-// (no walls, no mask) with an even nx: the same step as k_stream_collide (AA pattern, direct-form
-// collision of Sec. II, optional second-order Hermite truncations), restructured for the 16-bit
-// kernel's real limit, instruction issue rather than HBM bandwidth:
-//  * the populations of a node pair move as aligned 32-bit words (two 16-bit values): on even
-//    steps the pair (x, x + 1), x even, one load and one store per direction; on odd steps the
-//    pair (x - 1, x), whose sources and targets are aligned words for the 18 directions with
-//    c_x = +-1 (the other 9 take two loads and two 16-bit stores);
-//  * the collision runs on packed FP32 pairs (__fadd2_rn / __fmul2_rn / __ffma2_rn), one
-//    instruction for both nodes.
+// Stream-collide with two nodes per thread on fully periodic grids (no walls, no mask) with an even nx: the
+// same step as k_stream_collide (AA pattern, collision of Sec. II, optional second-order Hermite
+// truncations).  The populations of a node pair move as aligned words of two values: on even steps the pair
+// (x, x + 1), x even, one load and one store per direction; on odd steps the pair (x - 1, x), whose sources
+// and targets are aligned words for the 18 directions with c_x = +-1 (the other 9 take two loads and two
+// stores of one value).  The collision runs on packed FP32 pairs (__fadd2_rn / __fmul2_rn / __ffma2_rn), one
+// instruction for both nodes.
+//  * 16-bit storage (k_stream_collide_x2, 32-bit words, direct form): the one-node kernel's limit there is
+//    instruction issue rather than HBM bandwidth.
+//  * FP32 (k_stream_collide_x2f, 64-bit words, increment form): 8-byte accesses, which L2 and HBM serve
+//    faster than 4-byte ones.
+//  * k_psi_x2: the Shan-Chen pseudo-potential from the same words, for both.
 // Included by lbm_kernels.cuh.
 #pragma once
 

@@ -546,7 +546,7 @@ __device__ __forceinline__ void unstage_block(bf16* __restrict__ out, const MixD
 // cp.async (16 bytes per lane and copy, coalesced 512-byte reads): 16-byte chunk c4 of row o at place
 // c4 ^ (o mod 8) of the row, so that lanes reading one chunk of 8 different rows, or 32 consecutive 8-byte
 // words of one row, meet no bank conflict.  With rows padded instead, and the outputs staged apart from
-// the inputs, two blocks fit an SM (20.6 us per launch at 64^3, batch 4); now three do (19.3 us).
+// the inputs, two blocks fit an SM (20.6 us per launch at 64^3, batch 4); now three do (19.3, and 18 with load_run).
 constexpr int MIX_PITCH = 2 * MIX_W;
 constexpr int MIX_SMAT = MIX_MODES * MIX_W * MIX_PITCH * (int)sizeof(float);  // 65,536 B of dynamic shared memory
 __device__ __forceinline__ int mix_chunk(int o, int c4) { return o * MIX_PITCH + ((c4 ^ (o & 7)) << 2); }
