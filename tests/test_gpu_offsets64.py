@@ -1,6 +1,6 @@
 """Domains with links whose element offsets need 64 bits (27 N >= 2^32) against the 32-bit form.  A small box
 with walls and a mask (32-bit offsets, walked forwards) and the same box repeated along z until it is beyond
-the limit (64-bit offsets, odd steps backwards) hold the same flow; every node runs the same arithmetic, so
+the limit (64-bit offsets) hold the same flow; every node runs the same arithmetic, so
 the fields of every repetition agree to the bit."""
 import numpy as np
 import pytest
